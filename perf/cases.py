@@ -276,7 +276,7 @@ def prepare(case, seed):
     st = dict(case=case, plan=_plan(p), **t)
     if case["op"] == "grad":
         st["x"].requires_grad_(True)
-    if case["op"] in ("objective", "wavelet"):
+    if case["op"] == "objective":
         st["u"].requires_grad_(True)
     return st
 
@@ -296,10 +296,8 @@ def run(st):
         J = autograd.reconstruction_loss(st["plan"], st["u"], st["y"], case["alpha"], case["s"])
         (gu,) = torch.autograd.grad(J, st["u"])
         return [J.detach(), gu]
-    if op == "wavelet":  # x = E_s u and gu = E_s* gx
-        x = autograd.Es(st["plan"], case["s"], st["u"])
-        (gu,) = torch.autograd.grad(x, st["u"], st["gx"])
-        return [x.detach(), gu]
+    if op == "wavelet":
+        return [st["plan"].Es(st["u"], case["s"]), st["plan"].EsT(st["gx"], case["s"])]
     if op == "kappa":
         return st["plan"].grad_kappa(st["x"].detach(), st["y"])
     return st["batch"].solve(st["ys"], st["alphas"], st["ss"], case["iters"])[0]
