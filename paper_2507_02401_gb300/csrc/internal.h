@@ -114,6 +114,7 @@ struct StepArgs {
   float c_lap;         // coefficient of kappa*L (1, or 0.5 for the first/last step)
   float c_cur;         // 3D: coefficient of the current field (2, or 1)
   float c_prev;        // 3D: coefficient of the previous field (1, or 0)
+  int flip;            // TMA kernels: walk the grid backwards (same results)
   // fused sampling of `cur` (forward): y[s*nt + t_sample] for s in [0, ns)
   int ns, nt, t_sample;
   const int* sens_cell;

@@ -193,6 +193,7 @@ static pat_status wave_forward_impl(pat_plan* p, const float* x, float* y, cudaS
     // increment form: F_0 = x, F_n = wv[(n-1) % 2], D = wv[2]; step n makes F_{n+1}, samples F_n
     a.dbuf = p->d_wv[2];
     for (int n = 0; n < nt - 1; ++n) {
+      a.flip = n & 1;
       a.cur = (n == 0) ? x : p->d_wv[(n - 1) % 2];
       a.next = p->d_wv[n % 2];
       a.d_zero = (n == 0);
@@ -204,18 +205,21 @@ static pat_status wave_forward_impl(pat_plan* p, const float* x, float* y, cudaS
                                y, st));
     return PAT_OK;
   }
-  // three-level form: F_0 = x, F_n = wv[(n-1) % 3]
+  // three-level form: F_0 = x, F_n = wv[(n-1) % 2].  F_{n+1} overwrites F_{n-1} (each cell's previous value
+  // is read by the thread that writes the new one) and the sweep direction alternates: two buffers instead
+  // of three, and each step starts where the last one ended, on the part that is still in L2.
   for (int n = 0; n < nt - 1; ++n) {
-    a.cur = (n == 0) ? x : p->d_wv[(n - 1) % 3];
-    a.prev = (n == 0) ? nullptr : (n == 1 ? x : p->d_wv[(n - 2) % 3]);
-    a.next = p->d_wv[n % 3];
+    a.flip = n & 1;
+    a.cur = (n == 0) ? x : p->d_wv[(n - 1) % 2];
+    a.prev = (n == 0) ? nullptr : (n == 1 ? x : p->d_wv[(n - 2) % 2]);
+    a.next = p->d_wv[n % 2];
     a.c_cur = (n == 0) ? 1.f : 2.f;
     a.c_prev = (n == 0) ? 0.f : 1.f;
     a.c_lap = (n == 0) ? 0.5f : 1.f;
     a.t_sample = n;
     PAT_TRY_CUDA(step_launch(p, false, a, st));
   }
-  PAT_TRY_CUDA(sample_launch(p->d_wv[(nt - 2) % 3], p->ns, nt, nt - 1, p->d_sens_cell, p->d_sens_w, p->corners, y, st));
+  PAT_TRY_CUDA(sample_launch(p->d_wv[(nt - 2) % 2], p->ns, nt, nt - 1, p->d_sens_cell, p->d_sens_w, p->corners, y, st));
   return PAT_OK;
 }
 
@@ -255,6 +259,7 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
     a.dbuf_lo = p->d_wv[5];
     a.inj_r = y;  // G^{m+1} + S^T r_m, injected by (or just before) each step
     for (int m = nt - 1; m >= 1; --m) {
+      a.flip = m & 1;
       a.inj_t = m;
       a.cur = Qbuf(m + 1);
       a.cur_lo = Qlo(m + 1);
@@ -265,6 +270,7 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
       a.c_lap = 1.f;
       PAT_TRY_CUDA(step_launch(p, true, a, st));
     }
+    a.flip = 0;
     a.inj_t = 0;
     a.cur = Qbuf(1);
     a.cur_lo = Qlo(1);
@@ -277,12 +283,13 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
     if (staged) PAT_TRY_CUDA(cudaMemcpyAsync(x, Qbuf(2), sizeof(float) * p->N, cudaMemcpyDeviceToDevice, st));
     return PAT_OK;
   }
-  // three-level form: Q^m lives in wv[(nt-1-m) % 3]
-  auto Qbuf = [&](int m) { return p->d_wv[(nt - 1 - m) % 3]; };
+  // three-level form: Q^m lives in wv[(nt-1-m) % 2], over Q^{m+2} (as in the forward map)
+  auto Qbuf = [&](int m) { return p->d_wv[(nt - 1 - m) % 2]; };
   PAT_TRY_CUDA(fill_launch(Qbuf(nt - 1), p->N, 0.f, st));
   PAT_TRY_CUDA(inject(Qbuf(nt - 1), nt - 1));
   a.inj_r = y;  // S^T r_m added to Q^m by (or just after) the step that makes it
   for (int m = nt - 2; m >= 1; --m) {
+    a.flip = m & 1;
     a.cur = Qbuf(m + 1);
     a.prev = (m + 2 <= nt - 1) ? Qbuf(m + 2) : nullptr;
     a.next = Qbuf(m);
@@ -292,6 +299,7 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
     a.inj_t = m;
     PAT_TRY_CUDA(step_launch(p, true, a, st));
   }
+  a.flip = 0;
   a.cur = Qbuf(1);
   a.prev = (nt >= 3) ? Qbuf(2) : nullptr;
   a.next = x;

@@ -108,7 +108,8 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
 
   auto issue = [&](int tile, int s) {
     float* st = stage0 + s * G::STAGE;
-    const int gx0 = (tile % tiles_x) * TX, gy0 = (tile / tiles_x) * TY;
+    const int tt = a.flip ? ntiles - 1 - tile : tile;
+    const int gx0 = (tt % tiles_x) * TX, gy0 = (tt / tiles_x) * TY;
     mbar_expect_tx(&bars[s], stage_bytes);
     tma_load_2d(st, &mp, gx0 - XH, gy0 - R, &bars[s]);
     if (ADJ) tma_load_2d(st + G::PBOX, &ml, gx0 - XH, gy0 - R, &bars[s]);
@@ -134,7 +135,8 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
         ++issued;
       }
     }
-    const int gx0 = (tile % tiles_x) * TX, gy0 = (tile / tiles_x) * TY;
+    const int tt = a.flip ? ntiles - 1 - tile : tile;
+    const int gx0 = (tt % tiles_x) * TX, gy0 = (tt / tiles_x) * TY;
     const int gx = gx0 + c0;
     // own-cell fields straight into registers, in flight while the boxes land
     float4 d4[RUN], kh4[RUN], kl4[RUN];

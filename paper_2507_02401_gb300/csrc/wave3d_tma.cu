@@ -111,7 +111,10 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   const int z1 = (int)((zr + 1) * nz / nchunks);
   const int gx0 = (col % cols_x) * TX, gy0 = (col / cols_x) * TY;
   const int nloc = z1 - z0;   // planes computed
-  const int ncur = nloc + R;  // cur planes j = 0 .. ncur-1 (z = z0 + j) go through the ring
+  const int ncur = nloc + R;  // cur planes j = 0 .. ncur-1 (z = zb + j zd) go through the ring
+  // march upwards from z0, or downwards from z1 - 1 (a.flip): the stencil is symmetric in z and each pair
+  // is summed first, so both directions give the same bits
+  const int zb = a.flip ? z1 - 1 : z0, zd = a.flip ? -1 : 1;
   if (t == 0) {
     for (int s = 0; s < G::NS + G::NSP; ++s) mbar_init(&bars[s], 1);
     fence_mbar_init();
@@ -121,13 +124,13 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
     issued = j + 1;
     const int s = j % G::NS;
     mbar_expect_tx(&bars[s], G::PLANE * 4);
-    tma_load_3d(ring + s * G::PLANE, &mcur, gx0 - XH, gy0 - R, z0 + j, &bars[s]);
+    tma_load_3d(ring + s * G::PLANE, &mcur, gx0 - XH, gy0 - R, zb + j * zd, &bars[s]);
   };
   auto issue_prev = [&](int j) {
     issued_prev = j + 1;
     const int s = j % G::NSP;
     mbar_expect_tx(&pbars[s], G::PREV * 4);
-    tma_load_3d(pring + s * G::PREV, &mprev, gx0, gy0, z0 + j, &pbars[s]);
+    tma_load_3d(pring + s * G::PREV, &mprev, gx0, gy0, zb + j * zd, &pbars[s]);
   };
   if (t == 0) {
     for (int j = 0; j < min(R + PD, ncur); ++j) issue_cur(j);
@@ -136,20 +139,20 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   }
   fused_sample3(a, bid, t);  // the forward's sensor samples of cur, while the first copies are in flight
 
-  // register ring of the own cells: at the first plane q[k] = plane z0 - R + k
+  // register ring of the own cells: at the first plane q[k] = plane zb + (k - R) zd
   float4 q[2 * R + 1][2];
 #pragma unroll
-  for (int i = 0; i < R; ++i)  // planes z0-R .. z0-1 straight from global memory
+  for (int i = 0; i < R; ++i)  // the R planes before zb straight from global memory
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
-      const int z = z0 - R + i, gy = gy0 + r0 + rr, gx = gx0 + c0;
-      q[i][rr] = (z >= 0 && gy < ny && gx < nx)
+      const int z = zb + (i - R) * zd, gy = gy0 + r0 + rr, gx = gx0 + c0;
+      q[i][rr] = (z >= 0 && z < nz && gy < ny && gx < nx)
                      ? __ldg(reinterpret_cast<const float4*>(a.cur + z * plane + (long long)gy * nx + gx))
                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   bool ok = true;
 #pragma unroll
-  for (int i = 0; i < R; ++i) {  // planes z0 .. z0+R-1 from the ring
+  for (int i = 0; i < R; ++i) {  // planes zb .. zb + (R-1) zd from the ring
     ok = ok && (i >= ncur || mbar_wait(&bars[i % G::NS], (i / G::NS) & 1, timeout_ns));
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr)
@@ -183,7 +186,7 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
     const float* cen = ring + (i % G::NS) * G::PLANE;
     float2 L[2][2];  // packed pairs: cells (2p, 2p+1) of row rr
     lap_2x4_x2<R>(cen, BW, r0 + R, XH + c0, w2, L);
-    const int z = z0 + i;
+    const int z = zb + i * zd;
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
       const float4 pv = has_prev ? *reinterpret_cast<const float4*>(pring + (i % G::NSP) * G::PREV + (r0 + rr) * TX + c0)
