@@ -185,13 +185,6 @@ struct F4x2 {
   __device__ __forceinline__ void st(float* d) const { *reinterpret_cast<float4*>(d) = f4(); }
 };
 
-// Programmatic dependent launch: a level's grid may start while the previous
-// level's grid drains; griddepcontrol.wait (before any read of the previous
-// level's output) blocks until that grid has completed and its writes are
-// visible.  Without the launch attribute both instructions are no-ops.
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void griddep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Row stride of a staged 3D window: an odd number of 16-byte units.  The x
 // pass has each thread read 16 bytes every 32 bytes of a row, a warp spanning
 // four rows; with an even stride every row of the warp starts on the same
@@ -486,23 +479,6 @@ int grid3d(long long work, int cap) {
   return (int)(work < cap ? (work < 1 ? 1 : work) : cap);
 }
 
-// Launch with programmatic stream serialization (the kernel waits on the
-// previous grid itself, griddep_wait).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int smem, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <int L>
 cudaError_t launch_a2(cudaStream_t st, const float* in, int nx, int ny, float* A, float* H, float* V, float* D,
                       float wdet, const Filt& f) {
@@ -512,7 +488,7 @@ cudaError_t launch_a2(cudaStream_t st, const float* in, int nx, int ny, float* A
   if (cap <= 0) return cudaErrorInvalidConfiguration;
   const int tx = ((nx >> 1) + A2F<L>::OX - 1) / A2F<L>::OX, ty = ((ny >> 1) + A2F<L>::OY - 1) / A2F<L>::OY;
   const int ntiles = tx * ty;
-  return launch_pdl(dwt2d_analysis_fast_kernel<L>, ntiles < cap ? ntiles : cap, A2F<L>::SMEM, st, in, nx, ny, A, H, V,
+  return launch_pdl(dwt2d_analysis_fast_kernel<L>, ntiles < cap ? ntiles : cap, 256, A2F<L>::SMEM, st, in, nx, ny, A, H, V,
                     D, wdet, f, tx, ntiles);
 }
 
@@ -525,7 +501,7 @@ cudaError_t launch_s2(cudaStream_t st, const float* A, const float* H, const flo
   if (cap <= 0) return cudaErrorInvalidConfiguration;
   const int tx = ((nx >> 1) + S2F<L>::OX - 1) / S2F<L>::OX, ty = ((ny >> 1) + S2F<L>::OY - 1) / S2F<L>::OY;
   const int ntiles = tx * ty;
-  return launch_pdl(dwt2d_synthesis_fast_kernel<L>, ntiles < cap ? ntiles : cap, S2F<L>::SMEM, st, A, H, V, D, wdet,
+  return launch_pdl(dwt2d_synthesis_fast_kernel<L>, ntiles < cap ? ntiles : cap, 256, S2F<L>::SMEM, st, A, H, V, D, wdet,
                     nx, ny, out, f, tx, ntiles);
 }
 
@@ -987,9 +963,9 @@ cudaError_t launch_a3(cudaStream_t st, const float* in, int nx, int ny, int nz, 
   const int ncols = cols_x * (((ny >> 1) + A3F<L>::OY - 1) / A3F<L>::OY);
   const long long work = (long long)ncols * (nz >> 1);
   if (work <= cap_pp)  // every (column, output plane) item in one wave: no serial plane march
-    return launch_pdl(dwt3d_analysis_pp_kernel<L>, (int)work, A3P<L>::SMEM, st, in, nx, ny, nz, b, wdet, f, cols_x,
+    return launch_pdl(dwt3d_analysis_pp_kernel<L>, (int)work, 256, A3P<L>::SMEM, st, in, nx, ny, nz, b, wdet, f, cols_x,
                       ncols);
-  return launch_pdl(dwt3d_analysis_fast_kernel<L>, grid3d(work, cap), A3F<L>::SMEM, st, in, nx, ny, nz, b, wdet, f,
+  return launch_pdl(dwt3d_analysis_fast_kernel<L>, grid3d(work, cap), 256, A3F<L>::SMEM, st, in, nx, ny, nz, b, wdet, f,
                     cols_x, ncols);
 }
 
@@ -1003,7 +979,7 @@ cudaError_t launch_s3(cudaStream_t st, const CBands8& b, float wdet, int nx, int
   const int cols_x = ((nx >> 1) + S3F<L>::OX - 1) / S3F<L>::OX;
   const int ncols = cols_x * (((ny >> 1) + S3F<L>::OY - 1) / S3F<L>::OY);
   const long long work = (long long)ncols * (nz >> 1);
-  return launch_pdl(dwt3d_synthesis_fast_kernel<L>, grid3d(work, cap), 0, st, b, wdet, nx, ny, nz, out, f, cols_x,
+  return launch_pdl(dwt3d_synthesis_fast_kernel<L>, grid3d(work, cap), 256, 0, st, b, wdet, nx, ny, nz, out, f, cols_x,
                     ncols);
 }
 

@@ -121,8 +121,9 @@ struct StepArgs {
   const float* sens_w;
   int corners;
   float* y;
-  // Adjoint injection S^T r_{inj_t} (nullptr = none): 2D, into dbuf by a separate injection launch
-  // before the step; 3D, fused after the step through per-CTA lists (inj_tile_ptr / inj_tile).
+  // Adjoint injection S^T r_{inj_t} after the step (inj_r nullptr = none): 2D into dbuf (for the step that
+  // follows), 3D into next; fused in the TMA kernels through per-tile / per-CTA lists (inj_tile_ptr /
+  // inj_tile), a separate launch otherwise.
   // 2D absorbing layer (nullptr = none): per-cell factors a, b of the damped update and the layer
   // width in cells (tiles farther than that from every face skip the factors)
   const float* sp_a;
@@ -171,6 +172,7 @@ cudaError_t step3d_tma_launch(int R, const StepArgs& a, const CUtensorMap& cur, 
 
 // wave2d_tma.cu: 2D increment-form step with TMA tile pipelines (forward; constant-medium adjoint)
 bool tma2d_supported(int nx, int R);
+int tma2d_tile();  // tile edge in cells (tiles numbered row by row)
 // P boxes (80 x (64+2R)) and own-tile boxes (64 x 64) of an nx x ny float field
 cudaError_t tma2d_encode(const float* base, int nx, int ny, int R, CUtensorMap* halo, CUtensorMap* own);
 // mode 0: constant medium, 1: varying medium (forward), 2: constant medium with fused injection (adjoint),

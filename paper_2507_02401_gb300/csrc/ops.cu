@@ -101,7 +101,7 @@ static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t 
   cudaError_t e;
   if (p->dim == 2 && p->tma2d && tma_ready(p, a)) {
     // TMA tile pipelines: forward (constant or varying medium); adjoint in Z = kappa Q with Z
-    // compensated (boxes of Z and Z_lo), its injection S^T r_m added to G by a launch just before
+    // compensated (boxes of Z and Z_lo), the next step's injection added to G after each tile
     const int mode = adj ? 2 : (p->varc ? 1 : 0);
     const int sp = p->sponge_w > 0 ? (adj ? 2 : 1) : 0;
     const long long nthr = tma2d_threads(p->n[0], p->n[1], p->R, mode, sp);
@@ -118,30 +118,26 @@ static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t 
     }
     StepArgs b = a;
     if (!p->varc) b.kappa = b.kappa_lo = nullptr;
-    if (a.inj_r) {
-      e = inject_launch(a.dbuf, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, a.inj_r, p->nt,
-                        a.inj_t, 1.f, st);
-      if (e != cudaSuccess) return e;
-      b.inj_r = nullptr;
-    }
+    b.inj_tile_ptr = p->d_tinj_step_ptr;
+    b.inj_tile = p->d_tinj_step;
+    b.ent_sensor = p->d_ent_sensor;
+    b.ent_w = p->d_ent_w;
     e = step2d_tma_launch(p->R, mode, sp, b, mcur, mlo, p->d_status, p->timeout_ns, st);
   } else if (p->dim == 2) {
     const long long nthr = (long long)((p->n[0] + 63) / 64) * ((p->n[1] + 31) / 32) * 256;
     if (y && a.ns > nthr) a.y = nullptr;
-    if (a.inj_r) {
-      e = inject_launch(a.dbuf, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, a.inj_r, p->nt,
-                        a.inj_t, 1.f, st);
-      if (e != cudaSuccess) return e;
-    }
     StepArgs b = a;
     b.inj_r = nullptr;
     e = step2d_launch(p->R, adj, b, st);
+    if (e == cudaSuccess && a.inj_r)
+      e = inject_launch(a.dbuf, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, a.inj_r, p->nt,
+                        a.inj_t, 1.f, st);
   } else if (p->tma3d && tma_ready(p, a)) {
     const long long nthr = tma3d_threads(p->tma3d_split.nctas);
     if (y && a.ns > nthr) a.y = nullptr;
     if (a.inj_r) {  // the adjoint's post-step injection, fused per CTA
-      a.inj_tile_ptr = p->d_tinj3_ptr;
-      a.inj_tile = p->d_tinj3;
+      a.inj_tile_ptr = p->d_tinj_step_ptr;
+      a.inj_tile = p->d_tinj_step;
       a.ent_sensor = p->d_ent_sensor;
       a.ent_w = p->d_ent_w;
     }
@@ -255,12 +251,13 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
     PAT_TRY_CUDA(fill_launch(p->d_wv[5], p->N, 0.f, st));
     PAT_TRY_CUDA(fill_launch(Qbuf(nt), p->N, 0.f, st));
     PAT_TRY_CUDA(fill_launch(Qlo(nt), p->N, 0.f, st));
+    PAT_TRY_CUDA(inject(G, nt - 1));
     a.dbuf = G;
     a.dbuf_lo = p->d_wv[5];
-    a.inj_r = y;  // G^{m+1} + S^T r_m, injected by (or just before) each step
+    a.inj_r = y;  // each step leaves G^m + S^T r_{m-1} for the next
     for (int m = nt - 1; m >= 1; --m) {
       a.flip = m & 1;
-      a.inj_t = m;
+      a.inj_t = m - 1;
       a.cur = Qbuf(m + 1);
       a.cur_lo = Qlo(m + 1);
       a.next = Qbuf(m);
@@ -271,7 +268,7 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
       PAT_TRY_CUDA(step_launch(p, true, a, st));
     }
     a.flip = 0;
-    a.inj_t = 0;
+    a.inj_r = nullptr;
     a.cur = Qbuf(1);
     a.cur_lo = Qlo(1);
     const bool staged = p->tma2d && ((uintptr_t)x & 15) != 0;
@@ -328,7 +325,7 @@ static long long wave_kernels(const pat_plan* p, bool adj) {
   if (nt == 1) return adj ? 2 : 1;
   if (!adj) return nt;  // nt-1 steps + final sample
   const long long inj = p->n_inj > 0 ? 1 : 0;
-  if (p->dim == 2) return 4 + (nt - 1) * (1 + inj) + (1 + inj);  // 4 fills, (inject+step) x (nt-1), final
+  if (p->dim == 2) return 4 + inj + (nt - 1) * (p->tma2d ? 1 : 1 + inj) + 1;  // 4 fills, inject, steps, final
   if (p->tma3d) return (1 + inj) + (nt - 2) + 1;                   // fill+inject, steps with fused injection
   return (1 + inj) + (nt - 2) * (1 + inj) + (1 + inj);             // fill+inject, (step+inject), final
 }
@@ -625,11 +622,12 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
     PAT_TRY_CUDA(fill_launch(p->d_wv[5], N, 0.f, st));
     PAT_TRY_CUDA(fill_launch(Qbuf(nt), N, 0.f, st));
     PAT_TRY_CUDA(fill_launch(Qlo(nt), N, 0.f, st));
+    PAT_TRY_CUDA(inject(G, nt - 1));
     c.dbuf = G;
     c.dbuf_lo = p->d_wv[5];
-    c.inj_r = r;
+    c.inj_r = r;  // each step leaves G^m + S^T r_{m-1} for the next
     for (int m = nt - 1; m >= 1; --m) {
-      c.inj_t = m;
+      c.inj_t = m - 1;
       c.cur = Qbuf(m + 1);
       c.cur_lo = Qlo(m + 1);
       c.next = Qbuf(m);

@@ -484,13 +484,15 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
       p->tma3d = p->tma3d_split.nctas > 0;
     }
   }
-  if (p->tma3d) {  // injection lists per CTA of the 3D TMA grid (the adjoint injects after each step)
-    const int nx = p->n[0], ny = p->n[1], nz = p->n[2], G = p->tma3d_split.nctas;
-    std::vector<std::vector<InjCell>> bins((size_t)G);
+  if (p->tma3d || p->tma2d) {  // injection lists of the TMA step kernels (the adjoint injects after each step)
+    const int nx = p->n[0], ny = p->n[1], nz = p->n[2], T = tma2d_tile();
+    const int tx = (nx + T - 1) / T, ty = (ny + T - 1) / T;
+    std::vector<std::vector<InjCell>> bins((size_t)(p->tma3d ? p->tma3d_split.nctas : tx * ty));
     for (int i = 0; i < p->n_inj; ++i) {
       const long long c = p->h_inj_cell[i];
       const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-      bins[tma3d_cta_of(nx, ny, nz, p->tma3d_split, x, y, z)].push_back(InjCell{(int)c, p->h_inj_ptr[i], p->h_inj_ptr[i + 1]});
+      const int bin = p->tma3d ? tma3d_cta_of(nx, ny, nz, p->tma3d_split, x, y, z) : (y / T) * tx + x / T;
+      bins[bin].push_back(InjCell{(int)c, p->h_inj_ptr[i], p->h_inj_ptr[i + 1]});
     }
     std::vector<int> ptr(1, 0);
     std::vector<InjCell> cells;
@@ -498,12 +500,9 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
       cells.insert(cells.end(), b.begin(), b.end());
       ptr.push_back((int)cells.size());
     }
-    PAT_TRY(alloc_n(p, &p->d_tinj3_ptr, ptr.size(), "CTA injection lists"));
-    PAT_TRY(alloc_n(p, &p->d_tinj3, std::max<size_t>(cells.size(), 1), "CTA injection lists"));
-    PAT_TRY_CUDA(cudaMemcpyAsync(p->d_tinj3_ptr, ptr.data(), sizeof(int) * ptr.size(), cudaMemcpyHostToDevice, st));
-    if (!cells.empty())
-      PAT_TRY_CUDA(cudaMemcpyAsync(p->d_tinj3, cells.data(), sizeof(InjCell) * cells.size(), cudaMemcpyHostToDevice,
-                                   st));
+    PAT_TRY(upload(p, &p->d_tinj_step_ptr, ptr, "injection lists of the step kernels", st));
+    PAT_TRY(upload(p, &p->d_tinj_step, cells, "injection lists of the step kernels", st));
+    PAT_TRY_CUDA(cudaStreamSynchronize(st));  // the host vectors go out of scope
   }
   PAT_TRY_CUDA(cudaStreamSynchronize(st));
   return PAT_OK;

@@ -61,8 +61,8 @@ struct pat_plan {
   bool tma3d = false;  // 3D steps through the TMA plane-pipeline kernel
   pat::Tma3dSplit tma3d_split{0, 0};  // work split of a 3D TMA step launch
   bool tma2d = false;  // 2D steps through the TMA tile-pipeline kernel (where it applies)
-  int* d_tinj3_ptr = nullptr;       // 3D TMA kernel: injection lists per CTA (64 x 16 columns x z chunk)
-  pat::InjCell* d_tinj3 = nullptr;  // .local = linear cell index
+  int* d_tinj_step_ptr = nullptr;       // TMA step kernels: injection lists per tile (2D: 64 x 64 cells) or per
+  pat::InjCell* d_tinj_step = nullptr;  // CTA (3D: 64 x 16 columns x z range); .local = linear cell index
   struct TmaDesc {
     const float* base;
     CUtensorMap halo, own;  // stencil-input boxes with halo, own-tile boxes

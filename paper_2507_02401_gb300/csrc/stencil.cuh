@@ -116,9 +116,10 @@ __device__ __forceinline__ void lap_2x4_x2(const float* __restrict__ S, int pitc
   }
 #pragma unroll
   for (int rr = 0; rr < 2; ++rr) {
+    constexpr int NQ = (R + 3) / 4;  // 16-byte quads either side of the row's own
     float f[20];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
+    for (int q = 2 - NQ; q <= 2 + NQ; ++q) {
       const float4 v = *reinterpret_cast<const float4*>(S + (srow + rr) * pitch + scol - 8 + 4 * q);
       f[4 * q + 0] = v.x;
       f[4 * q + 1] = v.y;

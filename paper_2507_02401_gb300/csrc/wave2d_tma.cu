@@ -14,8 +14,8 @@
 // FP32 emulation of the 512^2, 1500-step, order-8 adjoint with noisy data
 // simulated from a phantom: 1.9e-5 for the plain pair-form recurrence
 // (constant and varying medium), 1.5e-5 with the difference form alone,
-// 7e-7 with the compensated Z.  The sensor injection S^T r_m is added to G by
-// a separate launch before the step.
+// 7e-7 with the compensated Z.  Each step also adds S^T r_{m-1}, the sensor
+// injection of the step after it, to the G it has just stored (lists per tile).
 //
 // Persistent CTAs walk 64 x 64 tiles; one thread issues the TMA load of the
 // next tile's boxes (80 x (64+2R) floats, halo included, zero outside the
@@ -114,6 +114,8 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
     tma_load_2d(st, &mp, gx0 - XH, gy0 - R, &bars[s]);
     if (ADJ) tma_load_2d(st + G::PBOX, &ml, gx0 - XH, gy0 - R, &bars[s]);
   };
+  griddep_wait();  // everything above overlaps the previous step's last CTAs
+  griddep_trigger();
   int first = blockIdx.x;
   if (t == 0 && first < ntiles) issue(first, 0);
   fused_sample2(a, blockIdx.x, t);  // while the first tile's boxes are in flight
@@ -250,6 +252,15 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
     else
       update(std::false_type{});
     __syncthreads();  // this stage is refilled by the next iteration's TMA
+    if (ADJ && a.inj_r) {  // G + S^T r for the next step, on this tile's cells (stored above, before the barrier)
+      const int e1 = a.inj_tile_ptr[tt + 1];
+      for (int e = a.inj_tile_ptr[tt] + t; e < e1; e += THREADS) {
+        const InjCell c = a.inj_tile[e];
+        float v = 0.f;
+        for (int q = c.beg; q < c.end; ++q) v = fmaf(a.ent_w[q], a.inj_r[(long long)a.ent_sensor[q] * a.nt + a.inj_t], v);
+        a.dbuf[c.local] += v;
+      }
+    }
   }
   // after a timed-out wait: give the copies in flight a bounded chance to land
   if (t == 0 && !ok)
@@ -290,6 +301,8 @@ size_t smem_for(int R, int mode) {
 }
 
 }  // namespace
+
+int tma2d_tile() { return TX; }
 
 bool tma2d_supported(int nx, int R) { return nx % 4 == 0 && (R == 1 || R == 3 || R == 5 || R == 7); }
 
@@ -344,7 +357,17 @@ cudaError_t step2d_tma_launch(int R, int mode, int sp, const StepArgs& a, const 
   CUtensorMap map = p, mapl = lo;
   StepArgs args = a;
   void* params[] = {&args, &map, &mapl, &status, &timeout_ns};
-  return cudaLaunchKernel(fn, dim3(nctas), dim3(threads_of(mode)), params, smem_for(R, mode), st);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(nctas);
+  cfg.blockDim = dim3(threads_of(mode));
+  cfg.dynamicSmemBytes = smem_for(R, mode);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];  // starts while the previous step drains (the kernel waits for it itself)
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, params);
 }
 
 }  // namespace pat

@@ -29,14 +29,16 @@ namespace pat {
 namespace {
 
 constexpr int TX = 64, TY = 16, THREADS = (TX / 4) * (TY / 2);  // 128
-constexpr int XH = 8;            // box columns left of the tile (>= R, 16-byte aligned)
-constexpr int BW = TX + 2 * XH;  // box width, 80 floats
-constexpr int PD = 2;            // prefetch distance in planes
 
 template <int R>
 struct G3 {
+  // prefetch distance in planes: one at order 6, where the shorter ring lets three CTAs share an SM
+  static constexpr int PD = R == 5 ? 1 : 2;
+  static constexpr int XH = R <= 4 ? 4 : 8;      // box columns left of the tile (>= R, 16-byte aligned)
+  static constexpr int BW = TX + 2 * XH;         // box width, 72 or 80 floats
   static constexpr int BH = TY + 2 * R;
-  static constexpr int PLANE = BW * BH;  // floats per cur slot (multiple of 32: 128-byte aligned slots)
+  static constexpr int BOX = BW * BH;            // floats a TMA load brings
+  static constexpr int PLANE = (BOX + 31) / 32 * 32;  // floats per cur slot (128-byte aligned slots)
   static constexpr int NS = R + 1 + PD;  // cur slots: centre plane .. queue plane + PD
   static constexpr int PREV = TX * TY;   // floats per prev slot
   static constexpr int NSP = PD + 1;
@@ -88,6 +90,7 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   uint64_t* bars = reinterpret_cast<uint64_t*>(pring + G::NSP * G::PREV);
   uint64_t* pbars = bars + G::NS;
 
+  constexpr int XH = G::XH, BW = G::BW, PD = G::PD;
   const int t = threadIdx.x;
   const long long bid = blockIdx.x;
 
@@ -120,10 +123,12 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
     fence_mbar_init();
   }
   __syncthreads();
+  griddep_wait();  // everything above overlaps the previous step's last CTAs
+  griddep_trigger();
   auto issue_cur = [&](int j) {
     issued = j + 1;
     const int s = j % G::NS;
-    mbar_expect_tx(&bars[s], G::PLANE * 4);
+    mbar_expect_tx(&bars[s], G::BOX * 4);
     tma_load_3d(ring + s * G::PLANE, &mcur, gx0 - XH, gy0 - R, zb + j * zd, &bars[s]);
   };
   auto issue_prev = [&](int j) {
@@ -138,6 +143,28 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
       for (int j = 0; j < min(PD, nloc); ++j) issue_prev(j);
   }
   fused_sample3(a, bid, t);  // the forward's sensor samples of cur, while the first copies are in flight
+
+  // The CTA's injected cells (thread t takes entry t): the chain list bounds -> cell -> sensor -> r_m is
+  // walked one load per plane of the march, so that no load is waited for; what is left after the march is
+  // one addition per thread (and the entries beyond the first THREADS, or beyond a cell's first sensor).
+  int ie0 = 0, ie1 = 0, is = 0;
+  InjCell ic{0, 0, 0};
+  float iw = 0.f, ir = 0.f;
+  auto inj_prefetch = [&](int i) {
+    if (i == 0) {
+      ie0 = a.inj_tile_ptr[bid] + t;
+      ie1 = a.inj_tile_ptr[bid + 1];
+    } else if (i == 1) {
+      if (ie0 < ie1) ic = a.inj_tile[ie0];
+    } else if (i == 2) {
+      if (ic.beg < ic.end) {
+        is = a.ent_sensor[ic.beg];
+        iw = a.ent_w[ic.beg];
+      }
+    } else if (i == 3) {
+      if (ic.beg < ic.end) ir = a.inj_r[(long long)is * a.nt + a.inj_t];
+    }
+  };
 
   // register ring of the own cells: at the first plane q[k] = plane zb + (k - R) zd
   float4 q[2 * R + 1][2];
@@ -166,11 +193,6 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   constexpr int Q = 2 * R + 1;
   auto step = [&](auto sc, int i) -> bool {
     constexpr int S = decltype(sc)::value;
-    if (t == 0) {
-      fence_proxy_async_shared();  // the slots refilled below were last read through the generic proxy
-      if (i + R + PD < ncur) issue_cur(i + R + PD);
-      if (has_prev && i + PD < nloc) issue_prev(i + PD);
-    }
     const int jq = i + R;  // queue plane
     bool good = ok && mbar_wait(&bars[jq % G::NS], (jq / G::NS) & 1, timeout_ns);
     if (has_prev) good = good && mbar_wait(&pbars[i % G::NSP], (i / G::NSP) & 1, timeout_ns);
@@ -178,11 +200,19 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
       if (t == 0) atomicCAS(status, (int)PAT_OK, (int)PAT_ERR_TIMEOUT);
       return false;
     }
+    // the slots refilled here were read while plane i - 1 was computed, which every thread has left at the
+    // barrier above: one barrier per plane
+    if (t == 0) {
+      fence_proxy_async_shared();  // their reads went through the generic proxy
+      if (i + R + PD < ncur) issue_cur(i + R + PD);
+      if (has_prev && i + PD < nloc) issue_prev(i + PD);
+    }
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr)
       q[(2 * R + S) % Q][rr] =
           *reinterpret_cast<const float4*>(ring + (jq % G::NS) * G::PLANE + (r0 + rr + R) * BW + XH + c0);
 
+    if (INJ) inj_prefetch(i);
     const float* cen = ring + (i % G::NS) * G::PLANE;
     float2 L[2][2];  // packed pairs: cells (2p, 2p+1) of row rr
     lap_2x4_x2<R>(cen, BW, r0 + R, XH + c0, w2, L);
@@ -212,7 +242,6 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
         *reinterpret_cast<float4*>(a.next + z * plane + (long long)gy * nx + gx) =
             make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
     }
-    __syncthreads();  // the centre slot is refilled by the next step's TMA
     return true;
   };
   if constexpr (RING) {
@@ -236,8 +265,14 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   }
   if (INJ && ok_all) {  // every thread's stores to `next` precede the injection (same CTA)
     __syncthreads();
-    for (int e = a.inj_tile_ptr[bid] + t; e < a.inj_tile_ptr[bid + 1]; e += THREADS)
-      a.next[a.inj_tile[e].local] += inj_sum(a, a.inj_tile[e]);
+    for (int i = nloc; i < 4; ++i) inj_prefetch(i);  // short marches
+    if (ie0 < ie1) {
+      float v = ic.beg < ic.end ? iw * ir : 0.f;
+      for (int q = ic.beg + 1; q < ic.end; ++q)
+        v = fmaf(a.ent_w[q], a.inj_r[(long long)a.ent_sensor[q] * a.nt + a.inj_t], v);
+      a.next[ic.local] += v;
+    }
+    for (int e = ie0 + THREADS; e < ie1; e += THREADS) a.next[a.inj_tile[e].local] += inj_sum(a, a.inj_tile[e]);
   }
   // after a timed-out wait: give the copies still in flight (the last one of
   // each slot) a bounded chance to land before the CTA's shared memory goes away
@@ -264,9 +299,8 @@ cudaError_t launch_r(const StepArgs& a, const CUtensorMap& mc, const CUtensorMap
                      int* status, long long timeout_ns, cudaStream_t st) {
   const cudaError_t attr_err = prepare_r<R, INJ, RING>();
   if (attr_err != cudaSuccess) return attr_err;
-  step3d_tma_kernel<R, INJ, RING><<<nctas, THREADS, G3<R>::SMEM, st>>>(a, mc, mp, (a.nx + TX - 1) / TX, nchunks,
-                                                                        status, timeout_ns);
-  return cudaGetLastError();
+  return launch_pdl(step3d_tma_kernel<R, INJ, RING>, nctas, THREADS, (int)G3<R>::SMEM, st, a, mc, mp,
+                    (a.nx + TX - 1) / TX, nchunks, status, timeout_ns);
 }
 
 template <int R, bool INJ, bool RING>
@@ -337,7 +371,7 @@ cudaError_t tma3d_encode(const float* base, int nx, int ny, int nz, int R, CUten
   const cuuint64_t dims[3] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz};
   const cuuint64_t strides[2] = {(cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4};
   const cuuint32_t estr[3] = {1, 1, 1};
-  const cuuint32_t box_c[3] = {(cuuint32_t)BW, (cuuint32_t)(TY + 2 * R), 1};
+  const cuuint32_t box_c[3] = {(cuuint32_t)(TX + (R <= 4 ? 8 : 16)), (cuuint32_t)(TY + 2 * R), 1};
   const cuuint32_t box_p[3] = {(cuuint32_t)TX, (cuuint32_t)TY, 1};
   CUresult r1 = fn(cur, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box_c, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -380,7 +414,7 @@ Tma3dSplit tma3d_split(int R, int nx, int ny, int nz) {
   // the register-ring march saves the queue's register moves where issue is the bound (one-wave grids:
   // 38.7 / 40.3 us against 39.4 / 41.2 per K / K* step at 256^3), but its larger body costs where DRAM is
   // (many columns: 274.5 / 278.7 us against 264.8 / 268.9 at 512^3)
-  return Tma3dSplit{(int)(cols * chunks), chunks, cols * 4 < cap};
+  return Tma3dSplit{(int)(cols * chunks), chunks, cols * 4 < cap && R <= 3};
 }
 
 // CTA holding cell (x, y, z) (the kernel's split: chunk zr holds z in [zr nz / k, (zr + 1) nz / k)).
