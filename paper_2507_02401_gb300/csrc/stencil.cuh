@@ -20,6 +20,8 @@ __device__ __forceinline__ float f4get(const float4& v, int j) {
   return j == 0 ? v.x : (j == 1 ? v.y : (j == 2 ? v.z : v.w));
 }
 
+__device__ __forceinline__ float f2get(const float2& v, int j) { return j == 0 ? v.x : v.y; }
+
 // Pair term of one stencil offset: (a + b) - 2c, or in the difference form
 // (a - c) + (b - c), whose differences are exact (Sterbenz) wherever the
 // field is smooth, so the rounding error follows the local variation rather

@@ -112,4 +112,86 @@ __device__ __forceinline__ void stencil_run(const float* __restrict__ box, int r
   }
 }
 
+// ------------------------------------------------ two columns per thread
+// A thread owns columns c, c + 1 (c even) of RUN consecutive rows: one packed FP32x2 pair per row.  Half the
+// window registers of the four-column form, so two 256-thread CTAs of the adjoint fit an SM.
+//
+// The row's pair shifted by m columns.  R is odd, so the floats c - R - 1 .. c + R + 2 are R + 2 aligned
+// pairs; h[k] holds the pair at offset 2 (k - (R + 1) / 2), h[(R + 1) / 2] the own pair.
+template <int R>
+struct RowPairs {
+  static constexpr int H = (R + 1) / 2;
+  float2 h[R + 2];
+  __device__ __forceinline__ void load(const float* __restrict__ own, float2 c) {
+#pragma unroll
+    for (int k = 0; k < R + 2; ++k)
+      h[k] = k == H ? c : *reinterpret_cast<const float2*>(own + 2 * (k - H));
+  }
+  __device__ __forceinline__ float at(int o) const {  // offset o = -R-1 .. R+2 from column c
+    const int k = (o + R + 1) / 2;
+    return ((o + R + 1) & 1) ? h[k].y : h[k].x;
+  }
+  __device__ __forceinline__ float2 pair(int m) const { return make_float2(at(m), at(m + 1)); }
+};
+
+// a + b and a - c of two pairs.  An odd shift straddles two aligned register pairs: packed arithmetic would
+// first move both halves, so those take two scalar additions (the same rounding).
+__device__ __forceinline__ float2 add_pair(float2 a, float2 b, bool aligned) {
+  return aligned ? __fadd2_rn(a, b) : make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
+
+// stencil_cells2 for one pair: y taps from the window, x taps from the row, in that order; each lane equals
+// stencil_cell's result.
+template <int R, bool DIFF>
+__device__ __forceinline__ float2 stencil_pair(const float2 (&win)[2 * R + 1], const RowPairs<R>& f,
+                                               const float2 (&w2)[R + 1]) {
+  const float2 c = win[R];
+  const float2 nc = __fmul2_rn(c, dup2(-1.f));
+  float2 acc = dup2(0.f);
+#pragma unroll
+  for (int m = 1; m <= R; ++m) acc = __ffma2_rn(w2[m], pair_term2<DIFF>(win[R + m], win[R - m], c, nc), acc);
+#pragma unroll
+  for (int m = 1; m <= R; ++m) {
+    const bool even = m % 2 == 0;
+    float2 t;
+    if (DIFF)
+      t = __fadd2_rn(add_pair(f.pair(m), nc, even), add_pair(f.pair(-m), nc, even));
+    else
+      t = __ffma2_rn(c, dup2(-2.f), add_pair(f.pair(m), f.pair(-m), even));
+    acc = __ffma2_rn(w2[m], t, acc);
+  }
+  return acc;
+}
+
+// stencil_run for the pair form: lo[rr] of the thread's RUN rows (box pitch BW, `own` the thread's first cell
+// in the box).
+template <int R, int RUN, int BW>
+__device__ __forceinline__ void stencil_run_pair(const float* __restrict__ own, const float2 (&w2)[R + 1], float2 nwc,
+                                                 float2 (&lo)[RUN]) {
+  float2 win[2 * R + 1];
+#pragma unroll
+  for (int i = 0; i < 2 * R; ++i) win[i] = *reinterpret_cast<const float2*>(own + (i - R) * BW);
+#pragma unroll
+  for (int rr = 0; rr < RUN; ++rr) {
+    win[2 * R] = *reinterpret_cast<const float2*>(own + (rr + R) * BW);
+    RowPairs<R> f;
+    f.load(own + rr * BW, win[R]);
+    float2 acc = __fmul2_rn(nwc, win[R]);
+#pragma unroll
+    for (int m = 1; m <= R; ++m) acc = __ffma2_rn(w2[m], __fadd2_rn(win[R + m], win[R - m]), acc);
+#pragma unroll
+    for (int m = 1; m <= R; ++m) acc = __ffma2_rn(w2[m], add_pair(f.pair(m), f.pair(-m), m % 2 == 0), acc);
+    lo[rr] = acc;
+#pragma unroll
+    for (int i = 0; i < 2 * R; ++i) win[i] = win[i + 1];
+  }
+}
+
+// 8-byte load of data read once per launch (streamed: no L1 allocation)
+__device__ __forceinline__ float2 ld_stream2(const float* p) {
+  float2 v;
+  asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+
 }  // namespace pat

@@ -46,11 +46,8 @@
 namespace pat {
 namespace {
 
-constexpr int TX = 64, TY = 64, TCOLS = TX / 4;
-// rows per thread: 8 for the forward (128 threads per tile); 4 for the adjoint (256 threads), whose
-// two stencils and two staged boxes need more registers and shared memory per cell
-__host__ __device__ constexpr int run_rows(int mode) { return mode == 2 ? 4 : 8; }
-__host__ __device__ constexpr int threads_of(int mode) { return TCOLS * (TY / run_rows(mode)); }
+constexpr int TX = 64, TY = 64, TCOLS = TX / 2, RUN = 8;
+constexpr int THREADS = TCOLS * (TY / RUN);  // 256: each thread owns 2 columns x 8 rows
 constexpr int XH = 8;            // box columns left of the tile (>= R, 16-byte aligned)
 constexpr int BW = TX + 2 * XH;  // box width, 80 floats
 
@@ -79,11 +76,10 @@ __device__ __forceinline__ void fused_sample2(const StepArgs& a, long long bid, 
 //   adjoint  G' = G + inc,  Q' = a Q + b G', i.e. Z' = a Z + b kappa G'  (final step: x = G' + ((a-1)/b) Q)
 // Tiles that do not reach the layer use a = b = 1 without loading the factors.
 template <int R, int MODE, int SP>
-__global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
+__global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
                                                              const __grid_constant__ CUtensorMap ml, int* status,
                                                              long long timeout_ns) {
   constexpr bool VARC = MODE == 1, ADJ = MODE == 2;
-  constexpr int RUN = run_rows(MODE), THREADS = threads_of(MODE);
   using G = G2<R, ADJ ? 2 : 1>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* stage0 = reinterpret_cast<float*>(smem_raw);
@@ -94,7 +90,7 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
   const int nx = a.nx, ny = a.ny;
   const int tiles_x = (nx + TX - 1) / TX;
   const int ntiles = tiles_x * ((ny + TY - 1) / TY);
-  const int c0 = (t % TCOLS) * 4, r0 = (t / TCOLS) * RUN;
+  const int c0 = (t % TCOLS) * 2, r0 = (t / TCOLS) * RUN;
   const bool load_d = !a.d_zero;
   const bool kv = a.kappa != nullptr;  // adjoint: varying medium (per-cell kappa)
   const unsigned stage_bytes = (unsigned)G::STAGE * 4u;
@@ -124,6 +120,10 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
   float2 w2[R + 1];  // stencil weights, packed
 #pragma unroll
   for (int m = 0; m <= R; ++m) w2[m] = dup2(a.w[m]);
+  float wc = 0.f;  // centre weight of the Z_lo stencil (sum form)
+#pragma unroll
+  for (int m = 1; m <= R; ++m) wc += a.w[m];
+  const float2 nwc = dup2(-(wc * 4.f));
   int k = 0;
   bool ok = true;
   int issued = (first < ntiles) ? 1 : 0;
@@ -141,17 +141,12 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
     const int gx0 = (tt % tiles_x) * TX, gy0 = (tt / tiles_x) * TY;
     const int gx = gx0 + c0;
     // own-cell fields straight into registers, in flight while the boxes land
-    float4 d4[RUN], kh4[RUN], kl4[RUN];
+    const float2 z2 = dup2(0.f);
+    float2 d2[RUN];
 #pragma unroll
     for (int rr = 0; rr < RUN; ++rr) {
       const int gy = gy0 + r0 + rr;
-      const bool in = gy < ny && gx < nx;
-      const long long gi = (long long)gy * nx + gx;
-      const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      d4[rr] = (load_d && in) ? ld_stream4(a.dbuf + gi) : z4;
-      kh4[rr] = ((VARC || (ADJ && kv && !a.final_step)) && in) ? __ldg(reinterpret_cast<const float4*>(a.kappa + gi))
-                                                               : z4;
-      kl4[rr] = (VARC && in) ? __ldg(reinterpret_cast<const float4*>(a.kappa_lo + gi)) : z4;
+      d2[rr] = (load_d && gy < ny && gx < nx) ? ld_stream2(a.dbuf + (long long)gy * nx + gx) : z2;
     }
     const bool good = mbar_wait(&bars[s], (k >> 1) & 1, timeout_ns);
     if (__syncthreads_or(!good)) {
@@ -168,64 +163,63 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
     // tiles outside it run exactly the code of the kernel without a layer
     auto update = [&](auto in_layer) {
       constexpr bool LAYER = decltype(in_layer)::value;
-      float lo[RUN][4];  // adjoint: the Z_lo part of the stencil, first pass
-      if (ADJ) stencil_run<R, RUN, BW, XH>(PL, r0, c0, a.w, lo);
-      // sliding window over this thread's 4 columns: win[i] = box row (row - R + i)
-      float4 win[2 * R + 1];
+      float2 lo[RUN];  // adjoint: the Z_lo part of the stencil, first pass
+      if (ADJ) stencil_run_pair<R, RUN, BW>(PL + (r0 + R) * BW + XH + c0, w2, nwc, lo);
+      // sliding window over this thread's 2 columns: win[i] = box row (row - R + i)
+      const float* own = P + (r0 + R) * BW + XH + c0;
+      float2 win[2 * R + 1];
 #pragma unroll
-      for (int i = 0; i < 2 * R; ++i) win[i] = *reinterpret_cast<const float4*>(P + (r0 + i) * BW + XH + c0);
+      for (int i = 0; i < 2 * R; ++i) win[i] = *reinterpret_cast<const float2*>(own + (i - R) * BW);
 #pragma unroll
       for (int rr = 0; rr < RUN; ++rr) {
-        win[2 * R] = *reinterpret_cast<const float4*>(P + (r0 + rr + 2 * R) * BW + XH + c0);
-        const int brow = r0 + rr + R;
-        float f[20];
-        load_row20(P + brow * BW + c0, f);
+        win[2 * R] = *reinterpret_cast<const float2*>(own + (rr + R) * BW);
+        RowPairs<R> f;
+        f.load(own + rr * BW, win[R]);
         const int gy = gy0 + r0 + rr;
         const long long gi = (long long)gy * nx + gx;
         const bool in = gy < ny && gx < nx;
-        float dn[4], pn[4], pl[4];
-        float4 sa4 = make_float4(1.f, 1.f, 1.f, 1.f), sb4 = sa4;
+        const bool want_k = (VARC || (ADJ && kv && !a.final_step)) && in;
+        const float2 kh2 = want_k ? __ldg(reinterpret_cast<const float2*>(a.kappa + gi)) : z2;
+        const float2 kl2 = (VARC && in) ? __ldg(reinterpret_cast<const float2*>(a.kappa_lo + gi)) : z2;
+        float2 sa2 = dup2(1.f), sb2 = sa2;
         if (LAYER && in) {
-          sa4 = __ldg(reinterpret_cast<const float4*>(a.sp_a + gi));
-          sb4 = __ldg(reinterpret_cast<const float4*>(a.sp_b + gi));
+          sa2 = __ldg(reinterpret_cast<const float2*>(a.sp_a + gi));
+          sb2 = __ldg(reinterpret_cast<const float2*>(a.sp_b + gi));
         }
-        float4 zl4 = make_float4(0.f, 0.f, 0.f, 0.f);  // adjoint: own Z_lo cells
-        if (ADJ) zl4 = *reinterpret_cast<const float4*>(PL + brow * BW + XH + c0);
+        float2 zl2 = z2;  // adjoint: own Z_lo cells
+        if (ADJ) zl2 = *reinterpret_cast<const float2*>(PL + (r0 + rr + R) * BW + XH + c0);
         // forward: zero-sum pair form (a + b) - 2c per tap; adjoint: difference form on Z
-        float st4[4];
-        stencil_cells2<R, ADJ>(win, f, w2, st4);
+        const float2 st2 = stencil_pair<R, ADJ>(win, f, w2);
+        float dn[2], pn[2], pl[2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float c = f[8 + j];  // own P or Z
+        for (int j = 0; j < 2; ++j) {
+          const float c = f2get(win[R], j);  // own P or Z
+          const float fa = f2get(sa2, j), fb = f2get(sb2, j);
           if (!ADJ) {
-            const float acc = st4[j];
-            const float inc = VARC ? fmaf(a.c_lap * f4get(kh4[rr], j), acc, (a.c_lap * f4get(kl4[rr], j)) * acc)
+            const float acc = f2get(st2, j);
+            const float inc = VARC ? fmaf(a.c_lap * f2get(kh2, j), acc, (a.c_lap * f2get(kl2, j)) * acc)
                                    : fmaf(ckh, acc, ckl * acc);
-            if (!LAYER) {
-              dn[j] = f4get(d4[rr], j) + inc;
-            } else {  // forward in the layer
-              const float fa = f4get(sa4, j), fb = f4get(sb4, j);
-              dn[j] = load_d ? fmaf(fa, f4get(d4[rr], j), fb * inc) : fmaf(fa - 1.f, c, fb * inc);
-            }
+            if (!LAYER)
+              dn[j] = f2get(d2[rr], j) + inc;
+            else  // forward in the layer
+              dn[j] = load_d ? fmaf(fa, f2get(d2[rr], j), fb * inc) : fmaf(fa - 1.f, c, fb * inc);
             pn[j] = c + dn[j];
             pl[j] = 0.f;
           } else {
-            const float acc = st4[j] + lo[rr][j];
-            const float g = f4get(d4[rr], j) + a.c_lap * acc;  // G' (S^T r injected into G beforehand)
-            const float zl = f4get(zl4, j);
+            const float acc = f2get(st2, j) + f2get(lo[rr], j);
+            const float g = f2get(d2[rr], j) + a.c_lap * acc;  // G' (S^T r injected into G beforehand)
+            const float zl = f2get(zl2, j);
             dn[j] = g;
             if (a.final_step) {
               pn[j] = g;
               if (LAYER) {  // x = G' + ((a-1)/b) Q,  Q = (Z + Z_lo) / kappa
-                const float fa = f4get(sa4, j), fb = f4get(sb4, j);
                 const float kap = kv ? a.kappa[gi + j] : a.kappa0;
                 if (in && fa != 1.f) pn[j] = fmaf((fa - 1.f) / fb, (c + zl) / kap, g);
               }
               pl[j] = 0.f;
             } else {
-              const float u = kv ? f4get(kh4[rr], j) * g : fmaf(a.kappa0, g, a.kappa0_lo * g);  // kappa G'
-              if (LAYER && (f4get(sa4, j) != 1.f || f4get(sb4, j) != 1.f)) {  // Z' = a Z + b kappa G'
-                const float fa = f4get(sa4, j), fb = f4get(sb4, j);
+              const float u = kv ? f2get(kh2, j) * g : fmaf(a.kappa0, g, a.kappa0_lo * g);  // kappa G'
+              if (LAYER && (fa != 1.f || fb != 1.f)) {  // Z' = a Z + b kappa G'
                 pn[j] = fmaf(fa, c, fb * u);
                 pl[j] = fa * zl;
               } else {
@@ -237,10 +231,10 @@ __global__ void __launch_bounds__(threads_of(MODE)) step2d_tma_kernel(const Step
           }
         }
         if (in) {
-          *reinterpret_cast<float4*>(a.next + gi) = make_float4(pn[0], pn[1], pn[2], pn[3]);
+          *reinterpret_cast<float2*>(a.next + gi) = make_float2(pn[0], pn[1]);
           if (!a.final_step) {
-            *reinterpret_cast<float4*>(a.dbuf + gi) = make_float4(dn[0], dn[1], dn[2], dn[3]);
-            if (ADJ) *reinterpret_cast<float4*>(a.next_lo + gi) = make_float4(pl[0], pl[1], pl[2], pl[3]);
+            *reinterpret_cast<float2*>(a.dbuf + gi) = make_float2(dn[0], dn[1]);
+            if (ADJ) *reinterpret_cast<float2*>(a.next_lo + gi) = make_float2(pl[0], pl[1]);
           }
         }
 #pragma unroll
@@ -335,7 +329,7 @@ int tma2d_ctas(int nx, int ny, int R, int mode, int sp) {
     const size_t smem = smem_for(R, mode);
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads_of(mode), smem) != cudaSuccess || per < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, THREADS, smem) != cudaSuccess || per < 1) {
       cudaGetLastError();
       per = 1;
     }
@@ -346,7 +340,7 @@ int tma2d_ctas(int nx, int ny, int R, int mode, int sp) {
 }
 
 long long tma2d_threads(int nx, int ny, int R, int mode, int sp) {
-  return (long long)tma2d_ctas(nx, ny, R, mode, sp) * threads_of(mode);
+  return (long long)tma2d_ctas(nx, ny, R, mode, sp) * THREADS;
 }
 
 cudaError_t step2d_tma_launch(int R, int mode, int sp, const StepArgs& a, const CUtensorMap& p, const CUtensorMap& lo,
@@ -359,7 +353,7 @@ cudaError_t step2d_tma_launch(int R, int mode, int sp, const StepArgs& a, const 
   void* params[] = {&args, &map, &mapl, &status, &timeout_ns};
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(nctas);
-  cfg.blockDim = dim3(threads_of(mode));
+  cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = smem_for(R, mode);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];  // starts while the previous step drains (the kernel waits for it itself)
