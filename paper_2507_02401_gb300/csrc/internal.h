@@ -94,10 +94,14 @@ struct Persist2DArgs {
 //   3D (three-level form): next = c_cur cur - c_prev prev + c_lap kappa L cur
 //      (adjoint: L(kappa cur)).
 //   2D adjoint carries compensation terms in cur_lo/next_lo (and dbuf_lo): the TMA kernel keeps
-//      the state Z = kappa Q with its low part in cur_lo/next_lo (G plain); the plain kernel keeps
-//      Q with Q_lo there and G_lo in dbuf_lo, feeding the stencil kappa*Q as a hi + lo pair.
+//      the state Z = kappa Q with its low part in cur_lo/next_lo (G plain, or with G_lo in dbuf_lo on
+//      grids of odd width); the plain kernel keeps Q with Q_lo there and G_lo in dbuf_lo, feeding the
+//      stencil kappa*Q as a hi + lo pair.
+//   3D adjoint of a varying medium on the TMA kernel: the state is Z = kappa Q (plain),
+//      Z^n = 2 Z^{n+1} - Z^{n+2} + kappa (L Z^{n+1} + S^T r_n); the final step divides by kappa.
 struct StepArgs {
   int nx, ny, nz;
+  int pitch;  // floats from one row of a field (and of kappa, sp_a, sp_b) to the next, >= nx
   float w[kMaxR + 1];
   float kappa0, kappa0_lo;
   const float* kappa;     // or nullptr
@@ -109,7 +113,7 @@ struct StepArgs {
   const float* prev;   // 3D: P^{n-1} or Q^{n+2}   (nullptr = 0)
   float* dbuf;         // 2D: increment D (forward) / G (adjoint), updated in place
   int d_zero;          // 2D: treat the incoming increment as 0
-  int final_step;      // 2D adjoint: next = dbuf + c_lap L(kappa cur)
+  int final_step;      // 2D adjoint: next = dbuf + c_lap L(kappa cur); 3D TMA, varying medium: leave Z = kappa Q
   float* next;         // P^{n+1} or Q^n (or the adjoint's result)
   float c_lap;         // coefficient of kappa*L (1, or 0.5 for the first/last step)
   float c_cur;         // 3D: coefficient of the current field (2, or 1)
@@ -154,33 +158,35 @@ cudaError_t persist2d_launch_layer(int R, bool adj, bool varc, const Persist2DAr
 cudaError_t persist2d_split_combine(const float* part, const int* split_sensor, int nsplit, int nt, float* y,
                                     cudaStream_t st);
 
-// wave3d_tma.cu: constant-medium 3D step with TMA plane pipelines
-bool tma3d_supported(int nx, int R, bool varc);
-// `cur` (80 x (16+2R) x 1 boxes) and `prev` (64 x 16 x 1) descriptors of an nx x ny x nz float field
-cudaError_t tma3d_encode(const float* base, int nx, int ny, int nz, int R, CUtensorMap* cur, CUtensorMap* prev);
+// wave3d_tma.cu: 3D step with TMA plane pipelines
+bool tma3d_supported(int R);
+// `cur` (halo) and `prev` (64 x 16 x 1) box descriptors of an nx x ny x nz float field of row pitch `pitch`
+cudaError_t tma3d_encode(const float* base, int nx, int pitch, int ny, int nz, int R, CUtensorMap* cur,
+                         CUtensorMap* prev);
 // Work split of a 3D TMA step launch: nctas = columns x nchunks CTAs, column-fastest, each a z range
 // of nz / nchunks planes; ring: the kernel form whose z queue is a register ring (one-wave grids).
 struct Tma3dSplit {
   int nctas, nchunks;
   bool ring;
 };
-Tma3dSplit tma3d_split(int R, int nx, int ny, int nz);
+Tma3dSplit tma3d_split(int R, bool varc, int nx, int ny, int nz);
 int tma3d_cta_of(int nx, int ny, int nz, const Tma3dSplit& sp, int x, int y, int z);  // CTA holding a cell
 long long tma3d_threads(int nctas);  // threads of one launch (fused sampling)
-cudaError_t step3d_tma_launch(int R, const StepArgs& a, const CUtensorMap& cur, const CUtensorMap& prev, const Tma3dSplit& sp,
-                              int* status, long long timeout_ns, cudaStream_t st);
+// a.kappa: varying medium (the adjoint in its Z form; a.final_step: the adjoint's last step)
+cudaError_t step3d_tma_launch(int R, const StepArgs& a, const CUtensorMap& cur, const CUtensorMap& prev,
+                              const Tma3dSplit& sp, int* status, long long timeout_ns, cudaStream_t st);
 
-// wave2d_tma.cu: 2D increment-form step with TMA tile pipelines (forward; constant-medium adjoint)
-bool tma2d_supported(int nx, int R);
+// wave2d_tma.cu: 2D increment-form step with TMA tile pipelines
+bool tma2d_supported(int R);
 int tma2d_tile();  // tile edge in cells (tiles numbered row by row)
-// P boxes (80 x (64+2R)) and own-tile boxes (64 x 64) of an nx x ny float field
-cudaError_t tma2d_encode(const float* base, int nx, int ny, int R, CUtensorMap* halo, CUtensorMap* own);
-// mode 0: constant medium, 1: varying medium (forward), 2: constant medium with fused injection (adjoint),
-// 3: varying-medium adjoint (k: kappa's halo-box descriptor, unused by the other modes);
-// sp 0: no absorbing layer, 1: layer with the forward update, 2: layer with the adjoint update
-long long tma2d_threads(int nx, int ny, int R, int mode, int sp);  // threads of one launch (fused sampling)
-cudaError_t step2d_tma_launch(int R, int mode, int sp, const StepArgs& a, const CUtensorMap& p, const CUtensorMap& k,
-                              int* status, long long timeout_ns, cudaStream_t st);
+// halo boxes (80 x (64+2R)) of an nx x ny float field of row pitch `pitch`
+cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CUtensorMap* halo);
+// mode 0: forward, constant medium; 1: forward, varying medium; 2: adjoint (either medium);
+// sp 0: no absorbing layer, 1: layer with the forward update, 2: layer with the adjoint update;
+// full: forward stencil in the difference form, adjoint with G compensated in a.dbuf_lo
+long long tma2d_threads(int nx, int ny, int R, int mode, int sp, bool full);  // threads of one launch
+cudaError_t step2d_tma_launch(int R, int mode, int sp, bool full, const StepArgs& a, const CUtensorMap& p,
+                              const CUtensorMap& lo, int* status, long long timeout_ns, cudaStream_t st);
 
 // wave_step.cu
 cudaError_t step2d_launch(int R, bool adj, const StepArgs& a, cudaStream_t st);
@@ -188,7 +194,11 @@ cudaError_t step3d_launch(int R, bool adj, const StepArgs& a, cudaStream_t st);
 cudaError_t sample_launch(const float* P, int ns, int nt, int t, const int* cell, const float* w, int corners,
                           float* y, cudaStream_t st);
 cudaError_t inject_launch(float* Q, int n_inj, const int* inj_cell, const int* inj_ptr, const int* ent_sensor,
-                          const float* ent_w, const float* r, int nt, int t, float scale, cudaStream_t st);
+                          const float* ent_w, const float* r, int nt, int t, const float* cell_scale,
+                          cudaStream_t st);  // cell_scale: per-cell factor (nullptr = 1)
+// rows of nx floats from one pitch to another
+cudaError_t pitch_copy_launch(float* dst, int dpitch, const float* src, int spitch, int nx, long long rows,
+                              cudaStream_t st);
 // zform: the adjoint state holds Z = kappa Q (2D TMA engine); the accumulator divides by kappa
 cudaError_t grad_acc_launch(int R, double* gacc, const float* Q, const float* Qlo, const float* P, float coef,
                             const StepArgs& a, int dim, bool zform, cudaStream_t st);

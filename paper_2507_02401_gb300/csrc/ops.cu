@@ -57,19 +57,20 @@ static StepArgs step_args(pat_plan* p) {
   a.nx = p->n[0];
   a.ny = p->n[1];
   a.nz = p->n[2];
+  a.pitch = p->pitch;
   for (int m = 0; m <= kMaxR; ++m) a.w[m] = p->w[m];
   a.kappa0 = p->kappa0;
   a.kappa0_lo = p->kappa0_lo;
-  a.kappa = p->varc ? p->d_kappa : nullptr;
-  a.kappa_lo = p->varc ? p->d_kappa_lo : nullptr;
+  a.kappa = p->varc ? p->s_kappa : nullptr;
+  a.kappa_lo = p->varc ? p->s_kappa_lo : nullptr;
   a.ns = p->ns;
   a.nt = p->nt;
   a.sens_cell = p->d_sens_cell;
   a.sens_w = p->d_sens_w;
   a.corners = p->corners;
   if (p->sponge_w > 0) {
-    a.sp_a = p->d_sp_a;
-    a.sp_b = p->d_sp_b;
+    a.sp_a = p->s_sp_a;
+    a.sp_b = p->s_sp_b;
     a.sp_w = p->sponge_w;
   }
   return a;
@@ -81,30 +82,45 @@ static const pat_plan::TmaDesc* tma_desc(pat_plan* p, const float* base) {
     if (d.base == base) return &d;
   pat_plan::TmaDesc d;
   d.base = base;
-  const cudaError_t e = p->dim == 3 ? tma3d_encode(base, p->n[0], p->n[1], p->n[2], p->R, &d.halo, &d.own)
-                                     : tma2d_encode(base, p->n[0], p->n[1], p->R, &d.halo, &d.own);
+  const cudaError_t e = p->dim == 3 ? tma3d_encode(base, p->n[0], p->pitch, p->n[1], p->n[2], p->R, &d.halo, &d.own)
+                                     : tma2d_encode(base, p->n[0], p->pitch, p->n[1], p->R, &d.halo);
   if (e != cudaSuccess) return nullptr;
   if (p->tma_desc.size() >= 16) p->tma_desc.erase(p->tma_desc.begin());
   p->tma_desc.push_back(d);
   return &p->tma_desc.back();
 }
 
-// The TMA kernels take 16-byte aligned fields (descriptor bases, float4 stores).
-static bool tma_ready(pat_plan* p, const StepArgs& a) {
-  auto al = [](const void* q) { return q == nullptr || ((uintptr_t)q & 15) == 0; };
-  return al(a.cur) && al(a.prev) && al(a.next) && (p->dim == 3 || (al(a.dbuf) && al(a.cur_lo) && al(a.next_lo)));
+// Whether a caller's image can serve as a field of the step engines as it stands: dense rows, and for the TMA
+// kernels a 16-byte aligned base.
+static bool image_is_field(const pat_plan* p, const float* img) {
+  return p->pitch == p->n[0] && (!(p->tma2d || p->tma3d) || ((uintptr_t)img & 15) == 0);
 }
+
+static cudaError_t image_to_field(const pat_plan* p, float* field, const float* img, cudaStream_t st) {
+  return pitch_copy_launch(field, p->pitch, img, p->n[0], p->n[0], (long long)p->n[1] * p->n[2], st);
+}
+
+static cudaError_t field_to_image(const pat_plan* p, float* img, const float* field, cudaStream_t st) {
+  return pitch_copy_launch(img, p->n[0], field, p->pitch, p->n[0], (long long)p->n[1] * p->n[2], st);
+}
+
+// Per-cell factor of the adjoint's injection: kappa where the state is Z = kappa Q injected after the kappa
+// product (3D TMA kernel, varying medium).
+static const float* inj_scale(const pat_plan* p) { return p->tma3d && p->varc ? p->s_kappa : nullptr; }
 
 static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t st) {
   // sample separately when the step grid has fewer threads than sensors
   float* y = a.y;
   cudaError_t e;
-  if (p->dim == 2 && p->tma2d && tma_ready(p, a)) {
+  if (p->tma2d) {
     // TMA tile pipelines: forward (constant or varying medium); adjoint in Z = kappa Q with Z
     // compensated (boxes of Z and Z_lo), the next step's injection added to G after each tile
     const int mode = adj ? 2 : (p->varc ? 1 : 0);
     const int sp = p->sponge_w > 0 ? (adj ? 2 : 1) : 0;
-    const long long nthr = tma2d_threads(p->n[0], p->n[1], p->R, mode, sp);
+    // odd widths used to take the plain kernel, whose forward stencil is the difference form and whose adjoint
+    // carries G as a compensated pair: the kernel's full form keeps that accuracy
+    const bool full = p->n[0] % 4 != 0;
+    const long long nthr = tma2d_threads(p->n[0], p->n[1], p->R, mode, sp, full);
     if (y && a.ns > nthr) a.y = nullptr;
     // copies: a second lookup may move the cached descriptors
     const pat_plan::TmaDesc* dp = tma_desc(p, a.cur);
@@ -122,7 +138,7 @@ static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t 
     b.inj_tile = p->d_tinj_step;
     b.ent_sensor = p->d_ent_sensor;
     b.ent_w = p->d_ent_w;
-    e = step2d_tma_launch(p->R, mode, sp, b, mcur, mlo, p->d_status, p->timeout_ns, st);
+    e = step2d_tma_launch(p->R, mode, sp, full, b, mcur, mlo, p->d_status, p->timeout_ns, st);
   } else if (p->dim == 2) {
     const long long nthr = (long long)((p->n[0] + 63) / 64) * ((p->n[1] + 31) / 32) * 256;
     if (y && a.ns > nthr) a.y = nullptr;
@@ -131,8 +147,8 @@ static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t 
     e = step2d_launch(p->R, adj, b, st);
     if (e == cudaSuccess && a.inj_r)
       e = inject_launch(a.dbuf, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, a.inj_r, p->nt,
-                        a.inj_t, 1.f, st);
-  } else if (p->tma3d && tma_ready(p, a)) {
+                        a.inj_t, nullptr, st);
+  } else if (p->tma3d) {
     const long long nthr = tma3d_threads(p->tma3d_split.nctas);
     if (y && a.ns > nthr) a.y = nullptr;
     if (a.inj_r) {  // the adjoint's post-step injection, fused per CTA
@@ -161,7 +177,7 @@ static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t 
     e = step3d_launch(p->R, adj, b, st);
     if (e == cudaSuccess && a.inj_r)  // the adjoint's injection after the step
       e = inject_launch(a.next, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, a.inj_r, p->nt,
-                        a.inj_t, 1.f, st);
+                        a.inj_t, nullptr, st);
   }
   if (e == cudaSuccess && y && !a.y)
     e = sample_launch(a.cur, p->ns, p->nt, a.t_sample, p->d_sens_cell, p->d_sens_w, p->corners, y, st);
@@ -179,6 +195,11 @@ static pat_status wave_forward_impl(pat_plan* p, const float* x, float* y, cudaS
     return PAT_OK;
   }
   const int nt = p->nt;
+  if (!image_is_field(p, x)) {  // into a buffer that the steps below leave alone
+    float* f = p->dim == 2 ? p->d_wv[3] : p->d_wv[2];
+    PAT_TRY_CUDA(image_to_field(p, f, x, st));
+    x = f;
+  }
   if (nt == 1) {
     PAT_TRY_CUDA(sample_launch(x, p->ns, nt, 0, p->d_sens_cell, p->d_sens_w, p->corners, y, st));
     return PAT_OK;
@@ -228,30 +249,33 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
     return PAT_OK;
   }
   const int nt = p->nt;
-  auto inject = [&](float* Q, int t) {
-    return inject_launch(Q, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, y, nt, t, 1.f, st);
+  auto inject = [&](float* Q, int t, const float* scale) {
+    return inject_launch(Q, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, y, nt, t, scale, st);
   };
+  // the last step's result: the caller's image, or a free field buffer copied to it at the end
+  const bool direct = image_is_field(p, x);
+  auto result = [&](float* free_field) { return direct ? x : free_field; };
   if (nt == 1) {
-    PAT_TRY_CUDA(fill_launch(x, p->N, 0.f, st));
-    PAT_TRY_CUDA(inject(x, 0));
+    float* f = result(p->d_wv[0]);
+    PAT_TRY_CUDA(fill_launch(f, p->Np, 0.f, st));
+    PAT_TRY_CUDA(inject(f, 0, nullptr));
+    if (!direct) PAT_TRY_CUDA(field_to_image(p, x, f, st));
     return PAT_OK;
   }
   StepArgs a = step_args(p);
   a.y = nullptr;
   if (p->dim == 2) {
     // increment form with compensation: G = wv[2] (+ wv[5]); Q^m in wv[(nt-m) % 2]
-    // (+ wv[3 + (nt-m) % 2]) with Q^nt = 0.  The TMA kernel keeps Z = kappa Q there (and no G_lo);
-    // the plain kernel Q itself, so every step of one application runs on the same kernel: with
-    // the TMA kernel an output that is not 16-byte aligned is written to a free field buffer
-    // (Q^2's, no longer read by the final step) and copied.
+    // (+ wv[3 + (nt-m) % 2]) with Q^nt = 0.  The TMA kernel keeps Z = kappa Q there (and G_lo on odd widths
+    // only); the plain kernel Q itself.
     float* G = p->d_wv[2];
     auto Qbuf = [&](int m) { return p->d_wv[(nt - m) % 2]; };
     auto Qlo = [&](int m) { return p->d_wv[3 + (nt - m) % 2]; };
-    PAT_TRY_CUDA(fill_launch(G, p->N, 0.f, st));
-    PAT_TRY_CUDA(fill_launch(p->d_wv[5], p->N, 0.f, st));
-    PAT_TRY_CUDA(fill_launch(Qbuf(nt), p->N, 0.f, st));
-    PAT_TRY_CUDA(fill_launch(Qlo(nt), p->N, 0.f, st));
-    PAT_TRY_CUDA(inject(G, nt - 1));
+    PAT_TRY_CUDA(fill_launch(G, p->Np, 0.f, st));
+    PAT_TRY_CUDA(fill_launch(p->d_wv[5], p->Np, 0.f, st));
+    PAT_TRY_CUDA(fill_launch(Qbuf(nt), p->Np, 0.f, st));
+    PAT_TRY_CUDA(fill_launch(Qlo(nt), p->Np, 0.f, st));
+    PAT_TRY_CUDA(inject(G, nt - 1, nullptr));
     a.dbuf = G;
     a.dbuf_lo = p->d_wv[5];
     a.inj_r = y;  // each step leaves G^m + S^T r_{m-1} for the next
@@ -271,19 +295,19 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
     a.inj_r = nullptr;
     a.cur = Qbuf(1);
     a.cur_lo = Qlo(1);
-    const bool staged = p->tma2d && ((uintptr_t)x & 15) != 0;
-    a.next = staged ? Qbuf(2) : x;
+    a.next = result(Qbuf(2));
     a.next_lo = nullptr;
     a.final_step = 1;
     a.c_lap = 0.5f;
     PAT_TRY_CUDA(step_launch(p, true, a, st));
-    if (staged) PAT_TRY_CUDA(cudaMemcpyAsync(x, Qbuf(2), sizeof(float) * p->N, cudaMemcpyDeviceToDevice, st));
+    if (!direct) PAT_TRY_CUDA(field_to_image(p, x, a.next, st));
     return PAT_OK;
   }
-  // three-level form: Q^m lives in wv[(nt-1-m) % 2], over Q^{m+2} (as in the forward map)
+  // three-level form: Q^m (Z^m = kappa Q^m where inj_scale says so) lives in wv[(nt-1-m) % 2], over Q^{m+2}
+  // (as in the forward map)
   auto Qbuf = [&](int m) { return p->d_wv[(nt - 1 - m) % 2]; };
-  PAT_TRY_CUDA(fill_launch(Qbuf(nt - 1), p->N, 0.f, st));
-  PAT_TRY_CUDA(inject(Qbuf(nt - 1), nt - 1));
+  PAT_TRY_CUDA(fill_launch(Qbuf(nt - 1), p->Np, 0.f, st));
+  PAT_TRY_CUDA(inject(Qbuf(nt - 1), nt - 1, inj_scale(p)));
   a.inj_r = y;  // S^T r_m added to Q^m by (or just after) the step that makes it
   for (int m = nt - 2; m >= 1; --m) {
     a.flip = m & 1;
@@ -299,12 +323,14 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
   a.flip = 0;
   a.cur = Qbuf(1);
   a.prev = (nt >= 3) ? Qbuf(2) : nullptr;
-  a.next = x;
+  a.next = result(p->d_wv[2]);
+  a.final_step = 1;
   a.c_cur = 1.f;
   a.c_prev = 1.f;
   a.c_lap = 0.5f;
   a.inj_t = 0;
   PAT_TRY_CUDA(step_launch(p, true, a, st));
+  if (!direct) PAT_TRY_CUDA(field_to_image(p, x, a.next, st));
   return PAT_OK;
 }
 
@@ -492,11 +518,11 @@ static void kg_free(pat_plan* p) {
 static pat_status kg_alloc(pat_plan* p, int C, int nseg) {
   if (p->kg_segment == C) return PAT_OK;
   kg_free(p);
-  const size_t N = (size_t)p->N;
+  const size_t N = (size_t)p->Np;
   cudaError_t e = cudaMalloc(&p->kg_ckpt, sizeof(float) * N * 2 * nseg);
   if (e == cudaSuccess) e = cudaMalloc(&p->kg_seg, sizeof(float) * N * C);
   if (e == cudaSuccess) e = cudaMalloc(&p->kg_work, sizeof(float) * N * 3);
-  if (e == cudaSuccess) e = cudaMalloc(&p->kg_acc, sizeof(double) * N);
+  if (e == cudaSuccess) e = cudaMalloc(&p->kg_acc, sizeof(double) * (size_t)p->N);
   if (e != cudaSuccess) {
     cudaGetLastError();
     kg_free(p);
@@ -507,10 +533,10 @@ static pat_status kg_alloc(pat_plan* p, int C, int nseg) {
 }
 
 pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float* g, int C, cudaStream_t st) {
-  const long long N = p->N;
+  const long long N = p->Np;  // floats of a field
   const int nt = p->nt;
   if (nt < 2) {
-    PAT_TRY_CUDA(fill_launch(g, N, 0.f, st));
+    PAT_TRY_CUDA(fill_launch(g, p->N, 0.f, st));
     return PAT_OK;
   }
   if (C <= 0) C = (int)std::ceil(std::sqrt((double)nt));
@@ -528,6 +554,10 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
   };
   StepArgs a = step_args(p);
   a.y = nullptr;
+  if (!image_is_field(p, x)) {  // a field buffer that only the adjoint run below uses
+    PAT_TRY_CUDA(image_to_field(p, p->d_wv[0], x, st));
+    x = p->d_wv[0];
+  }
 
   // ---- forward run keeping the restart state at n = 0, C, 2C, ...
   if (two_d) {  // increment form: state (P^n, D^n)
@@ -603,14 +633,15 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
     const int n = m - 1;
     if (n / C != loaded) PAT_TRY(load_segment(n / C));
     PAT_TRY_CUDA(grad_acc_launch(p->R, p->kg_acc, Q, Qlo, seg(n - loaded * C), n == 0 ? 0.5f : 1.f, a, p->dim,
-                                 two_d && p->tma2d, st));
+                                 two_d ? p->tma2d : p->tma3d && p->varc, st));
     return PAT_OK;
   };
-  PAT_TRY_CUDA(dfill_launch(p->kg_acc, N, st));
+  PAT_TRY_CUDA(dfill_launch(p->kg_acc, p->N, st));
 
   // ---- adjoint run with the residual r, accumulating the gradient
   auto inject = [&](float* Q, int t) {
-    return inject_launch(Q, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, r, nt, t, 1.f, st);
+    return inject_launch(Q, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, r, nt, t,
+                         inj_scale(p), st);
   };
   StepArgs c = step_args(p);
   c.y = nullptr;
@@ -655,7 +686,7 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
       PAT_TRY(accumulate(m, Qbuf(m), nullptr));
     }
   }
-  PAT_TRY_CUDA(d2f_launch(g, p->kg_acc, N, st));
+  PAT_TRY_CUDA(d2f_launch(g, p->kg_acc, p->N, st));
   return PAT_OK;
 }
 

@@ -15,6 +15,7 @@
 #include <tuple>
 
 #include "plan.h"
+#include "tma.cuh"
 
 namespace pat {
 
@@ -158,6 +159,20 @@ bool daubechies_filter(int nv, double* h) {
     if (std::fabs(s - (m == 0 ? 1.0 : 0.0)) > 1e-12) return false;
   }
   return true;
+}
+
+// A dense device array at the step engines' row pitch: a padded copy, or the array itself when they agree.
+static pat_status pitched(pat_plan* p, float* dense, float** out, const char* what, cudaStream_t st) {
+  if (p->pitch == p->n[0]) {
+    *out = dense;
+    return PAT_OK;
+  }
+  if (!*out) {
+    PAT_TRY(plan_alloc(p, reinterpret_cast<void**>(out), sizeof(float) * (size_t)p->Np, what));
+    PAT_TRY_CUDA(cudaMemsetAsync(*out, 0, sizeof(float) * (size_t)p->Np, st));
+  }
+  PAT_TRY_CUDA(pitch_copy_launch(*out, p->pitch, dense, p->n[0], p->n[0], (long long)p->n[1] * p->n[2], st));
+  return PAT_OK;
 }
 
 // --------------------------------------------------- persistent 2D set-up
@@ -305,6 +320,24 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
   p->ns = ns;
   p->corners = 1 << p->dim;
 
+  // ---- step engines: TMA kernels when the driver provides the descriptor encoder.  Their rows start on
+  // 16-byte boundaries, so fields of other widths get padded rows (the pad columns are never read back: the
+  // descriptors end at nx).
+  const char* env2 = getenv("PAT_STEP2D");
+  const char* env3 = getenv("PAT_STEP3D");
+  const char* env = p->dim == 2 ? env2 : env3;
+  bool tma = tma_encoder() != nullptr && !(env && strcmp(env, "plain") == 0) &&
+             (p->dim == 2 ? tma2d_supported(p->R) : tma3d_supported(p->R));
+  p->pitch = p->n[0];
+  if (tma) {
+    p->pitch = (p->n[0] + 3) / 4 * 4;
+    if ((long long)p->pitch * p->n[1] * p->n[2] >= (1LL << 31)) {  // cell indices are int
+      tma = p->n[0] % 4 == 0;
+      p->pitch = p->n[0];
+    }
+  }
+  p->Np = (long long)p->pitch * p->n[1] * p->n[2];
+
   // ---- medium and CFL (c_max dt / h <= 1 / (sqrt(d) sum |c_k|))
   double cmax = 0.0, cmin = 0.0;
   bool constant = true;
@@ -356,6 +389,9 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
     }
     PAT_TRY(upload(p, &p->d_kappa, kap, "kappa", st));
     PAT_TRY(upload(p, &p->d_kappa_lo, kap_lo, "kappa residual", st));
+    PAT_TRY(pitched(p, p->d_kappa, &p->s_kappa, "kappa", st));
+    PAT_TRY(pitched(p, p->d_kappa_lo, &p->s_kappa_lo, "kappa residual", st));
+    PAT_TRY_CUDA(cudaStreamSynchronize(st));  // the host vectors go out of scope
   }
 
   // ---- sensors: interpolation weights in FP64, cell index floor(u) clamped to n-2
@@ -407,9 +443,15 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
   }
   p->h_inj_ptr.push_back((int)ent.size());
   p->n_inj = (int)p->h_inj_cell.size();
-  PAT_TRY(upload(p, &p->d_sens_cell, p->h_sens_cell, "sensor cells", st));
+  auto pitched_cells = [&](std::vector<int> v) {  // dense cell indices -> indices into the step engines' fields
+    if (p->pitch != p->n[0])
+      for (int& c : v) c = (int)((long long)(c / p->n[0]) * p->pitch + c % p->n[0]);
+    return v;
+  };
+  const std::vector<int> sens_cell = pitched_cells(p->h_sens_cell), inj_cell = pitched_cells(p->h_inj_cell);
+  PAT_TRY(upload(p, &p->d_sens_cell, sens_cell, "sensor cells", st));
   PAT_TRY(upload(p, &p->d_sens_w, p->h_sens_w, "sensor weights", st));
-  PAT_TRY(upload(p, &p->d_inj_cell, p->h_inj_cell, "injection cells", st));
+  PAT_TRY(upload(p, &p->d_inj_cell, inj_cell, "injection cells", st));
   PAT_TRY(upload(p, &p->d_inj_ptr, p->h_inj_ptr, "injection offsets", st));
   PAT_TRY(upload(p, &p->d_ent_sensor, ent_sensor, "injection sensors", st));
   PAT_TRY(upload(p, &p->d_ent_w, ent_w, "injection weights", st));
@@ -431,7 +473,7 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
 
   // ---- workspace
   const size_t N = (size_t)p->N;
-  for (int i = 0; i < (p->dim == 2 ? 6 : 3); ++i) PAT_TRY(alloc_n(p, &p->d_wv[i], N, "wave fields"));
+  for (int i = 0; i < (p->dim == 2 ? 6 : 3); ++i) PAT_TRY(alloc_n(p, &p->d_wv[i], (size_t)p->Np, "wave fields"));
   PAT_TRY(alloc_n(p, &p->d_dwt_a, N >> p->dim, "dwt approximation"));
   PAT_TRY(alloc_n(p, &p->d_dwt_b, N >> p->dim, "dwt approximation"));
   if (p->dim == 3) {
@@ -464,23 +506,17 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
     }
   }
   p->path = p->persist_ok ? PAT_PATH_PERSISTENT : PAT_PATH_STEP;
-  const char* env = getenv("PAT_WAVE_PATH");
-  if (env && strcmp(env, "step") == 0) p->path = PAT_PATH_STEP;
+  const char* env_path = getenv("PAT_WAVE_PATH");
+  if (env_path && strcmp(env_path, "step") == 0) p->path = PAT_PATH_STEP;
 
-  // 2D per-step engine: TMA tile pipelines when the driver can encode the descriptors
-  p->tma2d = false;
-  const char* env2 = getenv("PAT_STEP2D");
-  if (p->dim == 2 && tma2d_supported(p->n[0], p->R) && !(env2 && strcmp(env2, "plain") == 0)) {
-    CUtensorMap mh, mo;
-    if (tma2d_encode(p->d_wv[0], p->n[0], p->n[1], p->R, &mh, &mo) == cudaSuccess) p->tma2d = true;
-  }
-  // 3D constant media: TMA plane pipelines when the driver can encode the descriptors
-  p->tma3d = false;
-  const char* env3 = getenv("PAT_STEP3D");
-  if (p->dim == 3 && tma3d_supported(p->n[0], p->R, p->varc) && !(env3 && strcmp(env3, "plain") == 0)) {
+  p->tma2d = p->tma3d = false;
+  if (tma && p->dim == 2) {
+    CUtensorMap mh;
+    p->tma2d = tma2d_encode(p->d_wv[0], p->n[0], p->pitch, p->n[1], p->R, &mh) == cudaSuccess;
+  } else if (tma) {
     CUtensorMap mc, mp;
-    if (tma3d_encode(p->d_wv[0], p->n[0], p->n[1], p->n[2], p->R, &mc, &mp) == cudaSuccess) {
-      p->tma3d_split = tma3d_split(p->R, p->n[0], p->n[1], p->n[2]);
+    if (tma3d_encode(p->d_wv[0], p->n[0], p->pitch, p->n[1], p->n[2], p->R, &mc, &mp) == cudaSuccess) {
+      p->tma3d_split = tma3d_split(p->R, p->varc, p->n[0], p->n[1], p->n[2]);
       p->tma3d = p->tma3d_split.nctas > 0;
     }
   }
@@ -492,7 +528,7 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
       const long long c = p->h_inj_cell[i];
       const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
       const int bin = p->tma3d ? tma3d_cta_of(nx, ny, nz, p->tma3d_split, x, y, z) : (y / T) * tx + x / T;
-      bins[bin].push_back(InjCell{(int)c, p->h_inj_ptr[i], p->h_inj_ptr[i + 1]});
+      bins[bin].push_back(InjCell{inj_cell[i], p->h_inj_ptr[i], p->h_inj_ptr[i + 1]});
     }
     std::vector<int> ptr(1, 0);
     std::vector<InjCell> cells;
@@ -654,6 +690,8 @@ pat_status pat_plan_set_sponge(pat_plan* plan, int width, double sigma_max, void
     }
   PAT_TRY_CUDA(cudaMemcpyAsync(plan->d_sp_a, fa.data(), sizeof(float) * plan->N, cudaMemcpyHostToDevice, st));
   PAT_TRY_CUDA(cudaMemcpyAsync(plan->d_sp_b, fb.data(), sizeof(float) * plan->N, cudaMemcpyHostToDevice, st));
+  PAT_TRY(pitched(plan, plan->d_sp_a, &plan->s_sp_a, "layer factors", st));
+  PAT_TRY(pitched(plan, plan->d_sp_b, &plan->s_sp_b, "layer factors", st));
   PAT_TRY_CUDA(cudaStreamSynchronize(st));
   plan->sponge_w = width;
   plan->sponge_sigma_max = smax;

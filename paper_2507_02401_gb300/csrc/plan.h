@@ -10,6 +10,8 @@ struct pat_plan {
   int dim = 2;
   int n[3] = {1, 1, 1};  // nx, ny, nz
   long long N = 0;
+  int pitch = 1;      // row pitch of the step engines' fields: nx, rounded up to 4 for the TMA kernels
+  long long Np = 0;   // floats of such a field (pitch * ny * nz)
   double h = 0, dt = 0;
   int nt = 0, order = 2, M = 1, R = 1, ns = 0, corners = 4;
   double c_max = 0;
@@ -18,9 +20,11 @@ struct pat_plan {
   float kappa0_lo = 0.f;  // rounding residual of kappa0
   float* d_kappa = nullptr;
   float* d_kappa_lo = nullptr;  // rounding residual of kappa (varying medium)
+  float *s_kappa = nullptr, *s_kappa_lo = nullptr;  // the same at the step engines' pitch (aliases when it is nx)
   float w[pat::kMaxR + 1] = {0};  // composed stencil weights w[1..R]
 
-  // ---- sensors: sampling (ns x corners) and the transposed injection CSR
+  // ---- sensors: sampling (ns x corners) and the transposed injection CSR (device cell indices are those of
+  // the step engines' pitched fields, host ones those of the dense grid)
   int* d_sens_cell = nullptr;
   float* d_sens_w = nullptr;
   std::vector<int> h_sens_cell;
@@ -58,6 +62,7 @@ struct pat_plan {
   double sponge_sigma_max = 0.0;
   float* d_sp_a = nullptr;
   float* d_sp_b = nullptr;
+  float *s_sp_a = nullptr, *s_sp_b = nullptr;  // at the step engines' pitch (aliases when it is nx)
   bool tma3d = false;  // 3D steps through the TMA plane-pipeline kernel
   pat::Tma3dSplit tma3d_split{0, 0};  // work split of a 3D TMA step launch
   bool tma2d = false;  // 2D steps through the TMA tile-pipeline kernel (where it applies)
@@ -65,7 +70,7 @@ struct pat_plan {
   pat::InjCell* d_tinj_step = nullptr;  // CTA (3D: 64 x 16 columns x z range); .local = linear cell index
   struct TmaDesc {
     const float* base;
-    CUtensorMap halo, own;  // stencil-input boxes with halo, own-tile boxes
+    CUtensorMap halo, own;  // stencil-input boxes with halo; 3D: own-tile boxes
   };
   std::vector<TmaDesc> tma_desc;  // descriptors by field address (small, most recent last)
 

@@ -75,7 +75,9 @@ __device__ __forceinline__ void fused_sample2(const StepArgs& a, long long bid, 
 //   forward  D' = a D + b inc (first step: D' = (a-1) P + b inc),  P' = P + D'
 //   adjoint  G' = G + inc,  Q' = a Q + b G', i.e. Z' = a Z + b kappa G'  (final step: x = G' + ((a-1)/b) Q)
 // Tiles that do not reach the layer use a = b = 1 without loading the factors.
-template <int R, int MODE, int SP>
+// FULL (grids of odd width): the forward's stencil takes the difference form and the adjoint keeps G as a
+// compensated pair too (G_lo in dbuf_lo), with the rounding of kappa G carried into Z_lo.
+template <int R, int MODE, int SP, bool FULL>
 __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
                                                              const __grid_constant__ CUtensorMap ml, int* status,
                                                              long long timeout_ns) {
@@ -87,7 +89,7 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
 
   const int t = threadIdx.x;
 
-  const int nx = a.nx, ny = a.ny;
+  const int nx = a.nx, ny = a.ny, pitch = a.pitch;
   const int tiles_x = (nx + TX - 1) / TX;
   const int ntiles = tiles_x * ((ny + TY - 1) / TY);
   const int c0 = (t % TCOLS) * 2, r0 = (t / TCOLS) * RUN;
@@ -140,14 +142,26 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
     const int tt = a.flip ? ntiles - 1 - tile : tile;
     const int gx0 = (tt % tiles_x) * TX, gy0 = (tt / tiles_x) * TY;
     const int gx = gx0 + c0;
-    // own-cell fields straight into registers, in flight while the boxes land
+    // own-cell fields straight into registers, in flight while the boxes land: D or G of every row; kappa
+    // and G_lo (fetch) two rows ahead of their use
     const float2 z2 = dup2(0.f);
-    float2 d2[RUN];
+    float2 d2[RUN], kh2[RUN], kl2[RUN], gl2[RUN];
+    const bool need_k = VARC || (ADJ && kv && !a.final_step);
+    auto fetch = [&](int rr) {
+      const int gy = gy0 + r0 + rr;
+      const long long gi = (long long)gy * pitch + gx;
+      const bool in = gy < ny && gx < nx;
+      kh2[rr] = need_k && in ? __ldg(reinterpret_cast<const float2*>(a.kappa + gi)) : z2;
+      kl2[rr] = (VARC || FULL) && need_k && in ? __ldg(reinterpret_cast<const float2*>(a.kappa_lo + gi)) : z2;
+      gl2[rr] = ADJ && FULL && in ? ld_stream2(a.dbuf_lo + gi) : z2;
+    };
 #pragma unroll
     for (int rr = 0; rr < RUN; ++rr) {
       const int gy = gy0 + r0 + rr;
-      d2[rr] = (load_d && gy < ny && gx < nx) ? ld_stream2(a.dbuf + (long long)gy * nx + gx) : z2;
+      d2[rr] = (load_d && gy < ny && gx < nx) ? ld_stream2(a.dbuf + (long long)gy * pitch + gx) : z2;
     }
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) fetch(rr);
     const bool good = mbar_wait(&bars[s], (k >> 1) & 1, timeout_ns);
     if (__syncthreads_or(!good)) {
       if (t == 0) atomicCAS(status, (int)PAT_OK, (int)PAT_ERR_TIMEOUT);
@@ -176,11 +190,9 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
         RowPairs<R> f;
         f.load(own + rr * BW, win[R]);
         const int gy = gy0 + r0 + rr;
-        const long long gi = (long long)gy * nx + gx;
+        const long long gi = (long long)gy * pitch + gx;
         const bool in = gy < ny && gx < nx;
-        const bool want_k = (VARC || (ADJ && kv && !a.final_step)) && in;
-        const float2 kh2 = want_k ? __ldg(reinterpret_cast<const float2*>(a.kappa + gi)) : z2;
-        const float2 kl2 = (VARC && in) ? __ldg(reinterpret_cast<const float2*>(a.kappa_lo + gi)) : z2;
+        if (rr + 2 < RUN) fetch(rr + 2);
         float2 sa2 = dup2(1.f), sb2 = sa2;
         if (LAYER && in) {
           sa2 = __ldg(reinterpret_cast<const float2*>(a.sp_a + gi));
@@ -188,44 +200,57 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
         }
         float2 zl2 = z2;  // adjoint: own Z_lo cells
         if (ADJ) zl2 = *reinterpret_cast<const float2*>(PL + (r0 + rr + R) * BW + XH + c0);
-        // forward: zero-sum pair form (a + b) - 2c per tap; adjoint: difference form on Z
-        const float2 st2 = stencil_pair<R, ADJ>(win, f, w2);
-        float dn[2], pn[2], pl[2];
+        // forward: zero-sum pair form (a + b) - 2c per tap; adjoint (and FULL): difference form
+        const float2 st2 = stencil_pair<R, ADJ || FULL>(win, f, w2);
+        float dn[2], pn[2], pl[2], gn[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const float c = f2get(win[R], j);  // own P or Z
           const float fa = f2get(sa2, j), fb = f2get(sb2, j);
           if (!ADJ) {
             const float acc = f2get(st2, j);
-            const float inc = VARC ? fmaf(a.c_lap * f2get(kh2, j), acc, (a.c_lap * f2get(kl2, j)) * acc)
+            const float inc = VARC ? fmaf(a.c_lap * f2get(kh2[rr], j), acc, (a.c_lap * f2get(kl2[rr], j)) * acc)
                                    : fmaf(ckh, acc, ckl * acc);
             if (!LAYER)
               dn[j] = f2get(d2[rr], j) + inc;
             else  // forward in the layer
               dn[j] = load_d ? fmaf(fa, f2get(d2[rr], j), fb * inc) : fmaf(fa - 1.f, c, fb * inc);
             pn[j] = c + dn[j];
-            pl[j] = 0.f;
+            pl[j] = gn[j] = 0.f;
           } else {
             const float acc = f2get(st2, j) + f2get(lo[rr], j);
-            const float g = f2get(d2[rr], j) + a.c_lap * acc;  // G' (S^T r injected into G beforehand)
             const float zl = f2get(zl2, j);
+            const float kap = kv ? f2get(kh2[rr], j) : a.kappa0;
+            float g, gl = 0.f;  // G' = G + L Z (S^T r injected into G beforehand)
+            if (FULL && !a.final_step)
+              g = two_sum(f2get(d2[rr], j), a.c_lap * acc + f2get(gl2[rr], j), gl);
+            else
+              g = fmaf(a.c_lap, acc, FULL ? f2get(d2[rr], j) + f2get(gl2[rr], j) : f2get(d2[rr], j));
             dn[j] = g;
+            gn[j] = gl;
             if (a.final_step) {
               pn[j] = g;
               if (LAYER) {  // x = G' + ((a-1)/b) Q,  Q = (Z + Z_lo) / kappa
-                const float kap = kv ? a.kappa[gi + j] : a.kappa0;
-                if (in && fa != 1.f) pn[j] = fmaf((fa - 1.f) / fb, (c + zl) / kap, g);
+                const float kq = kv ? a.kappa[gi + j] : a.kappa0;
+                if (in && fa != 1.f) pn[j] = fmaf((fa - 1.f) / fb, (c + zl) / kq, g);
               }
               pl[j] = 0.f;
             } else {
-              const float u = kv ? f2get(kh2, j) * g : fmaf(a.kappa0, g, a.kappa0_lo * g);  // kappa G'
+              float u, ul = 0.f;  // kappa G', and what its rounding dropped (FULL)
+              if (FULL) {
+                const float kl = kv ? f2get(kl2[rr], j) : a.kappa0_lo;
+                u = kap * g;
+                ul = fmaf(kap, g, -u) + fmaf(kap, gl, kl * g);
+              } else {
+                u = kv ? kap * g : fmaf(a.kappa0, g, a.kappa0_lo * g);
+              }
               if (LAYER && (fa != 1.f || fb != 1.f)) {  // Z' = a Z + b kappa G'
                 pn[j] = fmaf(fa, c, fb * u);
-                pl[j] = fa * zl;
+                pl[j] = FULL ? fmaf(fa, zl, fb * ul) : fa * zl;
               } else {
                 float e;
                 pn[j] = two_sum(c, u, e);
-                pl[j] = zl + e;
+                pl[j] = zl + (FULL ? e + ul : e);
               }
             }
           }
@@ -235,6 +260,7 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
           if (!a.final_step) {
             *reinterpret_cast<float2*>(a.dbuf + gi) = make_float2(dn[0], dn[1]);
             if (ADJ) *reinterpret_cast<float2*>(a.next_lo + gi) = make_float2(pl[0], pl[1]);
+            if (ADJ && FULL) *reinterpret_cast<float2*>(a.dbuf_lo + gi) = make_float2(gn[0], gn[1]);
           }
         }
 #pragma unroll
@@ -261,30 +287,25 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
     for (int j = max(0, issued - 2); j < issued; ++j) mbar_wait(&bars[j & 1], (j >> 1) & 1, timeout_ns);
 }
 
-template <int R, int MODE, int SP>
-const void* kfn() {
-  return reinterpret_cast<const void*>(&step2d_tma_kernel<R, MODE, SP>);
-}
-
-template <int R>
+template <int R, bool FULL>
 const void* kernel_r(int mode, int sp) {
   switch (mode * 3 + sp) {
-    case 0: return kfn<R, 0, 0>();
-    case 1: return kfn<R, 0, 1>();
-    case 3: return kfn<R, 1, 0>();
-    case 4: return kfn<R, 1, 1>();
-    case 6: return kfn<R, 2, 0>();
-    case 8: return kfn<R, 2, 2>();
+    case 0: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 0, 0, FULL>);
+    case 1: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 0, 1, FULL>);
+    case 3: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 1, 0, FULL>);
+    case 4: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 1, 1, FULL>);
+    case 6: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 2, 0, FULL>);
+    case 8: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 2, 2, FULL>);
     default: return nullptr;  // mismatched layer modes are not instantiated
   }
 }
 
-const void* kernel_for(int R, int mode, int sp) {
+const void* kernel_for(int R, int mode, int sp, bool full) {
   switch (R) {
-    case 1: return kernel_r<1>(mode, sp);
-    case 3: return kernel_r<3>(mode, sp);
-    case 5: return kernel_r<5>(mode, sp);
-    case 7: return kernel_r<7>(mode, sp);
+    case 1: return full ? kernel_r<1, true>(mode, sp) : kernel_r<1, false>(mode, sp);
+    case 3: return full ? kernel_r<3, true>(mode, sp) : kernel_r<3, false>(mode, sp);
+    case 5: return full ? kernel_r<5, true>(mode, sp) : kernel_r<5, false>(mode, sp);
+    case 7: return full ? kernel_r<7, true>(mode, sp) : kernel_r<7, false>(mode, sp);
     default: return nullptr;
   }
 }
@@ -298,34 +319,28 @@ size_t smem_for(int R, int mode) {
 
 int tma2d_tile() { return TX; }
 
-bool tma2d_supported(int nx, int R) { return nx % 4 == 0 && (R == 1 || R == 3 || R == 5 || R == 7); }
+bool tma2d_supported(int R) { return R == 1 || R == 3 || R == 5 || R == 7; }
 
-// Descriptors of a 2D field: P boxes (80 x (64+2R)) and own-tile boxes (64 x 64, kept for
-// kernels that stage own cells through shared memory).
-cudaError_t tma2d_encode(const float* base, int nx, int ny, int R, CUtensorMap* halo, CUtensorMap* own) {
+cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CUtensorMap* halo) {
   auto fn = tma_encoder();
   if (!fn) return cudaErrorNotSupported;
   const cuuint64_t dims[2] = {(cuuint64_t)nx, (cuuint64_t)ny};
-  const cuuint64_t strides[1] = {(cuuint64_t)nx * 4};
+  const cuuint64_t strides[1] = {(cuuint64_t)pitch * 4};
   const cuuint32_t estr[2] = {1, 1};
   const cuuint32_t box_h[2] = {(cuuint32_t)BW, (cuuint32_t)(TY + 2 * R)};
-  const cuuint32_t box_o[2] = {(cuuint32_t)TX, (cuuint32_t)TY};
-  CUresult r1 = fn(halo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box_h, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  CUresult r2 = fn(own, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box_o, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return (r1 == CUDA_SUCCESS && r2 == CUDA_SUCCESS) ? cudaSuccess : cudaErrorInvalidValue;
+  const CUresult r = fn(halo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box_h, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // Persistent grid: as many CTAs as fit on the device, at most one per tile.
-int tma2d_ctas(int nx, int ny, int R, int mode, int sp) {
-  static int cached[3][3][8] = {{{0}}};
-  int& c = cached[mode][sp][R];
+int tma2d_ctas(int nx, int ny, int R, int mode, int sp, bool full) {
+  static int cached[2][3][3][8] = {{{{0}}}};
+  int& c = cached[full][mode][sp][R];
   if (!c) {
     int dev = 0, sms = 148, per = 1;
-    const void* fn = kernel_for(R, mode, sp);
+    const void* fn = kernel_for(R, mode, sp, full);
     const size_t smem = smem_for(R, mode);
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -339,15 +354,15 @@ int tma2d_ctas(int nx, int ny, int R, int mode, int sp) {
   return ntiles < c ? ntiles : c;
 }
 
-long long tma2d_threads(int nx, int ny, int R, int mode, int sp) {
-  return (long long)tma2d_ctas(nx, ny, R, mode, sp) * THREADS;
+long long tma2d_threads(int nx, int ny, int R, int mode, int sp, bool full) {
+  return (long long)tma2d_ctas(nx, ny, R, mode, sp, full) * THREADS;
 }
 
-cudaError_t step2d_tma_launch(int R, int mode, int sp, const StepArgs& a, const CUtensorMap& p, const CUtensorMap& lo,
-                              int* status, long long timeout_ns, cudaStream_t st) {
-  const void* fn = kernel_for(R, mode, sp);
+cudaError_t step2d_tma_launch(int R, int mode, int sp, bool full, const StepArgs& a, const CUtensorMap& p,
+                              const CUtensorMap& lo, int* status, long long timeout_ns, cudaStream_t st) {
+  const void* fn = kernel_for(R, mode, sp, full);
   if (!fn) return cudaErrorInvalidValue;
-  const int nctas = tma2d_ctas(a.nx, a.ny, R, mode, sp);  // sets the kernel's attributes once
+  const int nctas = tma2d_ctas(a.nx, a.ny, R, mode, sp, full);  // sets the kernel's attributes once
   CUtensorMap map = p, mapl = lo;
   StepArgs args = a;
   void* params[] = {&args, &map, &mapl, &status, &timeout_ns};

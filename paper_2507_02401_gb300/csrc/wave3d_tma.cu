@@ -1,11 +1,14 @@
-// 3D wave step with TMA-fed plane pipelines (constant medium, the HBM-bound
-// volumes): one launch per time step of the three-level recurrence
+// 3D wave step with TMA-fed plane pipelines (the HBM-bound volumes): one
+// launch per time step of the three-level recurrence
 //
 //   next = c_cur cur - c_prev prev + c_lap (kappa_hi + kappa_lo) L cur
 //
 // (paper Sec. 2, Eq. wave_equation; forward P^{n+1} = 2P^n - P^{n-1} +
-// kappa L P^n and, because kappa is constant, the adjoint
-// Q^n = 2Q^{n+1} - Q^{n+2} + kappa L Q^{n+1} have the same form).
+// kappa L P^n).  The adjoint Q^n = 2Q^{n+1} - Q^{n+2} + L(kappa Q^{n+1}) has
+// this form for a constant kappa, and for a varying one in Z = kappa Q:
+// Z^n = 2Z^{n+1} - Z^{n+2} + kappa (L Z^{n+1} + S^T r_n); its final step,
+// x = (Z^1 - Z^2) / kappa + 1/2 L Z^1 + S^T r_0, leaves that variable.  So a
+// varying medium adds only the reads of the own cells' kappa (hi and lo).
 //
 // A CTA owns a 64 x 16 column of cells and marches through a range of z
 // planes.  One thread issues TMA loads of each plane of `cur` as an
@@ -79,7 +82,8 @@ __device__ __forceinline__ float inj_sum(const StepArgs& a, const InjCell& c) {
 // INJ: the adjoint's injection S^T r_m into the CTA's own cells of `next` after the step (per-CTA lists)
 // Work split (column-fastest): CTA b takes column b mod columns and the (b div columns)-th of
 // nchunks equal z ranges, so CTAs that run together stream neighbouring columns of the same rows.
-template <int R, bool INJ, bool RING>
+// VARC: varying medium (a.final_step: the adjoint's last step)
+template <int R, bool INJ, bool RING, bool VARC>
 __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mcur,
                                                              const __grid_constant__ CUtensorMap mprev, int cols_x,
                                                              int nchunks, int* status, long long timeout_ns) {
@@ -95,12 +99,14 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   const long long bid = blockIdx.x;
 
   const int nx = a.nx, ny = a.ny, nz = a.nz;
-  const long long plane = (long long)nx * ny;
+  const int pitch = a.pitch;
+  const long long plane = (long long)pitch * ny;
   const int c0 = (t % (TX / 4)) * 4, r0 = (t / (TX / 4)) * 2;
   const long long ncols = (long long)cols_x * ((ny + TY - 1) / TY);
   const bool has_prev = a.prev != nullptr;
   const float ck = a.c_lap * a.kappa0, ckl = a.c_lap * a.kappa0_lo;
-  const float2 ck2 = dup2(ck), ckl2 = dup2(ckl), ccur2 = dup2(a.c_cur), ncprev2 = dup2(-a.c_prev), m2 = dup2(-2.f);
+  const float2 ck2 = dup2(ck), ckl2 = dup2(ckl), ccur2 = dup2(a.c_cur), ncprev2 = dup2(-a.c_prev), m2 = dup2(-2.f),
+               clap2 = dup2(a.c_lap);
   float2 w2[R + 1];
 #pragma unroll
   for (int m = 0; m <= R; ++m) w2[m] = dup2(a.w[m]);
@@ -174,9 +180,24 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
     for (int rr = 0; rr < 2; ++rr) {
       const int z = zb + (i - R) * zd, gy = gy0 + r0 + rr, gx = gx0 + c0;
       q[i][rr] = (z >= 0 && z < nz && gy < ny && gx < nx)
-                     ? __ldg(reinterpret_cast<const float4*>(a.cur + z * plane + (long long)gy * nx + gx))
+                     ? __ldg(reinterpret_cast<const float4*>(a.cur + z * plane + (long long)gy * pitch + gx))
                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+  // varying medium: the own cells' kappa, one plane ahead of its use
+  float4 kh[2], kl[2];
+  auto fetch_kappa = [&](int i) {
+#pragma unroll
+    for (int rr = 0; rr < 2; ++rr) {
+      const int gy = gy0 + r0 + rr, gx = gx0 + c0;
+      kh[rr] = kl[rr] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < nloc && gy < ny && gx < nx) {
+        const long long gi = (zb + i * zd) * plane + (long long)gy * pitch + gx;
+        kh[rr] = ld_stream4(a.kappa + gi);
+        kl[rr] = ld_stream4(a.kappa_lo + gi);
+      }
+    }
+  };
+  if (VARC) fetch_kappa(0);
   bool ok = true;
 #pragma unroll
   for (int i = 0; i < R; ++i) {  // planes zb .. zb + (R-1) zd from the ring
@@ -235,13 +256,22 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
         // c_cur c - c_prev prev + (ck + ckl) acc, the last product rounded once
         float2 v = __fmul2_rn(ccur2, c);
         if (has_prev) v = __ffma2_rn(ncprev2, p ? hi2(pv) : lo2(pv), v);
-        out[p] = __fadd2_rn(v, __ffma2_rn(ck2, acc, __fmul2_rn(ckl2, acc)));
+        if (!VARC) {
+          out[p] = __fadd2_rn(v, __ffma2_rn(ck2, acc, __fmul2_rn(ckl2, acc)));
+        } else {
+          const float2 h = p ? hi2(kh[rr]) : lo2(kh[rr]), l = p ? hi2(kl[rr]) : lo2(kl[rr]);
+          if (a.final_step)
+            out[p] = make_float2(v.x / h.x + a.c_lap * acc.x, v.y / h.y + a.c_lap * acc.y);
+          else
+            out[p] = __fadd2_rn(v, __ffma2_rn(__fmul2_rn(clap2, h), acc, __fmul2_rn(__fmul2_rn(clap2, l), acc)));
+        }
       }
       const int gy = gy0 + r0 + rr, gx = gx0 + c0;
       if (gy < ny && gx < nx)
-        *reinterpret_cast<float4*>(a.next + z * plane + (long long)gy * nx + gx) =
+        *reinterpret_cast<float4*>(a.next + z * plane + (long long)gy * pitch + gx) =
             make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
     }
+    if (VARC) fetch_kappa(i + 1);
     return true;
   };
   if constexpr (RING) {
@@ -266,13 +296,15 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   if (INJ && ok_all) {  // every thread's stores to `next` precede the injection (same CTA)
     __syncthreads();
     for (int i = nloc; i < 4; ++i) inj_prefetch(i);  // short marches
+    auto scale = [&](const InjCell& c) { return VARC && !a.final_step ? a.kappa[c.local] : 1.f; };
     if (ie0 < ie1) {
       float v = ic.beg < ic.end ? iw * ir : 0.f;
       for (int q = ic.beg + 1; q < ic.end; ++q)
         v = fmaf(a.ent_w[q], a.inj_r[(long long)a.ent_sensor[q] * a.nt + a.inj_t], v);
-      a.next[ic.local] += v;
+      a.next[ic.local] += scale(ic) * v;
     }
-    for (int e = ie0 + THREADS; e < ie1; e += THREADS) a.next[a.inj_tile[e].local] += inj_sum(a, a.inj_tile[e]);
+    for (int e = ie0 + THREADS; e < ie1; e += THREADS)
+      a.next[a.inj_tile[e].local] += scale(a.inj_tile[e]) * inj_sum(a, a.inj_tile[e]);
   }
   // after a timed-out wait: give the copies still in flight (the last one of
   // each slot) a bounded chance to land before the CTA's shared memory goes away
@@ -283,63 +315,51 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   }
 }
 
-template <int R, bool INJ, bool RING>
-cudaError_t prepare_r() {
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(step3d_tma_kernel<R, INJ, RING>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)G3<R>::SMEM);
-  });
-  return attr_err;
-}
+using KernelFn = void (*)(const StepArgs, const CUtensorMap, const CUtensorMap, int, int, int*, long long);
 
-template <int R, bool INJ, bool RING>
-cudaError_t launch_r(const StepArgs& a, const CUtensorMap& mc, const CUtensorMap& mp, int nctas, int nchunks,
-                     int* status, long long timeout_ns, cudaStream_t st) {
-  const cudaError_t attr_err = prepare_r<R, INJ, RING>();
-  if (attr_err != cudaSuccess) return attr_err;
-  return launch_pdl(step3d_tma_kernel<R, INJ, RING>, nctas, THREADS, (int)G3<R>::SMEM, st, a, mc, mp,
-                    (a.nx + TX - 1) / TX, nchunks, status, timeout_ns);
-}
-
-template <int R, bool INJ, bool RING>
-int blocks_per_sm() {
-  int per = 0;
-  if (prepare_r<R, INJ, RING>() != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step3d_tma_kernel<R, INJ, RING>, THREADS, G3<R>::SMEM) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return 0;
+// The register ring is built for R <= 3 only (tma3d_split).
+template <int R, bool VARC>
+KernelFn kernel_rv(bool inj, bool ring) {
+  if constexpr (R <= 3) {
+    if (ring) return inj ? step3d_tma_kernel<R, true, true, VARC> : step3d_tma_kernel<R, false, true, VARC>;
   }
-  return per;
+  return inj ? step3d_tma_kernel<R, true, false, VARC> : step3d_tma_kernel<R, false, false, VARC>;
 }
 
-// Co-resident CTAs of the step kernel (every variant) on the current device.
-template <int R>
-int resident_r() {
-  int dev = 0, sms = 0;
+KernelFn kernel_for(int R, bool inj, bool ring, bool varc) {
+  switch (R) {
+    case 1: return varc ? kernel_rv<1, true>(inj, ring) : kernel_rv<1, false>(inj, ring);
+    case 3: return varc ? kernel_rv<3, true>(inj, ring) : kernel_rv<3, false>(inj, ring);
+    case 5: return varc ? kernel_rv<5, true>(inj, ring) : kernel_rv<5, false>(inj, ring);
+    case 7: return varc ? kernel_rv<7, true>(inj, ring) : kernel_rv<7, false>(inj, ring);
+    default: return nullptr;
+  }
+}
+
+int smem_for(int R) {
+  return (int)(R == 1 ? G3<1>::SMEM : R == 3 ? G3<3>::SMEM : R == 5 ? G3<5>::SMEM : G3<7>::SMEM);
+}
+
+// Co-resident CTAs of the step kernel (with and without injection and ring) on the current device; sets the
+// kernels' shared-memory attribute.
+int resident(int R, bool varc) {
+  int dev = 0, sms = 0, best = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  const int v[4] = {blocks_per_sm<R, false, false>(), blocks_per_sm<R, true, false>(), blocks_per_sm<R, false, true>(),
-                    blocks_per_sm<R, true, true>()};
-  int per = v[0];
-  for (int i = 1; i < 4; ++i) per = v[i] < per ? v[i] : per;
-  return sms * per;
-}
-
-template <bool INJ, bool RING>
-cudaError_t launch_i(int R, const StepArgs& a, const CUtensorMap& cur, const CUtensorMap& prev, int nctas,
-                     int nchunks, int* status, long long timeout_ns, cudaStream_t st) {
-  switch (R) {
-    case 1: return launch_r<1, INJ, RING>(a, cur, prev, nctas, nchunks, status, timeout_ns, st);
-    case 3: return launch_r<3, INJ, RING>(a, cur, prev, nctas, nchunks, status, timeout_ns, st);
-    case 5: return launch_r<5, INJ, RING>(a, cur, prev, nctas, nchunks, status, timeout_ns, st);
-    case 7: return launch_r<7, INJ, RING>(a, cur, prev, nctas, nchunks, status, timeout_ns, st);
-    default: return cudaErrorInvalidValue;
+  for (int v = 0; v < 4; ++v) {
+    const KernelFn fn = kernel_for(R, v & 1, v & 2, varc);
+    int per = 0;
+    if (!fn ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_for(R)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, THREADS, smem_for(R)) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    best = v == 0 || per < best ? per : best;
   }
+  return sms * best;
 }
 
 }  // namespace
@@ -362,14 +382,14 @@ void* tma_encoder_raw() {
 }
 
 
-bool tma3d_supported(int nx, int R, bool varc) { return !varc && nx % 4 == 0 && (R == 1 || R == 3 || R == 5 || R == 7); }
+bool tma3d_supported(int R) { return R == 1 || R == 3 || R == 5 || R == 7; }
 
-// Descriptors of a 3D field: `cur` boxes (80 x (16+2R) x 1) and `prev` boxes (64 x 16 x 1).
-cudaError_t tma3d_encode(const float* base, int nx, int ny, int nz, int R, CUtensorMap* cur, CUtensorMap* prev) {
+cudaError_t tma3d_encode(const float* base, int nx, int pitch, int ny, int nz, int R, CUtensorMap* cur,
+                         CUtensorMap* prev) {
   auto fn = tma_encoder();
   if (!fn) return cudaErrorNotSupported;
   const cuuint64_t dims[3] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz};
-  const cuuint64_t strides[2] = {(cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4};
+  const cuuint64_t strides[2] = {(cuuint64_t)pitch * 4, (cuuint64_t)pitch * ny * 4};
   const cuuint32_t estr[3] = {1, 1, 1};
   const cuuint32_t box_c[3] = {(cuuint32_t)(TX + (R <= 4 ? 8 : 16)), (cuuint32_t)(TY + 2 * R), 1};
   const cuuint32_t box_p[3] = {(cuuint32_t)TX, (cuuint32_t)TY, 1};
@@ -389,16 +409,9 @@ cudaError_t tma3d_encode(const float* base, int nx, int ny, int nz, int R, CUten
 // >= 6 CTAs per SM.  Measured at 256^3: 41.0 / 40.0 us per K / K* step against 41.4 / 44.1 us with
 // 16-plane ranges in 1024 CTAs (and 43.1 / 42.3 us with equal z-fastest shares of the (column, plane)
 // work, whose concurrent CTAs no longer share x/y halos through L2).
-Tma3dSplit tma3d_split(int R, int nx, int ny, int nz) {
-  int cap = 0;
-  switch (R) {
-    case 1: cap = resident_r<1>(); break;
-    case 3: cap = resident_r<3>(); break;
-    case 5: cap = resident_r<5>(); break;
-    case 7: cap = resident_r<7>(); break;
-    default: return Tma3dSplit{0, 0};
-  }
-  if (cap <= 0) return Tma3dSplit{0, 0};
+Tma3dSplit tma3d_split(int R, bool varc, int nx, int ny, int nz) {
+  const int cap = resident(R, varc);
+  if (cap <= 0) return Tma3dSplit{0, 0, false};
   const long long cols = (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
   int chunks;
   if (cols * 4 < cap) {
@@ -432,11 +445,10 @@ long long tma3d_threads(int nctas) { return (long long)nctas * THREADS; }
 
 cudaError_t step3d_tma_launch(int R, const StepArgs& a, const CUtensorMap& cur, const CUtensorMap& prev,
                               const Tma3dSplit& sp, int* status, long long timeout_ns, cudaStream_t st) {
-  if (sp.ring)
-    return a.inj_r ? launch_i<true, true>(R, a, cur, prev, sp.nctas, sp.nchunks, status, timeout_ns, st)
-                   : launch_i<false, true>(R, a, cur, prev, sp.nctas, sp.nchunks, status, timeout_ns, st);
-  return a.inj_r ? launch_i<true, false>(R, a, cur, prev, sp.nctas, sp.nchunks, status, timeout_ns, st)
-                 : launch_i<false, false>(R, a, cur, prev, sp.nctas, sp.nchunks, status, timeout_ns, st);
+  const KernelFn fn = kernel_for(R, a.inj_r != nullptr, sp.ring, a.kappa != nullptr);
+  if (!fn) return cudaErrorInvalidValue;
+  return launch_pdl(fn, sp.nctas, THREADS, smem_for(R), st, a, cur, prev, (a.nx + TX - 1) / TX, sp.nchunks, status,
+                    timeout_ns);
 }
 
 }  // namespace pat

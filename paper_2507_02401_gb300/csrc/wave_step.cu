@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(S2_THREADS) step2d_kernel(const StepArgs a) {
   auto stage = [&](int gx, int gy, int sidx) {
     float hi = 0.f, lo = 0.f;
     if (gx >= 0 && gy >= 0 && gx < nx && gy < ny) {
-      const long long gi = (long long)gy * nx + gx;
+      const long long gi = (long long)gy * a.pitch + gx;
       const float q = a.cur[gi];
       if (ADJ) {
         const float k = VARC ? a.kappa[gi] : a.kappa0;
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(S2_THREADS) step2d_kernel(const StepArgs a) {
     for (int j = 0; j < 4; ++j) {
       const int gx = gx0 + c0 + j, gy = gy0 + r0 + rr;
       if (gx >= nx || gy >= ny) continue;
-      const long long gi = (long long)gy * nx + gx;
+      const long long gi = (long long)gy * a.pitch + gx;
       // absorbing layer: factors a, b of the damped update (1 outside the layer)
       const float fa = a.sp_a ? a.sp_a[gi] : 1.f, fb = a.sp_a ? a.sp_b[gi] : 1.f;
       const bool layer = fa != 1.f || fb != 1.f;
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(S3_THREADS) step3d_kernel(const StepArgs a) {
   fused_sample(a, bid * S3_THREADS + t);
 
   const int nx = a.nx, ny = a.ny, nz = a.nz;
-  const long long plane = (long long)nx * ny;
+  const long long plane = (long long)a.pitch * ny;
   const int tx = t % (S3_TX / 4), ty = t / (S3_TX / 4);
   const int gx0 = blockIdx.x * S3_TX, gy0 = blockIdx.y * S3_TY;
   const int gx = gx0 + tx * 4, gy = gy0 + ty;
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(S3_THREADS) step3d_kernel(const StepArgs a) {
       const int x = gx + j;
       float val = 0.f;
       if (row_ok && x < nx && z >= 0 && z < nz) {
-        const long long gi = (long long)z * plane + (long long)gy * nx + x;
+        const long long gi = (long long)z * plane + (long long)gy * a.pitch + x;
         val = a.cur[gi];
         if (ADJ && VARC) val *= a.kappa[gi];
       }
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(S3_THREADS) step3d_kernel(const StepArgs a) {
   };
   auto fetch = [&](int x, int y, int z) -> float {
     if (x < 0 || y < 0 || x >= nx || y >= ny) return 0.f;
-    const long long gi = (long long)z * plane + (long long)y * nx + x;
+    const long long gi = (long long)z * plane + (long long)y * a.pitch + x;
     float v = a.cur[gi];
     if (ADJ && VARC) v *= a.kappa[gi];
     return v;
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(S3_THREADS) step3d_kernel(const StepArgs a) {
       for (int j = 0; j < 4; ++j) {
         const int x = gx + j;
         if (x >= nx) continue;
-        const long long gi = (long long)z * plane + (long long)gy * nx + x;
+        const long long gi = (long long)z * plane + (long long)gy * a.pitch + x;
         const float cur = (ADJ && VARC) ? a.cur[gi] : q[R][j];
         // kappa as hi + lo (a coherent rounding of a constant kappa would drift the phase)
         const float kap = ADJ ? (VARC ? 1.f : a.kappa0) : (VARC ? a.kappa[gi] : a.kappa0);
@@ -251,16 +251,17 @@ __global__ void sample_kernel(const float* __restrict__ P, int ns, int nt, int t
   y[(long long)s * nt + tsamp] = v;
 }
 
-// Q[cell] += scale * sum_e w_e r[sensor_e, t] over each injected cell's entries
+// Q[cell] += scale[cell] * sum_e w_e r[sensor_e, t] over each injected cell's entries
 __global__ void inject_kernel(float* __restrict__ Q, int n_inj, const int* __restrict__ inj_cell,
                               const int* __restrict__ inj_ptr, const int* __restrict__ ent_sensor,
                               const float* __restrict__ ent_w, const float* __restrict__ r, int nt, int tt,
-                              float scale) {
+                              const float* __restrict__ cell_scale) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_inj) return;
   float s = 0.f;
   for (int e = inj_ptr[i]; e < inj_ptr[i + 1]; ++e) s = fmaf(ent_w[e], r[(long long)ent_sensor[e] * nt + tt], s);
-  Q[inj_cell[i]] += scale * s;
+  const int c = inj_cell[i];
+  Q[c] += cell_scale ? cell_scale[c] * s : s;
 }
 
 __global__ void fill_kernel(float* p, long long n, float v) {
@@ -271,6 +272,16 @@ __global__ void fill_kernel(float* p, long long n, float v) {
 __global__ void copy_kernel(float* __restrict__ d, const float* __restrict__ s, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     d[i] = s[i];
+}
+
+__global__ void pitch_copy_kernel(float* __restrict__ d, int dpitch, const float* __restrict__ s, int spitch, int nx,
+                                  long long rows) {
+  const long long n = rows * nx;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long r = i / nx;
+    const int c = (int)(i - r * nx);
+    d[r * dpitch + c] = s[r * spitch + c];
+  }
 }
 
 template <bool ADJ, bool VARC>
@@ -333,15 +344,21 @@ cudaError_t sample_launch(const float* P, int ns, int nt, int t, const int* cell
 }
 
 cudaError_t inject_launch(float* Q, int n_inj, const int* inj_cell, const int* inj_ptr, const int* ent_sensor,
-                          const float* ent_w, const float* r, int nt, int t, float scale, cudaStream_t st) {
+                          const float* ent_w, const float* r, int nt, int t, const float* cell_scale, cudaStream_t st) {
   if (n_inj <= 0) return cudaSuccess;
-  inject_kernel<<<(n_inj + 127) / 128, 128, 0, st>>>(Q, n_inj, inj_cell, inj_ptr, ent_sensor, ent_w, r, nt, t, scale);
+  inject_kernel<<<(n_inj + 127) / 128, 128, 0, st>>>(Q, n_inj, inj_cell, inj_ptr, ent_sensor, ent_w, r, nt, t, cell_scale);
   return cudaGetLastError();
 }
 
 cudaError_t fill_launch(float* p, long long n, float v, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   fill_kernel<<<grid_for(n), 256, 0, st>>>(p, n, v);
+  return cudaGetLastError();
+}
+
+cudaError_t pitch_copy_launch(float* d, int dpitch, const float* s, int spitch, int nx, long long rows,
+                              cudaStream_t st) {
+  pitch_copy_kernel<<<grid_for(rows * nx), 256, 0, st>>>(d, dpitch, s, spitch, nx, rows);
   return cudaGetLastError();
 }
 
@@ -364,21 +381,23 @@ __global__ void grad_acc_kernel(double* __restrict__ gacc, const float* __restri
                                 const float* __restrict__ P, float coef, int nx, int ny, int nz, int dim, int zform,
                                 const StepArgs a) {
   const long long N = (long long)nx * ny * nz;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(i % nx);
-    const int y = (int)((i / nx) % ny);
-    const int z = (int)(i / ((long long)nx * ny));
+  const int pitch = a.pitch;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (long long)gridDim.x * blockDim.x) {
+    const int x = (int)(k % nx);
+    const int y = (int)((k / nx) % ny);
+    const int z = (int)(k / ((long long)nx * ny));
+    const long long i = ((long long)z * ny + y) * pitch + x;  // gacc is dense, the fields are pitched
     const float c = P[i];
     float acc = 0.f;
 #pragma unroll
     for (int m = 1; m <= R; ++m) {
       const float xp = (x + m < nx) ? P[i + m] : 0.f;
       const float xm = (x - m >= 0) ? P[i - m] : 0.f;
-      const float yp = (y + m < ny) ? P[i + (long long)m * nx] : 0.f;
-      const float ym = (y - m >= 0) ? P[i - (long long)m * nx] : 0.f;
+      const float yp = (y + m < ny) ? P[i + (long long)m * pitch] : 0.f;
+      const float ym = (y - m >= 0) ? P[i - (long long)m * pitch] : 0.f;
       float t = ((xp - c) + (xm - c)) + ((yp - c) + (ym - c));
       if (dim == 3) {
-        const long long pl = (long long)nx * ny;
+        const long long pl = (long long)pitch * ny;
         const float zp = (z + m < nz) ? P[i + m * pl] : 0.f;
         const float zm = (z - m >= 0) ? P[i - m * pl] : 0.f;
         t += (zp - c) + (zm - c);
@@ -388,7 +407,7 @@ __global__ void grad_acc_kernel(double* __restrict__ gacc, const float* __restri
     double q = (double)Q[i] + (Qlo ? (double)Qlo[i] : 0.0);
     if (zform)  // the state holds Z = kappa Q
       q /= a.kappa ? (double)a.kappa[i] + (double)a.kappa_lo[i] : (double)a.kappa0 + (double)a.kappa0_lo;
-    gacc[i] += (double)coef * q * (double)acc;
+    gacc[k] += (double)coef * q * (double)acc;
   }
 }
 
