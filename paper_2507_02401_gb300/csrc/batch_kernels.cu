@@ -36,15 +36,15 @@ namespace {
 
 constexpr int TX = 64, XH = 8, BW = TX + 2 * XH;
 
-// rows per thread: 8 for the forward; 4 for the adjoint, whose two stencils and two staged boxes
-// per tile need more registers and shared memory per cell (twice the threads per tile keep the
-// resident warps per SM up)
-constexpr int run_rows(bool adj) { return adj ? 4 : 8; }
+// Each thread owns 4 columns x 4 rows, as in the single-instance kernel: a 64-row tile is a CTA of 256
+// threads, a 32-row tile one of 128.  CTAs per SM to leave registers for with 32-row tiles: four, three in the
+// adjoint above order 4 (32 uneven instances, order 8, K us per step: 10.2 with four forward CTAs, 10.9 with three).
+constexpr int min_ctas(int R, int TY, bool adj) { return TY == 64 ? 1 : R > 3 && adj ? 3 : 4; }
+constexpr int NP = 2, RUN = 4, TCOLS = TX / (2 * NP);
 
 template <int R, int TY, bool ADJ>
 struct GB {
-  static constexpr int RUN = run_rows(ADJ);
-  static constexpr int THREADS = (TX / 4) * (TY / RUN);
+  static constexpr int THREADS = TCOLS * (TY / RUN);
   static constexpr int PBOX = BW * (TY + 2 * R);  // floats (multiple of 32: 128-byte aligned stages)
   static constexpr int STAGE = (ADJ ? 2 : 1) * PBOX;
   static constexpr size_t SMEM = sizeof(float) * 2 * STAGE + 16;
@@ -81,18 +81,22 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned round, int*
 }
 
 template <int R, int TY, bool ADJ, bool RUNALL>
-__global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS) batch_step_kernel(const BatchStepArgs a) {
+__global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS, min_ctas(R, TY, ADJ)) batch_step_kernel(const BatchStepArgs a) {
   using G = GB<R, TY, ADJ>;
-  constexpr int THREADS = G::THREADS, RUN = G::RUN;
+  constexpr int THREADS = G::THREADS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* stage0 = reinterpret_cast<float*>(smem_raw);
   uint64_t* bars = reinterpret_cast<uint64_t*>(stage0 + 2 * G::STAGE);
 
   const int t = threadIdx.x;
-  const int c0 = (t % (TX / 4)) * 4, r0 = (t / (TX / 4)) * RUN;
+  const int c0 = (t % TCOLS) * 2 * NP, r0 = (t / TCOLS) * RUN;
   float2 w2[R + 1];  // stencil weights, packed
 #pragma unroll
   for (int m = 0; m <= R; ++m) w2[m] = dup2(a.w[m]);
+  float wc = 0.f;  // centre weight of the Z_lo stencil (sum form)
+#pragma unroll
+  for (int m = 1; m <= R; ++m) wc += a.w[m];
+  const float2 nwc = dup2(-(wc * 4.f));
 
   if (t == 0) {
     mbar_init(&bars[0], 1);
@@ -100,6 +104,8 @@ __global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS) batch_step_kernel(con
     fence_mbar_init();
   }
   __syncthreads();
+  griddep_wait();  // one launch per step: everything above overlaps the previous step's last CTAs
+  griddep_trigger();
 
   int k = 0, issued = 0;  // tiles processed (stage k & 1, phase (k >> 1) & 1) and TMA pairs issued, over all steps
   bool ok = true;
@@ -161,13 +167,23 @@ __global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS) batch_step_kernel(con
     float* out = final_step ? const_cast<float*>(I.img) : I.P[(step + 1) & 1];
 
     const bool load_d = !(!ADJ && n == 0);
-    float4 d4[RUN];
+    Cells<NP> d2[RUN];
     auto load_own_d = [&]() {
 #pragma unroll
       for (int rr = 0; rr < RUN; ++rr) {
         const int gy = gy0 + r0 + rr;
         const bool in = compute && load_d && gy < ny && gx < nx;
-        d4[rr] = in ? ld_stream4(I.D + (long long)gy * nx + gx) : make_float4(0.f, 0.f, 0.f, 0.f);
+        d2[rr].fill(0.f);
+        if (in) d2[rr].stream(I.D + (long long)gy * nx + gx);
+      }
+    };
+    // G += S^T r_m on the tile's own cells
+    auto inject = [&](int m) {
+      for (int e = dc.e0 + t; e < dc.e1; e += THREADS) {
+        const InjCell c = I.inj[e];
+        float v = 0.f;
+        for (int q = c.beg; q < c.end; ++q) v = fmaf(I.ent_w[q], I.y[(long long)I.ent_sensor[q] * nt + m], v);
+        I.D[c.local] += v;
       }
     };
     if (!ADJ) {  // y[s, n] = sum_k w_k P^n[cell_k] for the sensors based in this tile
@@ -179,18 +195,26 @@ __global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS) batch_step_kernel(con
           v = fmaf(I.sens_w[sn * I.corners + q], cur[I.sens_cell[sn * I.corners + q]], v);
         I.y[(long long)sn * nt + n] = v;
       }
-    } else {  // G += S^T r_m on the tile's own cells
-      if (dc.e1 > dc.e0) {  // uniform over the CTA
-        for (int e = dc.e0 + t; e < dc.e1; e += THREADS) {
-          const InjCell c = I.inj[e];
-          float v = 0.f;
-          for (int q = c.beg; q < c.end; ++q) v = fmaf(I.ent_w[q], I.y[(long long)I.ent_sensor[q] * nt + n], v);
-          I.D[c.local] += v;
-        }
+    } else {
+      if (step == 0 && dc.e1 > dc.e0) {  // the later steps' injections are left by the step before (below)
+        inject(n);
         __syncthreads();  // the injected cells are read below by other threads of the CTA
       }
       load_own_d();
     }
+    const bool varying = I.kappa != nullptr;  // uniform over the tile (one instance)
+    Cells<NP> kh2[RUN], kl2[RUN];                // a varying medium's kappa (forward: hi and lo), two rows ahead
+    auto fetch = [&](int rr) {
+      const int gy = gy0 + r0 + rr;
+      const bool in = varying && gy < ny && gx < nx;
+      const long long gi = (long long)gy * nx + gx;
+      kh2[rr].fill(0.f);
+      kl2[rr].fill(0.f);
+      if (in) kh2[rr].ldg(I.kappa + gi);
+      if (!ADJ && in) kl2[rr].ldg(I.kappa_lo + gi);
+    };
+    fetch(0);
+    fetch(1);
 
     const bool good = mbar_wait(&bars[s], (k >> 1) & 1, a.timeout_ns);
     if (__syncthreads_or(!good)) {
@@ -202,59 +226,56 @@ __global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS) batch_step_kernel(con
       const float* P = stage0 + s * G::STAGE;  // P (forward) or Z (adjoint)
       const float* PL = P + G::PBOX;           // adjoint: Z_lo
       const float c_lap = (n == 0 || final_step) ? 0.5f : 1.f;
-      const float ckh = c_lap * I.kappa0, ckl = c_lap * I.kappa0_lo;
-      const bool varying = I.kappa != nullptr;  // uniform over the tile (one instance)
-      float lo[RUN][4];  // adjoint: the Z_lo part of the stencil, first pass
-      if (ADJ) stencil_run<R, RUN, BW, XH>(PL, r0, c0, a.w, lo);
-      float4 win[2 * R + 1];
+      const float k0h = I.kappa0, k0l = I.kappa0_lo, ckh = c_lap * k0h, ckl = c_lap * k0l;
+      float* const D = I.D;
+      float* const out_lo = I.P_lo[(step + 1) & 1];
+      Cells<NP> lo[RUN];  // adjoint: the Z_lo part of the stencil, first pass
+      if (ADJ) stencil_run_pair<R, RUN, BW>(PL + (r0 + R) * BW + XH + c0, w2, nwc, lo);
+      const float* own = P + (r0 + R) * BW + XH + c0;
+      Cells<NP> win[2 * R + 1];
 #pragma unroll
-      for (int i = 0; i < 2 * R; ++i) win[i] = *reinterpret_cast<const float4*>(P + (r0 + i) * BW + XH + c0);
+      for (int i = 0; i < 2 * R; ++i) win[i].load(own + (i - R) * BW);
 #pragma unroll
       for (int rr = 0; rr < RUN; ++rr) {
-        win[2 * R] = *reinterpret_cast<const float4*>(P + (r0 + rr + 2 * R) * BW + XH + c0);
-        const int brow = r0 + rr + R;
-        float f[20];
-        load_row20(P + brow * BW + c0, f);
-        float4 zl4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ADJ) zl4 = *reinterpret_cast<const float4*>(PL + brow * BW + XH + c0);
-        // a varying medium's kappa (forward: hi and lo parts) for this row, in flight during the stencil
+        win[2 * R].load(own + (rr + R) * BW);
+        Row<R, NP> f;
+        f.load(own + rr * BW, win[R]);
+        if (rr + 2 < RUN) fetch(rr + 2);
+        Cells<NP> zl2;
+        if (ADJ) zl2.load(PL + (r0 + rr + R) * BW + XH + c0);  // own Z_lo cells
         const int gy = gy0 + r0 + rr;
-        const bool own = gy < ny && gx < nx;
-        float4 kh = make_float4(0.f, 0.f, 0.f, 0.f), kl = kh;
-        if (varying && own) {
-          kh = __ldg(reinterpret_cast<const float4*>(I.kappa + (long long)gy * nx + gx));
-          if (!ADJ) kl = __ldg(reinterpret_cast<const float4*>(I.kappa_lo + (long long)gy * nx + gx));
-        }
-        float dn[4], pn[4], pl[4];
-        float st4[4];
-        stencil_cells2<R, ADJ>(win, f, w2, st4);
+        // forward: zero-sum pair form (a + b) - 2c per tap; adjoint: difference form on Z
+        Cells<NP> st2;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float c = f[8 + j];
-          if (!ADJ) {  // zero-sum pair form (a + b) - 2c per tap
-            const float acc = st4[j];
+        for (int p = 0; p < NP; ++p) st2.v[p] = stencil_pair<R, ADJ>(win, f, p, w2);
+        float dn[2 * NP], pn[2 * NP], pl[2 * NP];
+#pragma unroll
+        for (int j = 0; j < 2 * NP; ++j) {
+          const float c = win[R].get(j);
+          if (!ADJ) {
+            const float acc = st2.get(j);
             // D += c_lap (kappa_hi + kappa_lo) L, the product rounded once before it meets D
-            const float inc = varying ? fmaf(c_lap * f4get(kh, j), acc, (c_lap * f4get(kl, j)) * acc)
+            const float inc = varying ? fmaf(c_lap * kh2[rr].get(j), acc, (c_lap * kl2[rr].get(j)) * acc)
                                       : fmaf(ckh, acc, ckl * acc);
-            dn[j] = f4get(d4[rr], j) + inc;
+            dn[j] = d2[rr].get(j) + inc;
             pn[j] = c + dn[j];
             pl[j] = 0.f;
           } else {
-            const float acc = st4[j] + lo[rr][j];  // difference form on Z
-            const float g = fmaf(c_lap, acc, f4get(d4[rr], j));
+            const float acc = st2.get(j) + lo[rr].get(j);
+            const float g = fmaf(c_lap, acc, d2[rr].get(j));
             dn[j] = g;
             float e = 0.f;
-            const float u = varying ? f4get(kh, j) * g : fmaf(I.kappa0, g, I.kappa0_lo * g);  // kappa G
-            pn[j] = final_step ? g : two_sum(c, u, e);                                          // Z += kappa G
-            pl[j] = f4get(zl4, j) + e;
+            const float u = varying ? kh2[rr].get(j) * g : fmaf(k0h, g, k0l * g);  // kappa G
+            pn[j] = final_step ? g : two_sum(c, u, e);                                  // Z += kappa G
+            pl[j] = zl2.get(j) + e;
           }
         }
-        if (own) {
+        if (gy < ny && gx < nx) {
           const long long gi = (long long)gy * nx + gx;
-          *reinterpret_cast<float4*>(out + gi) = make_float4(pn[0], pn[1], pn[2], pn[3]);
+          store_cells<NP>(out + gi, pn);
           if (!final_step) {
-            *reinterpret_cast<float4*>(I.D + gi) = make_float4(dn[0], dn[1], dn[2], dn[3]);
-            if (ADJ) *reinterpret_cast<float4*>(I.P_lo[(step + 1) & 1] + gi) = make_float4(pl[0], pl[1], pl[2], pl[3]);
+            store_cells<NP>(D + gi, dn);
+            if (ADJ) store_cells<NP>(out_lo + gi, pl);
           }
         }
 #pragma unroll
@@ -262,6 +283,7 @@ __global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS) batch_step_kernel(con
       }
     }
     __syncthreads();  // this stage is refilled by the next iteration's TMA
+    if (ADJ && !final_step && dc.e1 > dc.e0) inject(n - 1);  // for the next step, on the G just stored
     dc = dn;
     dn = dnn;
   }
@@ -291,7 +313,7 @@ const void* kernel_for(int R, int variant, bool adj, bool runall = false) {
   }
 }
 
-int threads_for(int variant, bool adj) { return (TX / 4) * (batch_tile_y(variant) / run_rows(adj)); }
+int threads_for(int variant) { return TCOLS * (batch_tile_y(variant) / RUN); }
 
 }  // namespace
 
@@ -315,7 +337,7 @@ int batch_max_ctas(int R, int variant, bool adj) {
     int dev = 0, sms = 0, per = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads_for(variant, adj), smem) != cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads_for(variant), smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
@@ -331,7 +353,17 @@ cudaError_t batch_step_launch(int R, int variant, const BatchStepArgs& a, int nc
   if (!fn) return cudaErrorInvalidValue;
   const int grid = nctas < a.active ? nctas : a.active;
   void* args[] = {const_cast<BatchStepArgs*>(&a)};
-  return cudaLaunchKernel(fn, dim3(grid), dim3(threads_for(variant, adj)), args, batch_smem(R, variant, adj), st);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads_for(variant));
+  cfg.dynamicSmemBytes = batch_smem(R, variant, adj);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];  // starts while the previous step drains (the kernel waits for it itself)
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 cudaError_t batch_run_launch(int R, int variant, const BatchStepArgs& a, int nctas, cudaStream_t st) {
@@ -341,7 +373,7 @@ cudaError_t batch_run_launch(int R, int variant, const BatchStepArgs& a, int nct
   if (!fn || nctas <= 0) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(nctas);
-  cfg.blockDim = dim3(threads_for(variant, adj));
+  cfg.blockDim = dim3(threads_for(variant));
   cfg.dynamicSmemBytes = batch_smem(R, variant, adj);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];

@@ -178,8 +178,8 @@ cudaError_t step3d_tma_launch(int R, const StepArgs& a, const CUtensorMap& cur, 
 
 // wave2d_tma.cu: 2D increment-form step with TMA tile pipelines
 bool tma2d_supported(int R);
-int tma2d_tile();  // tile edge in cells (tiles numbered row by row)
-// halo boxes (80 x (64+2R)) of an nx x ny float field of row pitch `pitch`
+void tma2d_tile(int* tx, int* ty);  // tile extents in cells (tiles numbered row by row)
+// halo boxes (80 x (32+2R)) of an nx x ny float field of row pitch `pitch`
 cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CUtensorMap* halo);
 // mode 0: forward, constant medium; 1: forward, varying medium; 2: adjoint (either medium);
 // sp 0: no absorbing layer, 1: layer with the forward update, 2: layer with the adjoint update;

@@ -521,13 +521,15 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
     }
   }
   if (p->tma3d || p->tma2d) {  // injection lists of the TMA step kernels (the adjoint injects after each step)
-    const int nx = p->n[0], ny = p->n[1], nz = p->n[2], T = tma2d_tile();
-    const int tx = (nx + T - 1) / T, ty = (ny + T - 1) / T;
+    const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
+    int TX, TY;
+    tma2d_tile(&TX, &TY);
+    const int tx = (nx + TX - 1) / TX, ty = (ny + TY - 1) / TY;
     std::vector<std::vector<InjCell>> bins((size_t)(p->tma3d ? p->tma3d_split.nctas : tx * ty));
     for (int i = 0; i < p->n_inj; ++i) {
       const long long c = p->h_inj_cell[i];
       const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-      const int bin = p->tma3d ? tma3d_cta_of(nx, ny, nz, p->tma3d_split, x, y, z) : (y / T) * tx + x / T;
+      const int bin = p->tma3d ? tma3d_cta_of(nx, ny, nz, p->tma3d_split, x, y, z) : (y / TY) * tx + x / TX;
       bins[bin].push_back(InjCell{inj_cell[i], p->h_inj_ptr[i], p->h_inj_ptr[i + 1]});
     }
     std::vector<int> ptr(1, 0);

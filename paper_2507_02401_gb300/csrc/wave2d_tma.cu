@@ -17,18 +17,14 @@
 // 7e-7 with the compensated Z.  Each step also adds S^T r_{m-1}, the sensor
 // injection of the step after it, to the G it has just stored (lists per tile).
 //
-// Persistent CTAs walk 64 x 64 tiles; one thread issues the TMA load of the
-// next tile's boxes (80 x (64+2R) floats, halo included, zero outside the
+// Persistent CTAs walk 64 x 32 tiles; one thread issues the TMA load of the
+// next tile's boxes (80 x (32+2R) floats, halo included, zero outside the
 // grid: P for the forward, Z and Z_lo for the adjoint) into the second of two
 // shared-memory stages while the CTA computes the current one.  Each thread
-// owns 4 columns x 8 consecutive rows (4 rows in the adjoint, whose two boxes
-// and two stencils per cell need more registers: 256 threads of at most 170
-// registers per tile ran 6-19 % faster at 4096^2 than 128 threads of 238,
-// and faster than 256 threads capped at 128 registers, which spilled).
-// y neighbours come from a sliding register window of 2R+1 rows, x
-// neighbours from the shared-memory row; its own D / G (and kappa) cells are
-// loaded straight into registers (coalesced 16-byte loads issued before the
-// wait for the boxes).
+// owns 4 columns x 4 consecutive rows: y neighbours come from a sliding
+// register window of 2R+1 rows, x neighbours from the shared-memory row; its
+// own D / G cells are loaded straight into registers before the wait for the
+// boxes, kappa and G_lo two rows ahead of their use.
 // Compulsory DRAM traffic per point-update: forward P and D read, P^{n+1} and
 // D^{n+1} written (16 B), plus kappa hi/lo (8 B) for a varying medium;
 // adjoint Z, Z_lo, G read and written (24 B), plus kappa (4 B) for a varying
@@ -46,8 +42,19 @@
 namespace pat {
 namespace {
 
-constexpr int TX = 64, TY = 64, TCOLS = TX / 2, RUN = 8;
-constexpr int THREADS = TCOLS * (TY / RUN);  // 256: each thread owns 2 columns x 8 rows
+// 64 x 32 tiles, 128 threads, each with 2 NP columns x RUN rows.  Measured at order 8, K / K* us per step, on
+// 4000 x 3600 | 1400^2 | 1024^2 cells:
+//   4 columns x 4 rows, 64 x 32 tiles (3 CTAs per SM)   39.8 / 69.9 | 7.2 / 12.0 | 4.5 / 8.5
+//   2 columns x 8 rows, 64 x 64 tiles (2 CTAs per SM)   42.0 / 76.9 | 8.0 / 14.5 | 4.7 / 8.3
+//   2 columns x 8 rows, 64 x 32 tiles (3 CTAs)          42.0 / 73.1 | 8.0 / 12.5 | 4.8 / 8.9
+//   4 columns x 8 rows, 64 x 64 tiles (2 to 3 CTAs)     40.0 / 93.1 | 6.8 / 16.6 | 5.8 / 9.5
+// The first needs the fewest shared-memory wavefronts per cell of those that leave 12 warps on an SM in the
+// adjoint, whose two stencils keep the FP32 and shared-memory pipes about half busy each.
+constexpr int TX = 64, TY = 32, NP = 2, TCOLS = TX / (2 * NP), RUN = 4;
+constexpr int THREADS = TCOLS * (TY / RUN);
+// CTAs per SM to leave registers for: a fourth pays up to order 4 (1024^2 order 4 K* 6.3 against 7.4 us), except
+// in the full form, which spills then (1000 x 875 order 4 K* 7.8 against 6.8 us)
+constexpr int min_ctas(int R, bool full) { return R <= 3 && !full ? 4 : 3; }
 constexpr int XH = 8;            // box columns left of the tile (>= R, 16-byte aligned)
 constexpr int BW = TX + 2 * XH;  // box width, 80 floats
 
@@ -78,7 +85,7 @@ __device__ __forceinline__ void fused_sample2(const StepArgs& a, long long bid, 
 // FULL (grids of odd width): the forward's stencil takes the difference form and the adjoint keeps G as a
 // compensated pair too (G_lo in dbuf_lo), with the rounding of kappa G carried into Z_lo.
 template <int R, int MODE, int SP, bool FULL>
-__global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
+__global__ void __launch_bounds__(THREADS, min_ctas(R, FULL)) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
                                                              const __grid_constant__ CUtensorMap ml, int* status,
                                                              long long timeout_ns) {
   constexpr bool VARC = MODE == 1, ADJ = MODE == 2;
@@ -92,7 +99,7 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
   const int nx = a.nx, ny = a.ny, pitch = a.pitch;
   const int tiles_x = (nx + TX - 1) / TX;
   const int ntiles = tiles_x * ((ny + TY - 1) / TY);
-  const int c0 = (t % TCOLS) * 2, r0 = (t / TCOLS) * RUN;
+  const int c0 = (t % TCOLS) * 2 * NP, r0 = (t / TCOLS) * RUN;
   const bool load_d = !a.d_zero;
   const bool kv = a.kappa != nullptr;  // adjoint: varying medium (per-cell kappa)
   const unsigned stage_bytes = (unsigned)G::STAGE * 4u;
@@ -144,21 +151,24 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
     const int gx = gx0 + c0;
     // own-cell fields straight into registers, in flight while the boxes land: D or G of every row; kappa
     // and G_lo (fetch) two rows ahead of their use
-    const float2 z2 = dup2(0.f);
-    float2 d2[RUN], kh2[RUN], kl2[RUN], gl2[RUN];
+    Cells<NP> d2[RUN], kh2[RUN], kl2[RUN], gl2[RUN];
     const bool need_k = VARC || (ADJ && kv && !a.final_step);
     auto fetch = [&](int rr) {
       const int gy = gy0 + r0 + rr;
       const long long gi = (long long)gy * pitch + gx;
       const bool in = gy < ny && gx < nx;
-      kh2[rr] = need_k && in ? __ldg(reinterpret_cast<const float2*>(a.kappa + gi)) : z2;
-      kl2[rr] = (VARC || FULL) && need_k && in ? __ldg(reinterpret_cast<const float2*>(a.kappa_lo + gi)) : z2;
-      gl2[rr] = ADJ && FULL && in ? ld_stream2(a.dbuf_lo + gi) : z2;
+      kh2[rr].fill(0.f);
+      kl2[rr].fill(0.f);
+      gl2[rr].fill(0.f);
+      if (need_k && in) kh2[rr].ldg(a.kappa + gi);
+      if ((VARC || FULL) && need_k && in) kl2[rr].ldg(a.kappa_lo + gi);
+      if (ADJ && FULL && in) gl2[rr].stream(a.dbuf_lo + gi);
     };
 #pragma unroll
     for (int rr = 0; rr < RUN; ++rr) {
       const int gy = gy0 + r0 + rr;
-      d2[rr] = (load_d && gy < ny && gx < nx) ? ld_stream2(a.dbuf + (long long)gy * pitch + gx) : z2;
+      d2[rr].fill(0.f);
+      if (load_d && gy < ny && gx < nx) d2[rr].stream(a.dbuf + (long long)gy * pitch + gx);
     }
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) fetch(rr);
@@ -177,55 +187,58 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
     // tiles outside it run exactly the code of the kernel without a layer
     auto update = [&](auto in_layer) {
       constexpr bool LAYER = decltype(in_layer)::value;
-      float2 lo[RUN];  // adjoint: the Z_lo part of the stencil, first pass
+      Cells<NP> lo[RUN];  // adjoint: the Z_lo part of the stencil, first pass
       if (ADJ) stencil_run_pair<R, RUN, BW>(PL + (r0 + R) * BW + XH + c0, w2, nwc, lo);
-      // sliding window over this thread's 2 columns: win[i] = box row (row - R + i)
+      // sliding window over this thread's columns: win[i] = box row (row - R + i)
       const float* own = P + (r0 + R) * BW + XH + c0;
-      float2 win[2 * R + 1];
+      Cells<NP> win[2 * R + 1];
 #pragma unroll
-      for (int i = 0; i < 2 * R; ++i) win[i] = *reinterpret_cast<const float2*>(own + (i - R) * BW);
+      for (int i = 0; i < 2 * R; ++i) win[i].load(own + (i - R) * BW);
 #pragma unroll
       for (int rr = 0; rr < RUN; ++rr) {
-        win[2 * R] = *reinterpret_cast<const float2*>(own + (rr + R) * BW);
-        RowPairs<R> f;
+        win[2 * R].load(own + (rr + R) * BW);
+        Row<R, NP> f;
         f.load(own + rr * BW, win[R]);
         const int gy = gy0 + r0 + rr;
         const long long gi = (long long)gy * pitch + gx;
         const bool in = gy < ny && gx < nx;
         if (rr + 2 < RUN) fetch(rr + 2);
-        float2 sa2 = dup2(1.f), sb2 = sa2;
+        Cells<NP> sa2, sb2, zl2;
+        sa2.fill(1.f);
+        sb2.fill(1.f);
         if (LAYER && in) {
-          sa2 = __ldg(reinterpret_cast<const float2*>(a.sp_a + gi));
-          sb2 = __ldg(reinterpret_cast<const float2*>(a.sp_b + gi));
+          sa2.ldg(a.sp_a + gi);
+          sb2.ldg(a.sp_b + gi);
         }
-        float2 zl2 = z2;  // adjoint: own Z_lo cells
-        if (ADJ) zl2 = *reinterpret_cast<const float2*>(PL + (r0 + rr + R) * BW + XH + c0);
+        if (ADJ) zl2.load(PL + (r0 + rr + R) * BW + XH + c0);  // own Z_lo cells
         // forward: zero-sum pair form (a + b) - 2c per tap; adjoint (and FULL): difference form
-        const float2 st2 = stencil_pair<R, ADJ || FULL>(win, f, w2);
-        float dn[2], pn[2], pl[2], gn[2];
+        Cells<NP> st2;
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const float c = f2get(win[R], j);  // own P or Z
-          const float fa = f2get(sa2, j), fb = f2get(sb2, j);
+        for (int p = 0; p < NP; ++p) st2.v[p] = stencil_pair<R, ADJ || FULL>(win, f, p, w2);
+        float dn[2 * NP], pn[2 * NP], pl[2 * NP], gn[2 * NP];
+#pragma unroll
+        for (int j = 0; j < 2 * NP; ++j) {
+          const float c = win[R].get(j);  // own P or Z
+          const float fa = sa2.get(j), fb = sb2.get(j);
           if (!ADJ) {
-            const float acc = f2get(st2, j);
-            const float inc = VARC ? fmaf(a.c_lap * f2get(kh2[rr], j), acc, (a.c_lap * f2get(kl2[rr], j)) * acc)
+            const float acc = st2.get(j);
+            const float inc = VARC ? fmaf(a.c_lap * kh2[rr].get(j), acc, (a.c_lap * kl2[rr].get(j)) * acc)
                                    : fmaf(ckh, acc, ckl * acc);
             if (!LAYER)
-              dn[j] = f2get(d2[rr], j) + inc;
+              dn[j] = d2[rr].get(j) + inc;
             else  // forward in the layer
-              dn[j] = load_d ? fmaf(fa, f2get(d2[rr], j), fb * inc) : fmaf(fa - 1.f, c, fb * inc);
+              dn[j] = load_d ? fmaf(fa, d2[rr].get(j), fb * inc) : fmaf(fa - 1.f, c, fb * inc);
             pn[j] = c + dn[j];
             pl[j] = gn[j] = 0.f;
           } else {
-            const float acc = f2get(st2, j) + f2get(lo[rr], j);
-            const float zl = f2get(zl2, j);
-            const float kap = kv ? f2get(kh2[rr], j) : a.kappa0;
+            const float acc = st2.get(j) + lo[rr].get(j);
+            const float zl = zl2.get(j);
+            const float kap = kv ? kh2[rr].get(j) : a.kappa0;
             float g, gl = 0.f;  // G' = G + L Z (S^T r injected into G beforehand)
             if (FULL && !a.final_step)
-              g = two_sum(f2get(d2[rr], j), a.c_lap * acc + f2get(gl2[rr], j), gl);
+              g = two_sum(d2[rr].get(j), a.c_lap * acc + gl2[rr].get(j), gl);
             else
-              g = fmaf(a.c_lap, acc, FULL ? f2get(d2[rr], j) + f2get(gl2[rr], j) : f2get(d2[rr], j));
+              g = fmaf(a.c_lap, acc, FULL ? d2[rr].get(j) + gl2[rr].get(j) : d2[rr].get(j));
             dn[j] = g;
             gn[j] = gl;
             if (a.final_step) {
@@ -238,7 +251,7 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
             } else {
               float u, ul = 0.f;  // kappa G', and what its rounding dropped (FULL)
               if (FULL) {
-                const float kl = kv ? f2get(kl2[rr], j) : a.kappa0_lo;
+                const float kl = kv ? kl2[rr].get(j) : a.kappa0_lo;
                 u = kap * g;
                 ul = fmaf(kap, g, -u) + fmaf(kap, gl, kl * g);
               } else {
@@ -256,11 +269,11 @@ __global__ void __launch_bounds__(THREADS, 2) step2d_tma_kernel(const StepArgs a
           }
         }
         if (in) {
-          *reinterpret_cast<float2*>(a.next + gi) = make_float2(pn[0], pn[1]);
+          store_cells<NP>(a.next + gi, pn);
           if (!a.final_step) {
-            *reinterpret_cast<float2*>(a.dbuf + gi) = make_float2(dn[0], dn[1]);
-            if (ADJ) *reinterpret_cast<float2*>(a.next_lo + gi) = make_float2(pl[0], pl[1]);
-            if (ADJ && FULL) *reinterpret_cast<float2*>(a.dbuf_lo + gi) = make_float2(gn[0], gn[1]);
+            store_cells<NP>(a.dbuf + gi, dn);
+            if (ADJ) store_cells<NP>(a.next_lo + gi, pl);
+            if (ADJ && FULL) store_cells<NP>(a.dbuf_lo + gi, gn);
           }
         }
 #pragma unroll
@@ -317,7 +330,10 @@ size_t smem_for(int R, int mode) {
 
 }  // namespace
 
-int tma2d_tile() { return TX; }
+void tma2d_tile(int* tx, int* ty) {
+  *tx = TX;
+  *ty = TY;
+}
 
 bool tma2d_supported(int R) { return R == 1 || R == 3 || R == 5 || R == 7; }
 
