@@ -133,6 +133,13 @@ struct StepArgs {
   const float* sp_a;
   const float* sp_b;
   int sp_w;
+  // medium gradient (2D TMA kernel): the full-form forward writes L cur to lp (nullptr = not); the adjoint
+  // with gsum_hi set adds gcoef lp .* Z^m to the compensated sums gsum_hi + gsum_lo
+  int full;  // 2D TMA forward: the full form (difference-form stencil), whatever the width
+  float* lp;
+  float gcoef;
+  float* gsum_hi;
+  float* gsum_lo;
   const float* inj_r;
   int inj_t;
   const int* inj_tile_ptr;
@@ -181,7 +188,8 @@ bool tma2d_supported(int R);
 void tma2d_tile(int* tx, int* ty);  // tile extents in cells (tiles numbered row by row)
 // halo boxes (80 x (32+2R)) of an nx x ny float field of row pitch `pitch`
 cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CUtensorMap* halo);
-// mode 0: forward, constant medium; 1: forward, varying medium; 2: adjoint (either medium);
+// mode 0: forward, constant medium; 1: forward, varying medium; 2: adjoint (either medium); 3: adjoint with the
+// medium gradient's sum (sp 0);
 // sp 0: no absorbing layer, 1: layer with the forward update, 2: layer with the adjoint update;
 // full: forward stencil in the difference form, adjoint with G compensated in a.dbuf_lo
 long long tma2d_threads(int nx, int ny, int R, int mode, int sp, bool full);  // threads of one launch
@@ -202,6 +210,8 @@ cudaError_t pitch_copy_launch(float* dst, int dpitch, const float* src, int spit
 // zform: the adjoint state holds Z = kappa Q (2D TMA engine); the accumulator divides by kappa
 cudaError_t grad_acc_launch(int R, double* gacc, const float* Q, const float* Qlo, const float* P, float coef,
                             const StepArgs& a, int dim, bool zform, cudaStream_t st);
+// g = (hi + lo) / kappa per cell, from pitched sums to a dense image
+cudaError_t grad_finish_launch(float* g, const float* hi, const float* lo, const StepArgs& a, cudaStream_t st);
 cudaError_t d2f_launch(float* out, const double* in, long long n, cudaStream_t st);
 cudaError_t dfill_launch(double* p, long long n, cudaStream_t st);
 cudaError_t fill_launch(float* p, long long n, float v, cudaStream_t st);

@@ -115,11 +115,12 @@ static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t 
   if (p->tma2d) {
     // TMA tile pipelines: forward (constant or varying medium); adjoint in Z = kappa Q with Z
     // compensated (boxes of Z and Z_lo), the next step's injection added to G after each tile
-    const int mode = adj ? 2 : (p->varc ? 1 : 0);
+    const int mode = adj ? (a.gsum_hi ? 3 : 2) : (p->varc ? 1 : 0);
     const int sp = p->sponge_w > 0 ? (adj ? 2 : 1) : 0;
     // odd widths used to take the plain kernel, whose forward stencil is the difference form and whose adjoint
     // carries G as a compensated pair: the kernel's full form keeps that accuracy
-    const bool full = p->n[0] % 4 != 0;
+    // (as did the medium gradient's L P, whose difference form comes with the full forward)
+    const bool full = p->n[0] % 4 != 0 || (!adj && a.full);
     const long long nthr = tma2d_threads(p->n[0], p->n[1], p->R, mode, sp, full);
     if (y && a.ns > nthr) a.y = nullptr;
     // copies: a second lookup may move the cached descriptors
@@ -522,13 +523,94 @@ static pat_status kg_alloc(pat_plan* p, int C, int nseg) {
   cudaError_t e = cudaMalloc(&p->kg_ckpt, sizeof(float) * N * 2 * nseg);
   if (e == cudaSuccess) e = cudaMalloc(&p->kg_seg, sizeof(float) * N * C);
   if (e == cudaSuccess) e = cudaMalloc(&p->kg_work, sizeof(float) * N * 3);
-  if (e == cudaSuccess) e = cudaMalloc(&p->kg_acc, sizeof(double) * (size_t)p->N);
+  if (e == cudaSuccess) e = cudaMalloc(&p->kg_acc, sizeof(double) * N);
   if (e != cudaSuccess) {
     cudaGetLastError();
     kg_free(p);
     return cuda_fail(e, "cudaMalloc(gradient checkpoints)");
   }
   p->kg_segment = C;
+  return PAT_OK;
+}
+
+// The 2D TMA engine's run of the gradient: a segment keeps L P^n (which the forward step has at hand) instead
+// of P^n, and each adjoint step adds its own term, so a time step costs two forward steps and one adjoint
+// step and no pass of its own over the gradient.  The sums live in the FP64 accumulator's buffer, as FP32
+// pairs.  (384^2 order 8: 20 us per time step when every term was a launch that recomputed L P and divided by
+// kappa in FP64, 11 us so.)
+static pat_status kappa_grad_tma2d(pat_plan* p, const float* x, const float* r, float* g, int C, cudaStream_t st) {
+  const long long N = p->Np;  // floats of a field
+  const int nt = p->nt, last = (nt - 2) / C;  // segments 0 .. last of n = 0 .. nt-2
+  float* W[2] = {p->kg_work, p->kg_work + N};
+  float* D = p->kg_work + 2 * N;
+  auto ck = [&](int k, int f) { return p->kg_ckpt + ((size_t)k * 2 + f) * N; };
+  auto seg = [&](int j) { return p->kg_seg + (size_t)j * N; };
+  auto copy = [&](float* d, const float* s) {
+    return cudaMemcpyAsync(d, s, sizeof(float) * N, cudaMemcpyDeviceToDevice, st);
+  };
+  StepArgs f = step_args(p);
+  f.y = nullptr;
+  f.full = 1;  // L P through the difference form
+  f.dbuf = D;
+  // steps n0 .. n1-1 from the field cur (and D), L P^n of segment k kept
+  auto forward = [&](const float* cur, int n0, int n1, int k, bool checkpoints) -> pat_status {
+    for (int n = n0; n < n1; ++n) {
+      if (checkpoints && n % C == 0) {
+        PAT_TRY_CUDA(copy(ck(n / C, 0), cur));
+        if (n > 0) PAT_TRY_CUDA(copy(ck(n / C, 1), D));
+      }
+      f.cur = cur;
+      f.next = W[n % 2];
+      f.d_zero = (n == 0);
+      f.c_lap = (n == 0) ? 0.5f : 1.f;
+      f.flip = n & 1;
+      f.lp = n / C == k ? seg(n - k * C) : nullptr;
+      PAT_TRY_CUDA(step_launch(p, false, f, st));
+      cur = f.next;
+    }
+    return PAT_OK;
+  };
+  PAT_TRY(forward(x, 0, nt - 1, last, true));  // the last segment is kept in passing
+  int loaded = last;
+
+  float* G = p->d_wv[2];
+  auto Qbuf = [&](int m) { return p->d_wv[(nt - m) % 2]; };
+  auto Qlo = [&](int m) { return p->d_wv[3 + (nt - m) % 2]; };
+  float* hi = reinterpret_cast<float*>(p->kg_acc);
+  float* lo = hi + N;
+  PAT_TRY_CUDA(fill_launch(hi, 2 * N, 0.f, st));
+  PAT_TRY_CUDA(fill_launch(G, N, 0.f, st));
+  PAT_TRY_CUDA(fill_launch(p->d_wv[5], N, 0.f, st));
+  PAT_TRY_CUDA(fill_launch(Qbuf(nt), N, 0.f, st));
+  PAT_TRY_CUDA(fill_launch(Qlo(nt), N, 0.f, st));
+  PAT_TRY_CUDA(inject_launch(G, p->n_inj, p->d_inj_cell, p->d_inj_ptr, p->d_ent_sensor, p->d_ent_w, r, nt, nt - 1,
+                             nullptr, st));
+  StepArgs c = step_args(p);
+  c.y = nullptr;
+  c.dbuf = G;
+  c.dbuf_lo = p->d_wv[5];
+  c.inj_r = r;  // each step leaves G^m + S^T r_{m-1} for the next
+  c.c_lap = 1.f;
+  c.gsum_hi = hi;
+  c.gsum_lo = lo;
+  for (int m = nt - 1; m >= 1; --m) {  // Z^m, and its term kappa^{-1} Z^m .* L P^{m-1}, halved for m = 1
+    const int n = m - 1, k = n / C;
+    if (k != loaded) {
+      if (k > 0) PAT_TRY_CUDA(copy(D, ck(k, 1)));
+      PAT_TRY(forward(ck(k, 0), k * C, std::min(k * C + C, nt - 1), k, false));
+      loaded = k;
+    }
+    c.flip = m & 1;
+    c.inj_t = m - 1;
+    c.cur = Qbuf(m + 1);
+    c.cur_lo = Qlo(m + 1);
+    c.next = Qbuf(m);
+    c.next_lo = Qlo(m);
+    c.lp = seg(n - k * C);
+    c.gcoef = n == 0 ? 0.5f : 1.f;
+    PAT_TRY_CUDA(step_launch(p, true, c, st));
+  }
+  PAT_TRY_CUDA(grad_finish_launch(g, hi, lo, c, st));
   return PAT_OK;
 }
 
@@ -558,6 +640,7 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
     PAT_TRY_CUDA(image_to_field(p, p->d_wv[0], x, st));
     x = p->d_wv[0];
   }
+  if (p->tma2d) return kappa_grad_tma2d(p, x, r, g, C, st);
 
   // ---- forward run keeping the restart state at n = 0, C, 2C, ...
   if (two_d) {  // increment form: state (P^n, D^n)

@@ -54,7 +54,7 @@ constexpr int TX = 64, TY = 32, NP = 2, TCOLS = TX / (2 * NP), RUN = 4;
 constexpr int THREADS = TCOLS * (TY / RUN);
 // CTAs per SM to leave registers for: a fourth pays up to order 4 (1024^2 order 4 K* 6.3 against 7.4 us), except
 // in the full form, which spills then (1000 x 875 order 4 K* 7.8 against 6.8 us)
-constexpr int min_ctas(int R, bool full) { return R <= 3 && !full ? 4 : 3; }
+constexpr int min_ctas(int R, bool full, bool grad) { return grad ? 2 : R <= 3 && !full ? 4 : 3; }
 constexpr int XH = 8;            // box columns left of the tile (>= R, 16-byte aligned)
 constexpr int BW = TX + 2 * XH;  // box width, 80 floats
 
@@ -84,8 +84,11 @@ __device__ __forceinline__ void fused_sample2(const StepArgs& a, long long bid, 
 // Tiles that do not reach the layer use a = b = 1 without loading the factors.
 // FULL (grids of odd width): the forward's stencil takes the difference form and the adjoint keeps G as a
 // compensated pair too (G_lo in dbuf_lo), with the rounding of kappa G carried into Z_lo.
-template <int R, int MODE, int SP, bool FULL>
-__global__ void __launch_bounds__(THREADS, min_ctas(R, FULL)) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
+// GRAD (adjoint): adds this step's term gcoef Z^m .* L P^{m-1} of the medium gradient to a compensated sum.
+// The sums are pairs of FP32 (TwoSum with the product's rounding error, ~2^-47): FP64 arithmetic runs at 2
+// operations per clock and SM here, and dividing by kappa once at the end replaces a division per step.
+template <int R, int MODE, int SP, bool FULL, bool GRAD = false>
+__global__ void __launch_bounds__(THREADS, min_ctas(R, FULL, GRAD)) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
                                                              const __grid_constant__ CUtensorMap ml, int* status,
                                                              long long timeout_ns) {
   constexpr bool VARC = MODE == 1, ADJ = MODE == 2;
@@ -151,7 +154,7 @@ __global__ void __launch_bounds__(THREADS, min_ctas(R, FULL)) step2d_tma_kernel(
     const int gx = gx0 + c0;
     // own-cell fields straight into registers, in flight while the boxes land: D or G of every row; kappa
     // and G_lo (fetch) two rows ahead of their use
-    Cells<NP> d2[RUN], kh2[RUN], kl2[RUN], gl2[RUN];
+    Cells<NP> d2[RUN], kh2[RUN], kl2[RUN], gl2[RUN], lp2[RUN], sh2[RUN], sl2[RUN];
     const bool need_k = VARC || (ADJ && kv && !a.final_step);
     auto fetch = [&](int rr) {
       const int gy = gy0 + r0 + rr;
@@ -163,6 +166,11 @@ __global__ void __launch_bounds__(THREADS, min_ctas(R, FULL)) step2d_tma_kernel(
       if (need_k && in) kh2[rr].ldg(a.kappa + gi);
       if ((VARC || FULL) && need_k && in) kl2[rr].ldg(a.kappa_lo + gi);
       if (ADJ && FULL && in) gl2[rr].stream(a.dbuf_lo + gi);
+      if (GRAD && in) {
+        lp2[rr].stream(a.lp + gi);
+        sh2[rr].stream(a.gsum_hi + gi);
+        sl2[rr].stream(a.gsum_lo + gi);
+      }
     };
 #pragma unroll
     for (int rr = 0; rr < RUN; ++rr) {
@@ -270,10 +278,25 @@ __global__ void __launch_bounds__(THREADS, min_ctas(R, FULL)) step2d_tma_kernel(
         }
         if (in) {
           store_cells<NP>(a.next + gi, pn);
+          if (!ADJ && FULL && a.lp != nullptr) st2.store(a.lp + gi);
           if (!a.final_step) {
             store_cells<NP>(a.dbuf + gi, dn);
             if (ADJ) store_cells<NP>(a.next_lo + gi, pl);
             if (ADJ && FULL) store_cells<NP>(a.dbuf_lo + gi, gn);
+            if (GRAD) {
+              float sh[2 * NP], sl[2 * NP];
+#pragma unroll
+              for (int j = 0; j < 2 * NP; ++j) {
+                const float l = a.gcoef * lp2[rr].get(j);
+                const float ph = pn[j] * l;
+                const float pe = fmaf(pl[j], l, fmaf(pn[j], l, -ph));
+                float e;
+                sh[j] = two_sum(sh2[rr].get(j), ph, e);
+                sl[j] = sl2[rr].get(j) + (e + pe);
+              }
+              store_cells<NP>(a.gsum_hi + gi, sh);
+              store_cells<NP>(a.gsum_lo + gi, sl);
+            }
           }
         }
 #pragma unroll
@@ -309,6 +332,7 @@ const void* kernel_r(int mode, int sp) {
     case 4: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 1, 1, FULL>);
     case 6: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 2, 0, FULL>);
     case 8: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 2, 2, FULL>);
+    case 9: return reinterpret_cast<const void*>(&step2d_tma_kernel<R, 2, 0, FULL, true>);
     default: return nullptr;  // mismatched layer modes are not instantiated
   }
 }
@@ -324,7 +348,7 @@ const void* kernel_for(int R, int mode, int sp, bool full) {
 }
 
 size_t smem_for(int R, int mode) {
-  if (mode == 2) return R == 1 ? G2<1, 2>::SMEM : R == 3 ? G2<3, 2>::SMEM : R == 5 ? G2<5, 2>::SMEM : G2<7, 2>::SMEM;
+  if (mode >= 2) return R == 1 ? G2<1, 2>::SMEM : R == 3 ? G2<3, 2>::SMEM : R == 5 ? G2<5, 2>::SMEM : G2<7, 2>::SMEM;
   return R == 1 ? G2<1>::SMEM : R == 3 ? G2<3>::SMEM : R == 5 ? G2<5>::SMEM : G2<7>::SMEM;
 }
 
@@ -352,7 +376,7 @@ cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CU
 
 // Persistent grid: as many CTAs as fit on the device, at most one per tile.
 int tma2d_ctas(int nx, int ny, int R, int mode, int sp, bool full) {
-  static int cached[2][3][3][8] = {{{{0}}}};
+  static int cached[2][4][3][8] = {{{{0}}}};
   int& c = cached[full][mode][sp][R];
   if (!c) {
     int dev = 0, sms = 148, per = 1;

@@ -411,6 +411,16 @@ __global__ void grad_acc_kernel(double* __restrict__ gacc, const float* __restri
   }
 }
 
+__global__ void grad_finish_kernel(float* __restrict__ g, const float* __restrict__ hi, const float* __restrict__ lo,
+                                   const StepArgs a) {
+  const long long N = (long long)a.nx * a.ny;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (long long)gridDim.x * blockDim.x) {
+    const long long i = k / a.nx * a.pitch + k % a.nx;
+    const double kap = a.kappa ? (double)a.kappa[i] + (double)a.kappa_lo[i] : (double)a.kappa0 + (double)a.kappa0_lo;
+    g[k] = (float)(((double)hi[i] + (double)lo[i]) / kap);
+  }
+}
+
 __global__ void d2f_kernel(float* __restrict__ out, const double* __restrict__ in, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     out[i] = (float)in[i];
@@ -433,6 +443,11 @@ cudaError_t grad_acc_launch(int R, double* gacc, const float* Q, const float* Ql
     case 7: grad_acc_kernel<7><<<blocks, 256, 0, st>>>(gacc, Q, Qlo, P, coef, a.nx, a.ny, a.nz, dim, zform, a); break;
     default: return cudaErrorInvalidValue;
   }
+  return cudaGetLastError();
+}
+
+cudaError_t grad_finish_launch(float* g, const float* hi, const float* lo, const StepArgs& a, cudaStream_t st) {
+  grad_finish_kernel<<<grid_for((long long)a.nx * a.ny), 256, 0, st>>>(g, hi, lo, a);
   return cudaGetLastError();
 }
 
