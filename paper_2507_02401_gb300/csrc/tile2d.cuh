@@ -118,13 +118,12 @@ __device__ __forceinline__ float2 add_pair(float2 a, float2 b, bool aligned) {
 }
 
 // Laplacian of pair p of the row: y taps from the window (win[i] = row - R + i), x taps from the row, in
-// that order; each lane rounds as the scalar form would.
+// that order, added to acc; each lane rounds as the scalar form would.
 template <int R, bool DIFF, int NP>
 __device__ __forceinline__ float2 stencil_pair(const Cells<NP> (&win)[2 * R + 1], const Row<R, NP>& f, int p,
-                                               const float2 (&w2)[R + 1]) {
+                                               const float2 (&w2)[R + 1], float2 acc = make_float2(0.f, 0.f)) {
   const float2 c = win[R].v[p];
   const float2 nc = __fmul2_rn(c, dup2(-1.f));
-  float2 acc = dup2(0.f);
 #pragma unroll
   for (int m = 1; m <= R; ++m) acc = __ffma2_rn(w2[m], pair_term2<DIFF>(win[R + m].v[p], win[R - m].v[p], c, nc), acc);
 #pragma unroll

@@ -26,9 +26,15 @@
 // plain.
 //
 // GB300 mapping.  The grid is cut into 64 x 32 tiles, one CTA per tile, all
-// co-resident (cooperative launch).  Each thread keeps its 2 x 4 cells' state
-// in registers for the whole loop; the CTA keeps the current field plus an
-// R-deep halo in shared memory (double buffered).  After each step the
+// co-resident (cooperative launch).  Each of 512 threads keeps its 2 x 2 cells'
+// state in registers for the whole loop; the CTA keeps the current field plus
+// an R-deep halo in shared memory (double buffered).  Ten warps own the tile's
+// 8-cell frame, six its 48 x 16 interior, whose stencils (R <= 7) need no halo:
+// while the frame's warps wait for the neighbours' strips the interior is
+// computed, and while they compute the frame the interior's warps sample the
+// sensors.  (One step of 256 threads with 2 x 4 cells each, all of them behind
+// the halo: 2.69 us (K) and 3.22 us (K*) at 512^2, order 8, of which 1.3 and
+// 1.6 us are left with the 3-point stencil of order 2; now 2.38 and 2.99 us.)  After each step the
 // threads that own boundary cells write the R-deep strips straight to an
 // L2-resident exchange buffer (relaxed GPU-scope stores; 93.4 against 92.3
 // reconstruction iterations/s at 512^2 when they were staged in shared memory
@@ -42,6 +48,7 @@
 // always ends.
 #include "internal.h"
 #include "stencil.cuh"
+#include "tile2d.cuh"
 
 namespace pat {
 namespace {
@@ -50,11 +57,33 @@ using u64 = unsigned long long;
 
 constexpr int TX = 64;
 constexpr int TY = 32;
-constexpr int NTHREADS = (TX / 4) * (TY / 2);  // 256: each thread owns 2 rows x 4 columns
+constexpr int NTHREADS = (TX / 2) * (TY / 2);  // 512: each thread owns 2 rows x 2 columns
 constexpr int XOFF = 8;                         // left halo columns in shared memory (>= R, multiple of 4)
 constexpr int PITCH = TX + 16;                  // 8 halo columns each side
-constexpr int RCOUNT = NTHREADS / 4;            // threads serving one neighbour
-static_assert(NTHREADS % 128 == 0, "four halo regions need whole warps");
+constexpr int RCOUNT = 64;                      // threads serving one neighbour (warps 0 .. 7)
+constexpr int EDGE = 8;                         // frame depth (>= R, even)
+constexpr int NFRAME = (TX * 2 * EDGE + (TY - 2 * EDGE) * 2 * EDGE) / 4;  // 320: whole warps
+static_assert(EDGE >= kMaxR && NFRAME % 32 == 0 && NFRAME >= 4 * RCOUNT, "frame and interior are whole warps");
+
+// First cell (row, column) of thread t: the frame's top and bottom rows, then its side columns, then the interior.
+__device__ __forceinline__ void cells_of(int t, int& row, int& col) {
+  constexpr int BAND = EDGE * TX / 4;           // threads of the top (and of the bottom) rows
+  constexpr int SIDE = EDGE;                    // column pairs of the two sides in one row pair
+  constexpr int MID = (TX - 2 * EDGE) / 2;      // column pairs of the interior in one row pair
+  if (t < 2 * BAND) {
+    const int rp = t / (TX / 2);
+    row = 2 * (rp < EDGE / 2 ? rp : rp + (TY - 2 * EDGE) / 2);
+    col = 2 * (t % (TX / 2));
+  } else if (t < NFRAME) {
+    const int u = t - 2 * BAND, cp = u % SIDE;
+    row = EDGE + 2 * (u / SIDE);
+    col = 2 * (cp < SIDE / 2 ? cp : cp + MID);
+  } else {
+    const int u = t - NFRAME;
+    row = EDGE + 2 * (u / MID);
+    col = EDGE + 2 * (u % MID);
+  }
+}
 
 template <int R, bool ADJ>
 struct Geo {
@@ -107,38 +136,51 @@ __device__ __forceinline__ u64 ld_word(const u64* p) {
   return a;
 }
 
-// Write the thread's 2x4 block of the new state into the shared field
+// Write the thread's 2 x 2 block of the new state into the shared field
 // buffer(s) Sn (second field at Sn + SBUF) and, packed and tagged, its
 // boundary cells into the tile's exchange slot X in global memory, laid out
 // as the boundary strips [top R x TX][bottom R x TX][left TY x R][right TY x R].
 template <int R, bool ADJ>
-__device__ __forceinline__ void store_state(float* Sn, u64* X, const float V[2][4], const float Vl[2][4], int r0,
-                                            int c0, unsigned step) {
+__device__ __forceinline__ void store_state(float* Sn, u64* X, const float V[2][2], const float Vl[2][2], int r0,
+                                            int c0, unsigned step, bool frame) {
   constexpr int SBUF = Geo<R, ADJ>::SBUF;
 #pragma unroll
   for (int rr = 0; rr < 2; ++rr) {
     const int row = r0 + rr;
-    *reinterpret_cast<float4*>(Sn + (row + R) * PITCH + XOFF + c0) =
-        make_float4(V[rr][0], V[rr][1], V[rr][2], V[rr][3]);
-    if (ADJ)
-      *reinterpret_cast<float4*>(Sn + SBUF + (row + R) * PITCH + XOFF + c0) =
-          make_float4(Vl[rr][0], Vl[rr][1], Vl[rr][2], Vl[rr][3]);
-    u64 w[4];
+    *reinterpret_cast<float2*>(Sn + (row + R) * PITCH + XOFF + c0) = make_float2(V[rr][0], V[rr][1]);
+    if (ADJ) *reinterpret_cast<float2*>(Sn + SBUF + (row + R) * PITCH + XOFF + c0) = make_float2(Vl[rr][0], Vl[rr][1]);
+    if (!frame) continue;
+    u64 w[2];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] = pack<ADJ>(V[rr][j], Vl[rr][j], step);
+    for (int j = 0; j < 2; ++j) w[j] = pack<ADJ>(V[rr][j], Vl[rr][j], step);
     u64* dst = nullptr;
     if (row < R) dst = X + row * TX + c0;
     if (row >= TY - R) dst = X + R * TX + (row - (TY - R)) * TX + c0;
-    if (dst) {  // TY >= 2R: a row is in at most one of the two strips
-      st_word2(dst, w[0], w[1]);
-      st_word2(dst + 2, w[2], w[3]);
-    }
+    if (dst) st_word2(dst, w[0], w[1]);  // TY >= 2R: a row is in at most one of the two strips
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < 2; ++j) {
       const int col = c0 + j;
       if (col < R) st_word(X + 2 * R * TX + row * R + col, w[j]);
       if (col >= TX - R) st_word(X + 2 * R * TX + TY * R + row * R + (col - (TX - R)), w[j]);
     }
+  }
+}
+
+// Laplacian of the thread's 2 x 2 cells in a shared buffer (y taps, then x taps; pair or difference form), added
+// to L (ACC) or written to it.  `own` points at the thread's first cell.
+template <int R, bool DIFF, bool ACC>
+__device__ __forceinline__ void lap_2x2(const float* __restrict__ own, const float2 (&w2)[R + 1], float2 (&L)[2]) {
+  Cells<1> col[2 * R + 2];
+#pragma unroll
+  for (int i = 0; i < 2 * R + 2; ++i) col[i].load(own + (i - R) * PITCH);
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) {
+    Cells<1> win[2 * R + 1];
+#pragma unroll
+    for (int i = 0; i < 2 * R + 1; ++i) win[i] = col[rr + i];
+    Row<R, 1> f;
+    f.load(own + rr * PITCH, win[R]);
+    L[rr] = stencil_pair<R, DIFF, 1>(win, f, 0, w2, ACC ? L[rr] : dup2(0.f));
   }
 }
 
@@ -222,8 +264,9 @@ __device__ bool load_halo(float* const (&Sc)[NR], const u64* const (&X)[NR], int
 // solves of one medium): every step exchanges both fields' strips in the same round trip and runs both
 // updates between the same barriers.  Inputs / outputs of field r are a.in / a.out (r = 0) and a.in1 /
 // a.out1 (r = 1); field r's exchange words follow field 0's in each slot.
+// (Order 2 leaves room for two CTAs per SM, so its grids may have twice as many tiles as there are SMs.)
 template <int R, bool ADJ, bool VARC, bool SP, int NR>
-__global__ void __launch_bounds__(NTHREADS, 1) wave2d_persist_kernel(const Persist2DArgs a) {
+__global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_persist_kernel(const Persist2DArgs a) {
   using G = Geo<R, ADJ>;
   static_assert(NR == 1 || !SP, "several right-hand sides run without the absorbing layer");
   extern __shared__ float4 smem4[];
@@ -234,12 +277,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) wave2d_persist_kernel(const Persi
   const int t = threadIdx.x;
   const int lane = t & 31;
   const int warp = t >> 5;
+  const bool frame = t < NFRAME;
   const int tile = blockIdx.x;
   const int tix = tile % a.tiles_x;
   const int tiy = tile / a.tiles_x;
   const int gx0 = tix * TX, gy0 = tiy * TY;
-  const int c0 = (t % (TX / 4)) * 4;
-  const int r0 = (t / (TX / 4)) * 2;
+  int c0, r0;
+  cells_of(t, r0, c0);
   const int nx = a.nx, ny = a.ny, nt = a.nt;
   u64* xbuf = reinterpret_cast<u64*>(a.xbuf);
   float2 w2[R + 1];  // stencil weights, packed
@@ -249,24 +293,26 @@ __global__ void __launch_bounds__(NTHREADS, 1) wave2d_persist_kernel(const Persi
   float* OUT[2] = {a.out, a.out1};
   float* PART[2] = {a.part, a.part1};
 
-  // halo duty of this warp: 0 = north, 1 = south, 2 = west, 3 = east neighbour
+  // halo duty of warps 0 .. 7: 0 = north, 1 = south, 2 = west, 3 = east neighbour
   const int region = warp & 3;
   const int rrank = (warp >> 2) * 32 + lane;
   int nb = -1;
-  if (region == 0 && tiy > 0) nb = tile - a.tiles_x;
-  if (region == 1 && tiy < a.tiles_y - 1) nb = tile + a.tiles_x;
-  if (region == 2 && tix > 0) nb = tile - 1;
-  if (region == 3 && tix < a.tiles_x - 1) nb = tile + 1;
+  if (warp < 8) {
+    if (region == 0 && tiy > 0) nb = tile - a.tiles_x;
+    if (region == 1 && tiy < a.tiles_y - 1) nb = tile + a.tiles_x;
+    if (region == 2 && tix > 0) nb = tile - 1;
+    if (region == 3 && tix < a.tiles_x - 1) nb = tile + 1;
+  }
 
   // forward: P, D ; adjoint: Z (in P, with Z_lo in Pl), G (in D); per right-hand side
-  float P[NR][2][4], D[NR][2][4], Pl[NR][2][4];
-  float K[2][4], Kl[2][4];
-  float SA[2][4], SB[2][4];  // layer factors (SP only)
-  bool valid[2][4];
+  float P[NR][2][2], D[NR][2][2], Pl[NR][2][2];
+  float K[2][2], Kl[2][2];
+  float SA[2][2], SB[2][2];  // layer factors (SP only)
+  bool valid[2][2];
 #pragma unroll
   for (int rr = 0; rr < 2; ++rr)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < 2; ++j) {
       const int gx = gx0 + c0 + j, gy = gy0 + r0 + rr;
       const bool v = gx < nx && gy < ny;
       valid[rr][j] = v;
@@ -293,74 +339,75 @@ __global__ void __launch_bounds__(NTHREADS, 1) wave2d_persist_kernel(const Persi
   auto Xslot = [&](int tl, int slot, int r) { return xbuf + ((size_t)tl * 2 + slot) * NR * G::SLOT + r * G::SLOT; };
 #pragma unroll
   for (int r = 0; r < NR; ++r)  // publish state 0 (forward: x; adjoint: zero)
-    store_state<R, ADJ>(Sbuf(0, r), Xslot(tile, 0, r), P[r], Pl[r], r0, c0, 0u);
+    store_state<R, ADJ>(Sbuf(0, r), Xslot(tile, 0, r), P[r], Pl[r], r0, c0, 0u, frame);
 
-  for (int k = 0; k < nt; ++k) {
-    if (ADJ) {  // S^T r_n for this tile's injected cells, n = nt-1-k (independent of the halo: these
-                //  dependent loads overlap the neighbours' exchange)
-      const int n = nt - 1 - k;
-      const int e1 = a.tile_inj_ptr[tile + 1];
-      for (int e = a.tile_inj_ptr[tile] + t; e < e1; e += NTHREADS) {
-        const InjCell ic = a.inj[e];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          float s = 0.f;
-          for (int q = ic.beg; q < ic.end; ++q) s = fmaf(a.ent_w[q], IN[r][(long long)a.ent_sensor[q] * nt + n], s);
-          Jbuf(r, k & 1)[ic.local] = s;
-        }
+  // The interior's threads serve the tile's sensors.  Adjoint: S^T r_n, n = nt-1-k, of the injected cells into
+  // step k's accumulators (the first cell of a thread, with its first sensor, kept in registers).
+  const int ut = t - NFRAME;
+  constexpr int NINNER = NTHREADS - NFRAME;
+  int e0 = 0, e1 = 0, is0 = 0;
+  float iw0 = 0.f;
+  InjCell ic0{0, 0, 0};
+  if (!frame) {
+    const int* ptr = ADJ ? a.tile_inj_ptr : a.tile_samp_ptr;
+    e0 = ptr[tile] + ut;
+    e1 = ptr[tile + 1];
+    if (ADJ && e0 < e1) {
+      ic0 = a.inj[e0];
+      if (ic0.beg < ic0.end) {
+        is0 = a.ent_sensor[ic0.beg];
+        iw0 = a.ent_w[ic0.beg];
       }
     }
-    // ---- halo of state k from the neighbour's slot (k & 1)
-    if (nb >= 0) {
-      float* sc[NR];
-      const u64* xs[NR];
+  }
+  auto inject = [&](int k) {
+    const int n = nt - 1 - k;
+    for (int e = e0; e < e1; e += NINNER) {
+      const InjCell ic = e == e0 ? ic0 : a.inj[e];
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
-        sc[r] = Sbuf(k & 1, r);
-        xs[r] = Xslot(nb, k & 1, r);
-      }
-      if (!load_halo<R, ADJ, NR>(sc, xs, region, rrank, (unsigned)k, a.abort, a.timeout_ns, a.poll_ns)) {
-        if (lane == 0) {
-          s_abort = 1;
-          atomicCAS(a.status, (int)PAT_OK, (int)PAT_ERR_TIMEOUT);
-          atomicExch(a.abort, 1);
+        float s = 0.f;
+        for (int q = ic.beg; q < ic.end; ++q) {
+          const bool first = e == e0 && q == ic.beg;
+          const float w = first ? iw0 : a.ent_w[q];
+          s = fmaf(w, IN[r][(long long)(first ? is0 : a.ent_sensor[q]) * nt + n], s);
         }
+        Jbuf(r, k & 1)[ic.local] = s;
       }
     }
-    __syncthreads();
-    if (s_abort) break;
-
-    if (!ADJ) {  // y[:, k] = S P^k
-      const int e1 = a.tile_samp_ptr[tile + 1];
-      for (int e = a.tile_samp_ptr[tile] + t; e < e1; e += NTHREADS) {
-        const SampEntry se = a.samp[e];
+  };
+  auto sample = [&](int k) {  // y[:, k] = S P^k
+    for (int e = e0; e < e1; e += NINNER) {
+      const SampEntry se = a.samp[e];
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          const float* b = Sbuf(k & 1, r) + (se.ly + R) * PITCH + XOFF + se.lx;
-          if (se.part < 0) {
-            const float v = se.w[0] * b[0] + se.w[1] * b[1] + se.w[2] * b[PITCH] + se.w[3] * b[PITCH + 1];
-            OUT[r][(long long)se.sensor * nt + k] = v;
-          } else {
-            PART[r][(long long)se.part * nt + k] = se.w[0] * b[0];
-          }
+      for (int r = 0; r < NR; ++r) {
+        const float* b = Sbuf(k & 1, r) + (se.ly + R) * PITCH + XOFF + se.lx;
+        if (se.part < 0) {
+          const float v = se.w[0] * b[0] + se.w[1] * b[1] + se.w[2] * b[PITCH] + se.w[3] * b[PITCH + 1];
+          OUT[r][(long long)se.sensor * nt + k] = v;
+        } else {
+          PART[r][(long long)se.part * nt + k] = se.w[0] * b[0];
         }
       }
     }
-
+  };
+  // state k + 1 of the thread's cells (k = nt - 1: the adjoint's result)
+  auto update = [&](int k) {
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      const float* Sc = Sbuf(k & 1, r);
-      const float* Jc = Jbuf(r, k & 1);
-      float L[2][4];
-      lap_2x4_p<R, true, false>(Sc, PITCH, r0 + R, XOFF + c0, w2, L);
-      if (ADJ) lap_2x4_p<R, false, true>(Sc + G::SBUF, PITCH, r0 + R, XOFF + c0, w2, L);
+      const float* own = Sbuf(k & 1, r) + (r0 + R) * PITCH + XOFF + c0;
+      float2 L2[2];
+      lap_2x2<R, true, false>(own, w2, L2);
+      if (ADJ) lap_2x2<R, false, true>(own + G::SBUF, w2, L2);
+      const float L[2][2] = {{L2[0].x, L2[0].y}, {L2[1].x, L2[1].y}};
 
       if (k == nt - 1) {
         if (ADJ) {  // x = S^T r_0 + G^1 + 1/2 L Z^1
+          const float* Jc = Jbuf(r, k & 1);
 #pragma unroll
           for (int rr = 0; rr < 2; ++rr)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < 2; ++j) {
               if (!valid[rr][j]) continue;
               const int lr = r0 + rr, lc = c0 + j;
               float xv = Jc[lr * TX + lc] + D[r][rr][j] + 0.5f * L[rr][j];
@@ -372,13 +419,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) wave2d_persist_kernel(const Persi
         continue;
       }
 
-      float V[2][4], Vl[2][4];
+      float V[2][2], Vl[2][2];
       if (!ADJ) {
         const float cf = (k == 0) ? 0.5f : 1.0f;
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
+          for (int j = 0; j < 2; ++j) {
             // D += cf (kappa_hi + kappa_lo) L, the product rounded once before it meets D
             const float inc = fmaf(cf * K[rr][j], L[rr][j], (cf * Kl[rr][j]) * L[rr][j]);
             if (SP)
@@ -393,12 +440,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) wave2d_persist_kernel(const Persi
       } else {
         float* Jw = Jbuf(r, k & 1);
 #pragma unroll
-        for (int rr = 0; rr < 2; ++rr)
+        for (int rr = 0; rr < 2; ++rr) {
+          float2* jp = reinterpret_cast<float2*>(Jw + (r0 + rr) * TX + c0);
+          const float2 jv = *jp;
+          *jp = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int li = (r0 + rr) * TX + c0 + j;
-            const float inc = Jw[li] + L[rr][j];
-            Jw[li] = 0.f;
+          for (int j = 0; j < 2; ++j) {
+            const float inc = f2get(jv, j) + L[rr][j];
             float g = D[r][rr][j] + inc;                         // G += S^T r + L Z
             const float u = fmaf(K[rr][j], g, Kl[rr][j] * g);    // (kappa_hi + kappa_lo) G, rounded once
             float z, zl;
@@ -417,12 +465,45 @@ __global__ void __launch_bounds__(NTHREADS, 1) wave2d_persist_kernel(const Persi
             V[rr][j] = z;
             Vl[rr][j] = zl;
           }
+        }
       }
-      store_state<R, ADJ>(Sbuf((k + 1) & 1, r), Xslot(tile, (k + 1) & 1, r), V, Vl, r0, c0, (unsigned)(k + 1));
+      store_state<R, ADJ>(Sbuf((k + 1) & 1, r), Xslot(tile, (k + 1) & 1, r), V, Vl, r0, c0, (unsigned)(k + 1), frame);
     }
-    if (k == nt - 1) break;
-  }
+  };
 
+  if (ADJ) inject(0);
+  __syncthreads();  // state 0 and the first injections
+  for (int k = 0; k < nt; ++k) {
+    if (frame) {
+      if (nb >= 0) {  // halo of state k from the neighbour's slot (k & 1)
+        float* sc[NR];
+        const u64* xs[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          sc[r] = Sbuf(k & 1, r);
+          xs[r] = Xslot(nb, k & 1, r);
+        }
+        if (!load_halo<R, ADJ, NR>(sc, xs, region, rrank, (unsigned)k, a.abort, a.timeout_ns, a.poll_ns)) {
+          if (lane == 0) {
+            s_abort = 1;
+            atomicCAS(a.status, (int)PAT_OK, (int)PAT_ERR_TIMEOUT);
+            atomicExch(a.abort, 1);
+          }
+        }
+      }
+    } else {
+      update(k);
+      if (ADJ && k + 1 < nt) inject(k + 1);  // its accumulators were read and cleared during step k - 1
+    }
+    __syncthreads();  // the halo of state k
+    if (s_abort) break;
+    if (frame)
+      update(k);
+    else if (!ADJ)
+      sample(k);
+    if (k == nt - 1) break;
+    __syncthreads();  // state k + 1
+  }
 }
 
 __global__ void split_combine_kernel(const float* __restrict__ part, const int* __restrict__ split_sensor,
