@@ -35,7 +35,7 @@
 // sensors.  (One step of 256 threads with 2 x 4 cells each, all of them behind
 // the halo: 2.69 us (K) and 3.22 us (K*) at 512^2, order 8, of which 1.3 and
 // 1.6 us are left with the 3-point stencil of order 2; now 2.38 and 2.99 us.)  After each step the
-// threads that own boundary cells write the R-deep strips straight to an
+// threads that own boundary cells write their blocks straight to an
 // L2-resident exchange buffer (relaxed GPU-scope stores; 93.4 against 92.3
 // reconstruction iterations/s at 512^2 when they were staged in shared memory
 // and handed to the TMA engine), every value packed with the step it belongs
@@ -65,6 +65,14 @@ constexpr int EDGE = 8;                         // frame depth (>= R, even)
 constexpr int NFRAME = (TX * 2 * EDGE + (TY - 2 * EDGE) * 2 * EDGE) / 4;  // 320: whole warps
 static_assert(EDGE >= kMaxR && NFRAME % 32 == 0 && NFRAME >= 4 * RCOUNT, "frame and interior are whole warps");
 
+// Thread of the frame that owns row pair rp, column pair cp (the inverse of cells_of).
+__device__ __forceinline__ int frame_thread(int rp, int cp) {
+  constexpr int E2 = EDGE / 2, MIDR = (TY - 2 * EDGE) / 2, MID = (TX - 2 * EDGE) / 2;
+  if (rp < E2) return rp * (TX / 2) + cp;
+  if (rp >= E2 + MIDR) return (rp - MIDR) * (TX / 2) + cp;
+  return EDGE * TX / 2 + (rp - E2) * EDGE + (cp < E2 ? cp : cp - MID);
+}
+
 // First cell (row, column) of thread t: the frame's top and bottom rows, then its side columns, then the interior.
 __device__ __forceinline__ void cells_of(int t, int& row, int& col) {
   constexpr int BAND = EDGE * TX / 4;           // threads of the top (and of the bottom) rows
@@ -90,12 +98,14 @@ struct Geo {
   static constexpr int NF = ADJ ? 2 : 1;           // shared-memory fields: P, or (W_hi, W_lo)
   static constexpr int ROWS = TY + 2 * R;
   static constexpr int SBUF = ROWS * PITCH;        // one shared-memory field buffer
-  static constexpr int STRIP = 2 * R * (TX + TY);  // exchanged words per tile per slot
-  static constexpr int SLOT = STRIP;
-  static constexpr int NPAIR = R * TX / 2;         // word pairs of a north/south strip
-  static constexpr int NSIDE = TY * R;             // words of a west/east strip
-  static constexpr int PER_NS = (NPAIR + RCOUNT - 1) / RCOUNT;
-  static constexpr int PER_WE = (NSIDE + RCOUNT - 1) / RCOUNT;
+  // exchange: every frame thread within R cells of the edge (D = (R + 1) / 2 block rows or columns) publishes
+  // its 2 x 2 block as four consecutive words.  R = 1, where half of such a block is not needed: the tile's four
+  // edges as strips of words, [top TX][bottom TX][left TY][right TY] (512^2 order 2: K 1.21 us per step with
+  // strips, 1.23 with blocks; 64^2 0.81 and 0.89; 768 x 704, two CTAs per SM, 1.34 and 1.52).
+  static constexpr int D = (R + 1) / 2;
+  static constexpr int SLOT = 4 * NFRAME;          // words per tile, slot and right-hand side
+  static constexpr int PER = (D * TX / 2 + RCOUNT - 1) / RCOUNT;  // blocks a polling thread takes at most
+  static_assert(D * TY / 2 <= RCOUNT * PER, "west and east blocks fit as well");
 };
 
 // Exchange words.  The buffer is filled with 0xff bytes before every launch,
@@ -127,42 +137,49 @@ __device__ __forceinline__ void st_word2(u64* p, u64 a, u64 b) {
 __device__ __forceinline__ void st_word(u64* p, u64 a) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(a) : "memory");
 }
-__device__ __forceinline__ void ld_word2(const u64* p, u64& a, u64& b) {
-  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
-}
 __device__ __forceinline__ u64 ld_word(const u64* p) {
   u64 a;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(a) : "l"(p) : "memory");
   return a;
 }
+__device__ __forceinline__ void ld_word2(const u64* p, u64& a, u64& b) {
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
 
 // Write the thread's 2 x 2 block of the new state into the shared field
-// buffer(s) Sn (second field at Sn + SBUF) and, packed and tagged, its
-// boundary cells into the tile's exchange slot X in global memory, laid out
-// as the boundary strips [top R x TX][bottom R x TX][left TY x R][right TY x R].
+// buffer(s) Sn (second field at Sn + SBUF) and, packed and tagged, to X (its
+// block of the tile's exchange slot, for R = 1 the slot itself; nullptr for
+// blocks that no neighbour needs).  One 32-byte block per thread in thread order: two coalesced stores
+// and no case distinction, and a reader takes whole blocks (strips of exact
+// width cost up to eight predicated stores and as many 8-byte loads).
 template <int R, bool ADJ>
 __device__ __forceinline__ void store_state(float* Sn, u64* X, const float V[2][2], const float Vl[2][2], int r0,
-                                            int c0, unsigned step, bool frame) {
+                                            int c0, unsigned step) {
   constexpr int SBUF = Geo<R, ADJ>::SBUF;
+  if constexpr (R == 1) {
+    if (X) {
+      const u64 w[2][2] = {{pack<ADJ>(V[0][0], Vl[0][0], step), pack<ADJ>(V[0][1], Vl[0][1], step)},
+                           {pack<ADJ>(V[1][0], Vl[1][0], step), pack<ADJ>(V[1][1], Vl[1][1], step)}};
+      if (r0 == 0) st_word2(X + c0, w[0][0], w[0][1]);
+      if (r0 == TY - 2) st_word2(X + TX + c0, w[1][0], w[1][1]);
+      if (c0 == 0) {
+        st_word(X + 2 * TX + r0, w[0][0]);
+        st_word(X + 2 * TX + r0 + 1, w[1][0]);
+      }
+      if (c0 == TX - 2) {
+        st_word(X + 2 * TX + TY + r0, w[0][1]);
+        st_word(X + 2 * TX + TY + r0 + 1, w[1][1]);
+      }
+    }
+  } else if (X) {
+    st_word2(X, pack<ADJ>(V[0][0], Vl[0][0], step), pack<ADJ>(V[0][1], Vl[0][1], step));
+    st_word2(X + 2, pack<ADJ>(V[1][0], Vl[1][0], step), pack<ADJ>(V[1][1], Vl[1][1], step));
+  }
 #pragma unroll
   for (int rr = 0; rr < 2; ++rr) {
-    const int row = r0 + rr;
-    *reinterpret_cast<float2*>(Sn + (row + R) * PITCH + XOFF + c0) = make_float2(V[rr][0], V[rr][1]);
-    if (ADJ) *reinterpret_cast<float2*>(Sn + SBUF + (row + R) * PITCH + XOFF + c0) = make_float2(Vl[rr][0], Vl[rr][1]);
-    if (!frame) continue;
-    u64 w[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) w[j] = pack<ADJ>(V[rr][j], Vl[rr][j], step);
-    u64* dst = nullptr;
-    if (row < R) dst = X + row * TX + c0;
-    if (row >= TY - R) dst = X + R * TX + (row - (TY - R)) * TX + c0;
-    if (dst) st_word2(dst, w[0], w[1]);  // TY >= 2R: a row is in at most one of the two strips
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int col = c0 + j;
-      if (col < R) st_word(X + 2 * R * TX + row * R + col, w[j]);
-      if (col >= TX - R) st_word(X + 2 * R * TX + TY * R + row * R + (col - (TX - R)), w[j]);
-    }
+    *reinterpret_cast<float2*>(Sn + (r0 + rr + R) * PITCH + XOFF + c0) = make_float2(V[rr][0], V[rr][1]);
+    if (ADJ)
+      *reinterpret_cast<float2*>(Sn + SBUF + (r0 + rr + R) * PITCH + XOFF + c0) = make_float2(Vl[rr][0], Vl[rr][1]);
   }
 }
 
@@ -184,65 +201,118 @@ __device__ __forceinline__ void lap_2x2(const float* __restrict__ own, const flo
   }
 }
 
-// Copy the halo of state `step` of NR fields from the neighbour's strips X[r]
+// The blocks of a neighbour's frame that one polling thread copies: word offset in the neighbour's slot, float
+// offset of the block's first cell in the own shared buffer, and which of its two rows lie in the halo.
+template <int PER>
+struct HaloDuty {
+  int src[PER], dst[PER];
+  int rows[PER];  // bit 0: first row, bit 1: second; 0: no block
+};
+
+template <int R, bool ADJ>
+__device__ __forceinline__ HaloDuty<Geo<R, ADJ>::PER> halo_duty(int region, int rrank) {
+  using G = Geo<R, ADJ>;
+  HaloDuty<G::PER> h;
+#pragma unroll
+  for (int j = 0; j < G::PER; ++j) {
+    const int i = rrank + j * RCOUNT;
+    h.src[j] = h.dst[j] = h.rows[j] = 0;
+    if (R == 1) {  // north and south: a pair of words per thread; west and east: one word
+      if (i >= 32) continue;
+      h.src[j] = region == 0 ? TX + 2 * i : region == 1 ? 2 * i : region == 2 ? 2 * TX + TY + i : 2 * TX + i;
+      h.dst[j] = region == 0   ? XOFF + 2 * i
+                 : region == 1 ? (TY + 1) * PITCH + XOFF + 2 * i
+                 : region == 2 ? (i + 1) * PITCH + XOFF - 1
+                               : (i + 1) * PITCH + XOFF + TX;
+      h.rows[j] = region < 2 ? 1 : 2;  // kind
+      continue;
+    }
+    if (region < 2) {  // north: the neighbour's last D row pairs; south: its first D
+      if (i >= G::D * TX / 2) continue;
+      const int b = i / (TX / 2), cp = i % (TX / 2);
+      h.src[j] = 4 * frame_thread(region == 0 ? TY / 2 - G::D + b : b, cp);
+      h.dst[j] = (region == 0 ? R - 2 * G::D + 2 * b : R + TY + 2 * b) * PITCH + XOFF + 2 * cp;
+      // R is odd: the outermost block reaches one row beyond the halo
+      h.rows[j] = region == 0 ? (b == 0 ? 2 : 3) : (b == G::D - 1 ? 1 : 3);
+    } else {  // west: the neighbour's last D column pairs; east: its first D
+      if (i >= G::D * TY / 2) continue;
+      const int rp = i / G::D, g = i % G::D;
+      h.src[j] = 4 * frame_thread(rp, region == 2 ? TX / 2 - G::D + g : g);
+      h.dst[j] = (R + 2 * rp) * PITCH + (region == 2 ? XOFF - 2 * G::D : XOFF + TX) + 2 * g;
+      h.rows[j] = 3;
+    }
+  }
+  return h;
+}
+
+// Copy the halo of state `step` of NR fields from the neighbour's slots X[r]
 // into the shared buffers Sc[r] (second field at Sc[r] + SBUF).  Executed by
 // the RCOUNT threads of one region; returns false if the wait ran out.  Each
-// poll first issues the loads of every word still pending (all fields), then
+// poll first issues the loads of every block still pending (all fields), then
 // checks their tags, so the L2 round trips of one poll overlap instead of
 // following one another.
 template <int R, bool ADJ, int NR>
-__device__ bool load_halo(float* const (&Sc)[NR], const u64* const (&X)[NR], int region, int rrank, unsigned step,
-                          const int* abort, long long timeout_ns, int poll_ns) {
+__device__ __forceinline__ bool load_halo(float* const (&Sc)[NR], const u64* const (&X)[NR],
+                                          const HaloDuty<Geo<R, ADJ>::PER>& h, unsigned step, const int* abort,
+                                          long long timeout_ns, int poll_ns) {
   using G = Geo<R, ADJ>;
-  constexpr int PMAX = G::PER_NS > G::PER_WE ? G::PER_NS : G::PER_WE;
-  static_assert(NR * PMAX <= 32, "pending bits");
-  const bool ns = region < 2;
-  const int per = ns ? G::PER_NS : G::PER_WE;
-  const int count = ns ? G::NPAIR : G::NSIDE;
-  unsigned pending = 0;  // bit r * PMAX + j
+  static_assert(NR * G::PER <= 32, "pending bits");
+  unsigned pending = 0;  // bit r * PER + j
 #pragma unroll
   for (int r = 0; r < NR; ++r)
 #pragma unroll
-    for (int j = 0; j < PMAX; ++j)
-      if (j < per && rrank + j * RCOUNT < count) pending |= 1u << (r * PMAX + j);
+    for (int j = 0; j < G::PER; ++j)
+      if (h.rows[j]) pending |= 1u << (r * G::PER + j);
   unsigned long long t0 = 0;
   for (unsigned it = 0; it < (1u << 28); ++it) {
-    u64 wa[NR][PMAX], wb[NR][PMAX];
+    u64 w[NR][G::PER][4];
 #pragma unroll
     for (int r = 0; r < NR; ++r)
 #pragma unroll
-      for (int j = 0; j < PMAX; ++j) {
-        wa[r][j] = wb[r][j] = 0ull;
-        if (!(pending & (1u << (r * PMAX + j)))) continue;
-        const int i = rrank + j * RCOUNT;
-        if (ns)
-          ld_word2(X[r] + (region == 0 ? R * TX : 0) + 2 * i, wa[r][j], wb[r][j]);
-        else
-          wa[r][j] = ld_word(X[r] + 2 * R * TX + (region == 2 ? TY * R : 0) + i);
-      }
+      for (int j = 0; j < G::PER; ++j)
+        if (pending & (1u << (r * G::PER + j))) {
+          if constexpr (R == 1) {
+            if (h.rows[j] == 1)
+              ld_word2(X[r] + h.src[j], w[r][j][0], w[r][j][1]);
+            else
+              w[r][j][0] = w[r][j][1] = ld_word(X[r] + h.src[j]);
+          } else {
+            ld_word2(X[r] + h.src[j], w[r][j][0], w[r][j][1]);
+            ld_word2(X[r] + h.src[j] + 2, w[r][j][2], w[r][j][3]);
+          }
+        }
 #pragma unroll
     for (int r = 0; r < NR; ++r)
 #pragma unroll
-      for (int j = 0; j < PMAX; ++j) {
-        const unsigned bit = 1u << (r * PMAX + j);
+      for (int j = 0; j < G::PER; ++j) {
+        const unsigned bit = 1u << (r * G::PER + j);
         if (!(pending & bit)) continue;
-        const int i = rrank + j * RCOUNT;
-        if (ns) {
-          if (tag_ok<ADJ>(wa[r][j], step) && tag_ok<ADJ>(wb[r][j], step)) {
-            const int row = (2 * i) / TX, col = (2 * i) % TX;
-            const int o = (region == 0 ? row : TY + R + row) * PITCH + XOFF + col;
-            *reinterpret_cast<float2*>(Sc[r] + o) = make_float2(word_hi(wa[r][j]), word_hi(wb[r][j]));
-            if (ADJ) *reinterpret_cast<float2*>(Sc[r] + G::SBUF + o) = make_float2(word_lo(wa[r][j]), word_lo(wb[r][j]));
+        const u64* q = w[r][j];
+        if constexpr (R == 1) {
+          if (tag_ok<ADJ>(q[0], step) && tag_ok<ADJ>(q[1], step)) {
+            float* d = Sc[r] + h.dst[j];
+            if (h.rows[j] == 1) {
+              *reinterpret_cast<float2*>(d) = make_float2(word_hi(q[0]), word_hi(q[1]));
+              if (ADJ) *reinterpret_cast<float2*>(d + G::SBUF) = make_float2(word_lo(q[0]), word_lo(q[1]));
+            } else {
+              *d = word_hi(q[0]);
+              if (ADJ) d[G::SBUF] = word_lo(q[0]);
+            }
             pending &= ~bit;
           }
-        } else {
-          if (tag_ok<ADJ>(wa[r][j], step)) {
-            const int row = i / R, jj = i % R;
-            const int o = (row + R) * PITCH + (region == 2 ? XOFF - R + jj : XOFF + TX + jj);
-            Sc[r][o] = word_hi(wa[r][j]);
-            if (ADJ) Sc[r][G::SBUF + o] = word_lo(wa[r][j]);
-            pending &= ~bit;
-          }
+          continue;
+        }
+        if (tag_ok<ADJ>(q[0], step) && tag_ok<ADJ>(q[1], step) && tag_ok<ADJ>(q[2], step) && tag_ok<ADJ>(q[3], step)) {
+          float* d = Sc[r] + h.dst[j];
+#pragma unroll
+          for (int rr = 0; rr < 2; ++rr)
+            if (h.rows[j] & (1 << rr)) {
+              *reinterpret_cast<float2*>(d + rr * PITCH) = make_float2(word_hi(q[2 * rr]), word_hi(q[2 * rr + 1]));
+              if (ADJ)
+                *reinterpret_cast<float2*>(d + rr * PITCH + G::SBUF) =
+                    make_float2(word_lo(q[2 * rr]), word_lo(q[2 * rr + 1]));
+            }
+          pending &= ~bit;
         }
       }
     if (__all_sync(0xffffffffu, pending == 0)) return true;
@@ -337,12 +407,19 @@ __global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_pe
   auto Sbuf = [&](int slot, int r) { return S0 + (slot * NR + r) * G::NF * G::SBUF; };
   auto Jbuf = [&](int r, int slot) { return J0 + (r * 2 + slot) * TX * TY; };
   auto Xslot = [&](int tl, int slot, int r) { return xbuf + ((size_t)tl * 2 + slot) * NR * G::SLOT + r * G::SLOT; };
+  const HaloDuty<G::PER> duty = halo_duty<R, ADJ>(region, rrank);
+  // blocks within R cells of the tile's edge are published
+  const bool edge = r0 < R || r0 + 2 > TY - R || c0 < R || c0 + 2 > TX - R;
+  auto Xown = [&](int slot, int r) -> u64* {
+    return edge ? Xslot(tile, slot, r) + (R == 1 ? 0 : 4 * t) : nullptr;
+  };
 #pragma unroll
   for (int r = 0; r < NR; ++r)  // publish state 0 (forward: x; adjoint: zero)
-    store_state<R, ADJ>(Sbuf(0, r), Xslot(tile, 0, r), P[r], Pl[r], r0, c0, 0u, frame);
+    store_state<R, ADJ>(Sbuf(0, r), Xown(0, r), P[r], Pl[r], r0, c0, 0u);
 
   // The interior's threads serve the tile's sensors.  Adjoint: S^T r_n, n = nt-1-k, of the injected cells into
-  // step k's accumulators (the first cell of a thread, with its first sensor, kept in registers).
+  // step k's accumulators (KEEP: the first cell of a thread, with its first sensor, stays in registers).
+  constexpr bool KEEP = R > 1;
   const int ut = t - NFRAME;
   constexpr int NINNER = NTHREADS - NFRAME;
   int e0 = 0, e1 = 0, is0 = 0;
@@ -352,7 +429,7 @@ __global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_pe
     const int* ptr = ADJ ? a.tile_inj_ptr : a.tile_samp_ptr;
     e0 = ptr[tile] + ut;
     e1 = ptr[tile + 1];
-    if (ADJ && e0 < e1) {
+    if (ADJ && KEEP && e0 < e1) {
       ic0 = a.inj[e0];
       if (ic0.beg < ic0.end) {
         is0 = a.ent_sensor[ic0.beg];
@@ -363,12 +440,12 @@ __global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_pe
   auto inject = [&](int k) {
     const int n = nt - 1 - k;
     for (int e = e0; e < e1; e += NINNER) {
-      const InjCell ic = e == e0 ? ic0 : a.inj[e];
+      const InjCell ic = KEEP && e == e0 ? ic0 : a.inj[e];
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
         float s = 0.f;
         for (int q = ic.beg; q < ic.end; ++q) {
-          const bool first = e == e0 && q == ic.beg;
+          const bool first = KEEP && e == e0 && q == ic.beg;
           const float w = first ? iw0 : a.ent_w[q];
           s = fmaf(w, IN[r][(long long)(first ? is0 : a.ent_sensor[q]) * nt + n], s);
         }
@@ -467,30 +544,32 @@ __global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_pe
           }
         }
       }
-      store_state<R, ADJ>(Sbuf((k + 1) & 1, r), Xslot(tile, (k + 1) & 1, r), V, Vl, r0, c0, (unsigned)(k + 1), frame);
+      store_state<R, ADJ>(Sbuf((k + 1) & 1, r), Xown((k + 1) & 1, r), V, Vl, r0, c0, (unsigned)(k + 1));
     }
   };
 
-  if (ADJ) inject(0);
+  auto wait_halo = [&](int k) {  // halo of state k from the neighbour's slot (k & 1)
+    if (nb < 0) return;
+    float* sc[NR];
+    const u64* xs[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      sc[r] = Sbuf(k & 1, r);
+      xs[r] = Xslot(nb, k & 1, r);
+    }
+    if (!load_halo<R, ADJ, NR>(sc, xs, duty, (unsigned)k, a.abort, a.timeout_ns, a.poll_ns)) {
+      if (lane == 0) {
+        s_abort = 1;
+        atomicCAS(a.status, (int)PAT_OK, (int)PAT_ERR_TIMEOUT);
+        atomicExch(a.abort, 1);
+      }
+    }
+  };
+  if (ADJ && !frame) inject(0);
   __syncthreads();  // state 0 and the first injections
   for (int k = 0; k < nt; ++k) {
     if (frame) {
-      if (nb >= 0) {  // halo of state k from the neighbour's slot (k & 1)
-        float* sc[NR];
-        const u64* xs[NR];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          sc[r] = Sbuf(k & 1, r);
-          xs[r] = Xslot(nb, k & 1, r);
-        }
-        if (!load_halo<R, ADJ, NR>(sc, xs, region, rrank, (unsigned)k, a.abort, a.timeout_ns, a.poll_ns)) {
-          if (lane == 0) {
-            s_abort = 1;
-            atomicCAS(a.status, (int)PAT_OK, (int)PAT_ERR_TIMEOUT);
-            atomicExch(a.abort, 1);
-          }
-        }
-      }
+      wait_halo(k);
     } else {
       update(k);
       if (ADJ && k + 1 < nt) inject(k + 1);  // its accumulators were read and cleared during step k - 1
@@ -576,7 +655,7 @@ bool persist2d_supported(int R, bool) { return R == 1 || R == 3 || R == 5 || R =
 int persist2d_tile_x() { return TX; }
 int persist2d_tile_y() { return TY; }
 size_t persist2d_smem_bytes(int R, bool adj) { return smem_bytes(R, adj); }
-size_t persist2d_xbuf_words(int R, bool, int ntiles, int nr) { return (size_t)nr * ntiles * 2 * 2 * R * (TX + TY); }
+size_t persist2d_xbuf_words(int, bool, int ntiles, int nr) { return (size_t)nr * ntiles * 2 * 4 * NFRAME; }
 
 int persist2d_max_ctas(int R, bool adj, bool varc) {
   void* f = pick(R, adj, varc);
