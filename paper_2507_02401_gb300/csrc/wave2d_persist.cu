@@ -34,7 +34,7 @@
 // computed, and while they compute the frame the interior's warps sample the
 // sensors.  (One step of 256 threads with 2 x 4 cells each, all of them behind
 // the halo: 2.69 us (K) and 3.22 us (K*) at 512^2, order 8, of which 1.3 and
-// 1.6 us are left with the 3-point stencil of order 2; now 2.38 and 2.99 us.)  After each step the
+// 1.6 us are left with the 3-point stencil of order 2; now 1.75 and 2.44 us.)  After each step the
 // threads that own boundary cells write their blocks straight to an
 // L2-resident exchange buffer (relaxed GPU-scope stores; 93.4 against 92.3
 // reconstruction iterations/s at 512^2 when they were staged in shared memory
