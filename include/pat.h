@@ -333,8 +333,10 @@ pat_status pat_plan_check(pat_plan* plan, void* stream);
  * Wave engine of a plan (tuning and testing):
  *   PAT_PATH_AUTO        default choice (persistent when available)
  *   PAT_PATH_PERSISTENT  2D only: one cooperative launch per K / K* with the
- *                        wavefield kept on chip; available when every 64 x 32
- *                        tile of the grid can be resident at once
+ *                        wavefield kept on chip; available when every tile of
+ *                        the grid can be resident at once (tiles of 64 x 32
+ *                        cells, or of 128 x 64 where those beat a launch per
+ *                        step)
  *   PAT_PATH_STEP        one launch per time step (any grid; 3D always)
  * Both engines compute the same operators (to FP32 rounding).
  */

@@ -82,6 +82,9 @@ struct Persist2DArgs {
   int poll_ns;           // back-off between polls of the exchange (0 = spin)
   const float* sp_a;     // absorbing layer: per-cell factors a, b of the damped update (nullptr = none)
   const float* sp_b;
+  // 128 x 64 tiles only: floats from one row of kappa and the layer's factors to the next, and the layer's width
+  int pitch, sp_w;
+  float2 w2[kMaxR + 1];  // the stencil weights in pairs (128 x 64 tiles only)
   // second right-hand side (the two-field kernel only)
   const float* in1;
   float* out1;
@@ -162,6 +165,16 @@ int persist2d_max_ctas2(int R, bool adj, bool varc);
 cudaError_t persist2d_launch2(int R, bool adj, bool varc, const Persist2DArgs& a, int nctas, cudaStream_t st);
 // the same with the absorbing layer (a.sp_a, a.sp_b set)
 cudaError_t persist2d_launch_layer(int R, bool adj, bool varc, const Persist2DArgs& a, int nctas, cudaStream_t st);
+// the kernel with 128 x 64 tiles (wave2d_persist_large.cu); its injection lists are split into the tile's frame of
+// persist2dl_edge() cells and its interior (two list bounds per tile)
+int persist2dl_tile_x();
+int persist2dl_tile_y();
+int persist2dl_edge();
+size_t persist2dl_xbuf_words(int ntiles);
+int persist2dl_max_ctas(int R, bool adj, bool varc);  // with and without the layer; 0: no such kernel
+int persist2dl_min_tiles(int R, bool varc);  // worth it above this many 64 x 32 tiles per SM
+cudaError_t persist2dl_launch(int R, bool adj, bool varc, bool layer, const Persist2DArgs& a, int nctas,
+                              cudaStream_t st);
 cudaError_t persist2d_split_combine(const float* part, const int* split_sensor, int nsplit, int nt, float* y,
                                     cudaStream_t st);
 

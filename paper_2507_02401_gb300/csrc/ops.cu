@@ -37,6 +37,19 @@ static Persist2DArgs persist_args(pat_plan* p) {
     a.sp_a = p->d_sp_a;
     a.sp_b = p->d_sp_b;
   }
+  if (p->persist_large) {  // rows padded to 16 bytes
+    a.pitch = p->pitch;
+    a.sp_w = p->sponge_w;
+    for (int m = 0; m <= kMaxR; ++m) a.w2[m] = make_float2(p->w[m], p->w[m]);
+    if (p->varc) {
+      a.kappa = p->s_kappa;
+      a.kappa_lo = p->s_kappa_lo;
+    }
+    if (p->sponge_w > 0) {
+      a.sp_a = p->s_sp_a;
+      a.sp_b = p->s_sp_b;
+    }
+  }
   return a;
 }
 
@@ -45,7 +58,9 @@ static Persist2DArgs persist_args(pat_plan* p) {
 static pat_status persist_launch(pat_plan* p, bool adj, const Persist2DArgs& a, cudaStream_t st) {
   PAT_TRY_CUDA(cudaMemsetAsync(p->d_xbuf, 0xff, p->xbuf_bytes, st));
   PAT_TRY_CUDA(cudaMemsetAsync(p->d_abort, 0, sizeof(int), st));
-  if (p->sponge_w > 0)
+  if (p->persist_large)
+    PAT_TRY_CUDA(persist2dl_launch(p->R, adj, p->varc, p->sponge_w > 0, a, p->ntiles, st));
+  else if (p->sponge_w > 0)
     PAT_TRY_CUDA(persist2d_launch_layer(p->R, adj, p->varc, a, p->ntiles, st));
   else
     PAT_TRY_CUDA(persist2d_launch(p->R, adj, p->varc, a, p->ntiles, st));
@@ -834,7 +849,7 @@ static pat_status multi_setup(pat_plan* p, cudaStream_t st) {
   PAT_TRY_CUDA(cudaMemsetAsync(p->m2.counter, 0, sizeof(unsigned), st));
   PAT_TRY_CUDA(cudaMemsetAsync(p->m2.sc, 0, sizeof(CgScalars), st));
   p->m2.two_field = false;
-  if (p->path == PAT_PATH_PERSISTENT && p->sponge_w == 0 &&
+  if (p->path == PAT_PATH_PERSISTENT && !p->persist_large && p->sponge_w == 0 &&
       persist2d_max_ctas2(p->R, false, p->varc) >= p->ntiles && persist2d_max_ctas2(p->R, true, p->varc) >= p->ntiles) {
     PAT_TRY(fl(&p->m2.part, (size_t)4 * p->nsplit * p->nt, "split sensor parts (second)"));
     p->m2.xbuf_bytes = persist2d_xbuf_words(p->R, true, p->ntiles, 2) * 8;

@@ -177,7 +177,8 @@ static pat_status pitched(pat_plan* p, float* dense, float** out, const char* wh
 
 // --------------------------------------------------- persistent 2D set-up
 static pat_status setup_persistent(pat_plan* p, cudaStream_t st) {
-  const int TX = persist2d_tile_x(), TY = persist2d_tile_y();
+  const bool large = p->persist_large;
+  const int TX = large ? persist2dl_tile_x() : persist2d_tile_x(), TY = large ? persist2dl_tile_y() : persist2d_tile_y();
   p->tiles_x = (p->n[0] + TX - 1) / TX;
   p->tiles_y = (p->n[1] + TY - 1) / TY;
   p->ntiles = p->tiles_x * p->tiles_y;
@@ -228,8 +229,9 @@ static pat_status setup_persistent(pat_plan* p, cudaStream_t st) {
   }
   samp_ptr[p->ntiles] = (int)samp.size();
 
-  // injected cells grouped by tile
-  std::vector<std::vector<InjCell>> inj_tile(p->ntiles);
+  // injected cells grouped by tile (large tiles: frame, then interior)
+  const int nlist = large ? 2 : 1, edge = persist2dl_edge();
+  std::vector<std::vector<InjCell>> inj_tile((size_t)nlist * p->ntiles);
   for (int i = 0; i < p->n_inj; ++i) {
     const int c = p->h_inj_cell[i];
     const int cx = c % nx, cy = c / nx;
@@ -238,22 +240,23 @@ static pat_status setup_persistent(pat_plan* p, cudaStream_t st) {
     ic.local = (cy % TY) * TX + (cx % TX);
     ic.beg = p->h_inj_ptr[i];
     ic.end = p->h_inj_ptr[i + 1];
-    inj_tile[tile].push_back(ic);
+    const int lx = cx % TX, ly = cy % TY;
+    const bool inner = lx >= edge && lx < TX - edge && ly >= edge && ly < TY - edge;
+    inj_tile[(size_t)nlist * tile + (large && inner ? 1 : 0)].push_back(ic);
   }
-  std::vector<int> inj_ptr(p->ntiles + 1, 0);
+  std::vector<int> inj_ptr(1, 0);
   std::vector<InjCell> inj;
-  for (int t = 0; t < p->ntiles; ++t) {
-    inj_ptr[t] = (int)inj.size();
-    inj.insert(inj.end(), inj_tile[t].begin(), inj_tile[t].end());
+  for (const auto& cells : inj_tile) {
+    inj.insert(inj.end(), cells.begin(), cells.end());
+    inj_ptr.push_back((int)inj.size());
   }
-  inj_ptr[p->ntiles] = (int)inj.size();
 
   PAT_TRY(upload(p, &p->d_tile_samp_ptr, samp_ptr, "tile sampling offsets", st));
   PAT_TRY(upload(p, &p->d_samp, samp, "tile sampling entries", st));
   PAT_TRY(upload(p, &p->d_tile_inj_ptr, inj_ptr, "tile injection offsets", st));
   PAT_TRY(upload(p, &p->d_tinj, inj, "tile injection cells", st));
   // tagged exchange words, invalidated (0xff bytes) before every launch
-  p->xbuf_bytes = persist2d_xbuf_words(p->R, true, p->ntiles) * 8;
+  p->xbuf_bytes = (large ? persist2dl_xbuf_words(p->ntiles) : persist2d_xbuf_words(p->R, true, p->ntiles)) * 8;
   PAT_TRY(plan_alloc(p, &p->d_xbuf, p->xbuf_bytes, "exchange strips"));
   if (const char* e = getenv("PAT_POLL_NS")) p->poll_ns = std::max(0, atoi(e));
   PAT_TRY(alloc_n(p, &p->d_abort, 1, "abort flag"));
@@ -497,13 +500,20 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
   // ---- engine choice: the persistent kernel when all tiles can be co-resident
   p->persist_ok = false;
   if (p->dim == 2 && persist2d_supported(p->R, p->varc)) {
-    const int TX = persist2d_tile_x(), TY = persist2d_tile_y();
-    const int ntiles = ((p->n[0] + TX - 1) / TX) * ((p->n[1] + TY - 1) / TY);
-    const int cap = std::min(persist2d_max_ctas(p->R, false, p->varc), persist2d_max_ctas(p->R, true, p->varc));
-    if (ntiles <= cap) {
-      PAT_TRY(setup_persistent(p, st));
-      p->persist_ok = true;
+    auto tiles = [&](int TX, int TY) { return (long long)((p->n[0] + TX - 1) / TX) * ((p->n[1] + TY - 1) / TY); };
+    p->persist_ok = tiles(persist2d_tile_x(), persist2d_tile_y()) <=
+                    std::min(persist2d_max_ctas(p->R, false, p->varc), persist2d_max_ctas(p->R, true, p->varc));
+    // grids with too many 64 x 32 tiles: 128 x 64 tiles, whose kernel reads kappa and the layer's factors in pairs
+    if (!p->persist_ok && p->pitch % 2 == 0) {
+      const int cap = std::min(persist2dl_max_ctas(p->R, false, p->varc), persist2dl_max_ctas(p->R, true, p->varc));
+      int TX, TY, dev = 0, sms = 0;
+      tma2d_tile(&TX, &TY);
+      PAT_TRY_CUDA(cudaGetDevice(&dev));
+      PAT_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+      p->persist_ok = p->persist_large = tiles(persist2dl_tile_x(), persist2dl_tile_y()) <= cap &&
+                                         tiles(TX, TY) > (long long)persist2dl_min_tiles(p->R, p->varc) * sms;
     }
+    if (p->persist_ok) PAT_TRY(setup_persistent(p, st));
   }
   p->path = p->persist_ok ? PAT_PATH_PERSISTENT : PAT_PATH_STEP;
   const char* env_path = getenv("PAT_WAVE_PATH");

@@ -43,6 +43,7 @@ struct pat_plan {
   // ---- wave engine
   int path = PAT_PATH_STEP;       // engine in use
   bool persist_ok = false;        // persistent engine available for this plan
+  bool persist_large = false;     // the persistent engine runs 128 x 64 tiles (64 x 32 otherwise)
   int tiles_x = 0, tiles_y = 0, ntiles = 0;
   int* d_tile_samp_ptr = nullptr;
   pat::SampEntry* d_samp = nullptr;

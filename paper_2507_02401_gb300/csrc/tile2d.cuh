@@ -140,7 +140,20 @@ __device__ __forceinline__ float2 stencil_pair(const Cells<NP> (&win)[2 * R + 1]
   return acc;
 }
 
-// The low part's stencil of the thread's RUN rows (box pitch BW): lo[rr], centre weight -nwc.
+// The low part's stencil of pair p of the row, centre weight -nwc.
+template <int R, int NP>
+__device__ __forceinline__ float2 stencil_low(const Cells<NP> (&win)[2 * R + 1], const Row<R, NP>& f, int p,
+                                              const float2 (&w2)[R + 1], float2 nwc) {
+  float2 acc = __fmul2_rn(nwc, win[R].v[p]);
+#pragma unroll
+  for (int m = 1; m <= R; ++m) acc = __ffma2_rn(w2[m], __fadd2_rn(win[R + m].v[p], win[R - m].v[p]), acc);
+#pragma unroll
+  for (int m = 1; m <= R; ++m)
+    acc = __ffma2_rn(w2[m], add_pair(f.pair(2 * p + m), f.pair(2 * p - m), m % 2 == 0), acc);
+  return acc;
+}
+
+// The low part's stencil of the thread's RUN rows (box pitch BW): lo[rr].
 template <int R, int RUN, int BW, int NP>
 __device__ __forceinline__ void stencil_run_pair(const float* __restrict__ own, const float2 (&w2)[R + 1], float2 nwc,
                                                  Cells<NP> (&lo)[RUN]) {
@@ -153,15 +166,7 @@ __device__ __forceinline__ void stencil_run_pair(const float* __restrict__ own, 
     Row<R, NP> f;
     f.load(own + rr * BW, win[R]);
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      float2 acc = __fmul2_rn(nwc, win[R].v[p]);
-#pragma unroll
-      for (int m = 1; m <= R; ++m) acc = __ffma2_rn(w2[m], __fadd2_rn(win[R + m].v[p], win[R - m].v[p]), acc);
-#pragma unroll
-      for (int m = 1; m <= R; ++m)
-        acc = __ffma2_rn(w2[m], add_pair(f.pair(2 * p + m), f.pair(2 * p - m), m % 2 == 0), acc);
-      lo[rr].v[p] = acc;
-    }
+    for (int p = 0; p < NP; ++p) lo[rr].v[p] = stencil_low<R, NP>(win, f, p, w2, nwc);
 #pragma unroll
     for (int i = 0; i < 2 * R; ++i) win[i] = win[i + 1];
   }
