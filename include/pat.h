@@ -314,8 +314,9 @@ pat_status pat_batch_launch(pat_batch* batch, int mode, int* runall, double* ms)
  * P^{n+1} = 2P^n - P^{n-1} + kappa .* L P^n and adjoint states Q^n of K*r:
  *   g = sum_{n=1}^{nt-2} Q^{n+1} .* L P^n + 1/2 Q^1 .* L P^0.
  * The forward fields are needed in reverse order: the forward run keeps its
- * restart state every `segment` steps (0 = ceil(sqrt(nt))) and each segment is
- * recomputed when the adjoint reaches it.  Runs on the per-step engine.
+ * restart state every `segment` steps (0 = ceil(sqrt(nt)), in 2D as many more
+ * as 1 GiB of segment memory holds where that is free) and each segment but the
+ * last is recomputed when the adjoint reaches it.  Runs on the per-step engine.
  *   x  N floats;  r  ns*nt floats;  g  N floats (output).
  * Memory: (2 ceil((nt-1)/segment) + segment + 3) N floats + N doubles,
  * allocated by the first call and kept by the plan (PAT_ERR_OOM if absent).

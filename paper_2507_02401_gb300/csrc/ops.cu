@@ -549,10 +549,10 @@ static pat_status kg_alloc(pat_plan* p, int C, int nseg) {
 }
 
 // The 2D TMA engine's run of the gradient: a segment keeps L P^n (which the forward step has at hand) instead
-// of P^n, and each adjoint step adds its own term, so a time step costs two forward steps and one adjoint
-// step and no pass of its own over the gradient.  The sums live in the FP64 accumulator's buffer, as FP32
-// pairs.  (384^2 order 8: 20 us per time step when every term was a launch that recomputed L P and divided by
-// kappa in FP64, 11 us so.)
+// of P^n, and each adjoint step adds its own term, so a time step costs one forward step, or two where its segment
+// is recomputed, one adjoint step and no pass of its own over the gradient.  The sums live in the FP64 accumulator's
+// buffer, as FP32 pairs.  (384^2 order 8: 35 us per time step when every term was a launch that recomputed L P and
+// divided by kappa in FP64, 10 us with every segment recomputed, 7.4 us with the record kept.)
 static pat_status kappa_grad_tma2d(pat_plan* p, const float* x, const float* r, float* g, int C, cudaStream_t st) {
   const long long N = p->Np;  // floats of a field
   const int nt = p->nt, last = (nt - 2) / C;  // segments 0 .. last of n = 0 .. nt-2
@@ -636,10 +636,21 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
     PAT_TRY_CUDA(fill_launch(g, p->N, 0.f, st));
     return PAT_OK;
   }
-  if (C <= 0) C = (int)std::ceil(std::sqrt((double)nt));
+  // Default segment: sqrt(nt) steps.  The 2D TMA run keeps the last segment in passing and recomputes the others, so
+  // there it is as long as 1 GiB holds: with the whole record kept (384^2, 700 steps: 0.4 GiB) a time step costs one
+  // forward step instead of two (384^2 order 8: 10.1 -> 7.4 us per time step).  Without that memory, sqrt(nt).
+  const int root = std::min((int)std::ceil(std::sqrt((double)nt)), nt - 1);
+  const bool longer = C <= 0 && p->tma2d;
+  if (C <= 0) C = longer ? (int)std::max<long long>(root, (1LL << 28) / N) : root;
   if (C > nt - 1) C = nt - 1;
-  const int nseg = (nt - 2) / C + 1;  // segments of n = 0 .. nt-2
-  PAT_TRY(kg_alloc(p, C, nseg));
+  if (longer) C = (nt - 2) / ((nt - 2) / C + 1) + 1;  // equal segments: the last, kept one is as long as the others
+  auto segments = [&] { return (nt - 2) / C + 1; };  // of n = 0 .. nt-2
+  pat_status rc = kg_alloc(p, C, segments());
+  if (rc != PAT_OK && longer && C > root) {
+    C = root;
+    rc = kg_alloc(p, C, segments());
+  }
+  PAT_TRY(rc);
   const bool two_d = p->dim == 2;
   float* W0 = p->kg_work;
   float* W1 = p->kg_work + N;
