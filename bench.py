@@ -65,7 +65,7 @@ WORKLOADS = {
                  "s in {1,2} x alpha in {1e-3,1e-2}, 100 CG iterations, FP32 fields + FP64 CG scalars"),
         "kernel": "wave2d_persist_kernel<R=7,varc>",
         "profile": "wave2d_persist_512_o8.txt",
-        "sources": ("wave2d_persist.cu", "stencil.cuh"),
+        "sources": ("wave2d_persist.cu", "persist2d.cuh", "tile2d.cuh", "stencil.cuh"),
         "oracle_nt": None,
     },
     "tree3d": {
@@ -84,7 +84,7 @@ WORKLOADS = {
                  "alpha = 1e-2 (relative), 15 GMRES iterations on the paper's image-space system"),
         "kernel": "wave2d_persist_kernel<R=7> with the absorbing layer",
         "profile": "wave2d_persist_512_o8_layer.txt",
-        "sources": ("wave2d_persist.cu", "stencil.cuh"),
+        "sources": ("wave2d_persist.cu", "persist2d.cuh", "tile2d.cuh", "stencil.cuh"),
         "oracle_nt": 40,
     },
 }

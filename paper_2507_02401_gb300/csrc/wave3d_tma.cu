@@ -128,6 +128,23 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
     for (int s = 0; s < G::NS + G::NSP; ++s) mbar_init(&bars[s], 1);
     fence_mbar_init();
   }
+  // The CTA's injected cells (thread t takes entries t and t + THREADS; 256^3 with 4096 sensors has up to 302 in a
+  // CTA).  The chain list bounds -> cell -> sensor -> r_m is walked where the thread waits anyway (the previous step's
+  // end, the first copies, the first planes) and not in the march, whose instructions are the bound; what is left
+  // after it is two additions per thread (and the entries beyond those, or beyond a cell's first sensor).  us per K*
+  // step at 256^3, one entry walked link by link in the march -> this: order 2 30.6 -> 28.9, order 4 39.5 -> 38.0,
+  // order 6 58.1 -> 54.6, order 8 79.3 -> 76.3.  The lists are the plan's: they may be read before the wait.
+  constexpr int NPRE = R == 1 && VARC ? 1 : 2;  // a second one there costs the sixth CTA per SM (94 registers)
+  int ie0 = 0, ie1 = 0, is[NPRE] = {};
+  InjCell ic[NPRE] = {};
+  float iw[NPRE] = {}, ir[NPRE] = {};
+  if (INJ) {
+    ie0 = a.inj_tile_ptr[bid] + t;
+    ie1 = a.inj_tile_ptr[bid + 1];
+#pragma unroll
+    for (int j = 0; j < NPRE; ++j)
+      if (ie0 + j * THREADS < ie1) ic[j] = a.inj_tile[ie0 + j * THREADS];
+  }
   __syncthreads();
   griddep_wait();  // everything above overlaps the previous step's last CTAs
   griddep_trigger();
@@ -150,27 +167,12 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   }
   fused_sample3(a, bid, t);  // the forward's sensor samples of cur, while the first copies are in flight
 
-  // The CTA's injected cells (thread t takes entry t): the chain list bounds -> cell -> sensor -> r_m is
-  // walked one load per plane of the march, so that no load is waited for; what is left after the march is
-  // one addition per thread (and the entries beyond the first THREADS, or beyond a cell's first sensor).
-  int ie0 = 0, ie1 = 0, is = 0;
-  InjCell ic{0, 0, 0};
-  float iw = 0.f, ir = 0.f;
-  auto inj_prefetch = [&](int i) {
-    if (i == 0) {
-      ie0 = a.inj_tile_ptr[bid] + t;
-      ie1 = a.inj_tile_ptr[bid + 1];
-    } else if (i == 1) {
-      if (ie0 < ie1) ic = a.inj_tile[ie0];
-    } else if (i == 2) {
-      if (ic.beg < ic.end) {
-        is = a.ent_sensor[ic.beg];
-        iw = a.ent_w[ic.beg];
-      }
-    } else if (i == 3) {
-      if (ic.beg < ic.end) ir = a.inj_r[(long long)is * a.nt + a.inj_t];
+#pragma unroll
+  for (int j = 0; j < NPRE; ++j)
+    if (INJ && ic[j].beg < ic[j].end) {
+      is[j] = a.ent_sensor[ic[j].beg];
+      iw[j] = a.ent_w[ic[j].beg];
     }
-  };
 
   // register ring of the own cells: at the first plane q[k] = plane zb + (k - R) zd
   float4 q[2 * R + 1][2];
@@ -207,6 +209,10 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
       q[R + i][rr] = *reinterpret_cast<const float4*>(ring + (i % G::NS) * G::PLANE + (r0 + rr + R) * BW + XH + c0);
   }
 
+#pragma unroll
+  for (int j = 0; j < NPRE; ++j)
+    if (INJ && ic[j].beg < ic[j].end) ir[j] = a.inj_r[(long long)is[j] * a.nt + a.inj_t];
+
   // One plane of the march.  RING: the z queue is a ring in registers, logical entry k (plane z - R + k)
   // of plane i sitting in q[(k + i) % Q]; the loop is unrolled Q times, so S = i % Q is a compile-time
   // constant in every copy and no queue entry moves between registers (fewer instructions, a Q times
@@ -233,7 +239,6 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
       q[(2 * R + S) % Q][rr] =
           *reinterpret_cast<const float4*>(ring + (jq % G::NS) * G::PLANE + (r0 + rr + R) * BW + XH + c0);
 
-    if (INJ) inj_prefetch(i);
     const float* cen = ring + (i % G::NS) * G::PLANE;
     float2 L[2][2];  // packed pairs: cells (2p, 2p+1) of row rr
     lap_2x4_x2<R>(cen, BW, r0 + R, XH + c0, w2, L);
@@ -295,15 +300,16 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
   }
   if (INJ && ok_all) {  // every thread's stores to `next` precede the injection (same CTA)
     __syncthreads();
-    for (int i = nloc; i < 4; ++i) inj_prefetch(i);  // short marches
     auto scale = [&](const InjCell& c) { return VARC && !a.final_step ? a.kappa[c.local] : 1.f; };
-    if (ie0 < ie1) {
-      float v = ic.beg < ic.end ? iw * ir : 0.f;
-      for (int q = ic.beg + 1; q < ic.end; ++q)
-        v = fmaf(a.ent_w[q], a.inj_r[(long long)a.ent_sensor[q] * a.nt + a.inj_t], v);
-      a.next[ic.local] += scale(ic) * v;
-    }
-    for (int e = ie0 + THREADS; e < ie1; e += THREADS)
+#pragma unroll
+    for (int j = 0; j < NPRE; ++j)
+      if (ie0 + j * THREADS < ie1) {
+        float v = iw[j] * ir[j];
+        for (int q = ic[j].beg + 1; q < ic[j].end; ++q)
+          v = fmaf(a.ent_w[q], a.inj_r[(long long)a.ent_sensor[q] * a.nt + a.inj_t], v);
+        a.next[ic[j].local] += scale(ic[j]) * v;
+      }
+    for (int e = ie0 + NPRE * THREADS; e < ie1; e += THREADS)
       a.next[a.inj_tile[e].local] += scale(a.inj_tile[e]) * inj_sum(a, a.inj_tile[e]);
   }
   // after a timed-out wait: give the copies still in flight (the last one of
