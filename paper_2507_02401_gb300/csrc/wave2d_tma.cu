@@ -155,7 +155,9 @@ __global__ void __launch_bounds__(THREADS, min_ctas(R, FULL, GRAD)) step2d_tma_k
     // own-cell fields straight into registers, in flight while the boxes land: D or G of every row; kappa
     // and G_lo (fetch) two rows ahead of their use
     Cells<NP> d2[RUN], kh2[RUN], kl2[RUN], gl2[RUN], lp2[RUN], sh2[RUN], sl2[RUN];
-    const bool need_k = VARC || (ADJ && kv && !a.final_step);
+    // (the adjoint's final step takes kappa inside the layer; a partial tile has cells beyond the field, so every
+    // access to a field by cell is under a test like fetch's)
+    const bool need_k = VARC || (ADJ && kv && (SP || !a.final_step));
     auto fetch = [&](int rr) {
       const int gy = gy0 + r0 + rr;
       const long long gi = (long long)gy * pitch + gx;
@@ -251,10 +253,8 @@ __global__ void __launch_bounds__(THREADS, min_ctas(R, FULL, GRAD)) step2d_tma_k
             gn[j] = gl;
             if (a.final_step) {
               pn[j] = g;
-              if (LAYER) {  // x = G' + ((a-1)/b) Q,  Q = (Z + Z_lo) / kappa
-                const float kq = kv ? a.kappa[gi + j] : a.kappa0;
-                if (in && fa != 1.f) pn[j] = fmaf((fa - 1.f) / fb, (c + zl) / kq, g);
-              }
+              if (LAYER && in && fa != 1.f)  // x = G' + ((a-1)/b) Q,  Q = (Z + Z_lo) / kappa
+                pn[j] = fmaf((fa - 1.f) / fb, (c + zl) / kap, g);
               pl[j] = 0.f;
             } else {
               float u, ul = 0.f;  // kappa G', and what its rounding dropped (FULL)
