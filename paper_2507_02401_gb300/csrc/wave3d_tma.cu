@@ -174,7 +174,9 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
       iw[j] = a.ent_w[ic[j].beg];
     }
 
-  // register ring of the own cells: at the first plane q[k] = plane zb + (k - R) zd
+  // register ring of the own cells: at the first plane q[k] = plane zb + (k - R) zd.  Not through the read-only
+  // path (__ldg): it is for data that no one writes while the kernel lives, and this kernel starts while the
+  // previous step still writes `cur`.
   float4 q[2 * R + 1][2];
 #pragma unroll
   for (int i = 0; i < R; ++i)  // the R planes before zb straight from global memory
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(THREADS) step3d_tma_kernel(const StepArgs a, c
     for (int rr = 0; rr < 2; ++rr) {
       const int z = zb + (i - R) * zd, gy = gy0 + r0 + rr, gx = gx0 + c0;
       q[i][rr] = (z >= 0 && z < nz && gy < ny && gx < nx)
-                     ? __ldg(reinterpret_cast<const float4*>(a.cur + z * plane + (long long)gy * pitch + gx))
+                     ? ld_stream4(a.cur + z * plane + (long long)gy * pitch + gx)
                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   // varying medium: the own cells' kappa, one plane ahead of its use

@@ -24,3 +24,21 @@ def test_step2d_tma_reads_cells_only_under_a_bounds_test():
     # the injection's and the sensors' lists hold cells of the field
     assert re.findall(r"a\.dbuf\s*\[([^\]]*)\]", text) == ["c.local"]
     assert re.findall(r"a\.cur\s*\[(\S+?)\[", text) == ["a.sens_cell"]
+
+
+def test_programmatic_kernels_read_only_path_takes_plan_constants():
+    """A kernel launched programmatically starts while the previous grid of its
+    stream still writes.  The read-only path (ld.global.nc, __ldg) is defined
+    only for data that stay unwritten for the kernel's whole life, so there it
+    may serve a plan's constants, never a field of the recurrence."""
+    constants = r"a\.(kappa|kappa_lo|sp_a|sp_b|active_dev)\b|I\.(kappa|kappa_lo)\b|^p( \+ 1)?$"  # p: the tile table
+    seen = 0
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith(".cu") or "griddep_wait()" not in source(name):
+            continue
+        text = source(name)
+        assert "ld.global.nc" not in text
+        for m in re.finditer(r"(?:__ldg|\.ldg)\(((?:[^()]|\((?:[^()]|\([^()]*\))*\))*)\)", text):
+            seen += 1
+            assert re.search(constants, m.group(1)), (name, m.group(0))
+    assert seen >= 8
