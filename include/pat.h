@@ -320,6 +320,8 @@ pat_status pat_batch_launch(pat_batch* batch, int mode, int* runall, double* ms)
  *   x  N floats;  r  ns*nt floats;  g  N floats (output).
  * Memory: (2 ceil((nt-1)/segment) + segment + 3) N floats + N doubles,
  * allocated by the first call and kept by the plan (PAT_ERR_OOM if absent).
+ * The segment granted to the first call with 0 is the one of every later such
+ * call: these allocate nothing and may be captured.
  */
 pat_status pat_grad_kappa(pat_plan* plan, const float* x, const float* r, float* g, int segment, void* stream);
 

@@ -638,18 +638,27 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
   }
   // Default segment: sqrt(nt) steps.  The 2D TMA run keeps the last segment in passing and recomputes the others, so
   // there it is as long as 1 GiB holds: with the whole record kept (384^2, 700 steps: 0.4 GiB) a time step costs one
-  // forward step instead of two (384^2 order 8: 10.1 -> 7.4 us per time step).  Without that memory, sqrt(nt).
+  // forward step instead of two (384^2 order 8: 10.1 -> 7.4 us per time step).  Without that memory, sqrt(nt).  What
+  // was granted is the plan's default from then on, so that later calls find their buffers.
   const int root = std::min((int)std::ceil(std::sqrt((double)nt)), nt - 1);
-  const bool longer = C <= 0 && p->tma2d;
-  if (C <= 0) C = longer ? (int)std::max<long long>(root, (1LL << 28) / N) : root;
+  const bool by_default = C <= 0;
+  if (by_default && p->kg_default > 0) {
+    C = p->kg_default;
+  } else if (by_default) {
+    C = root;
+    if (p->tma2d) {
+      C = (int)std::min<long long>(nt - 1, std::max<long long>(root, (1LL << 28) / N));
+      C = (nt - 2) / ((nt - 2) / C + 1) + 1;  // equal segments: the last, kept one is as long as the others
+    }
+  }
   if (C > nt - 1) C = nt - 1;
-  if (longer) C = (nt - 2) / ((nt - 2) / C + 1) + 1;  // equal segments: the last, kept one is as long as the others
   auto segments = [&] { return (nt - 2) / C + 1; };  // of n = 0 .. nt-2
   pat_status rc = kg_alloc(p, C, segments());
-  if (rc != PAT_OK && longer && C > root) {
+  if (rc != PAT_OK && by_default && C > root) {
     C = root;
     rc = kg_alloc(p, C, segments());
   }
+  if (rc == PAT_OK && by_default) p->kg_default = C;
   PAT_TRY(rc);
   const bool two_d = p->dim == 2;
   float* W0 = p->kg_work;

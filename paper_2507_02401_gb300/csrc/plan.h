@@ -113,6 +113,7 @@ struct pat_plan {
 
   // ---- medium-gradient workspace (allocated by the first pat_grad_kappa call)
   int kg_segment = 0;           // checkpoint interval the buffers were sized for
+  int kg_default = 0;           // interval granted to the first call that named none (0: no such call yet)
   float* kg_ckpt = nullptr;     // per checkpoint: two fields (P and D, or P and P^{n-1})
   float* kg_seg = nullptr;      // one segment of recomputed fields
   float* kg_work = nullptr;     // forward-pass fields (3 x N)
