@@ -24,7 +24,6 @@
 // the end of one tile and the stencil of the next are the tile's own D cells
 // and the TMA boxes issued one tile ahead.
 #include <algorithm>
-#include <mutex>
 
 #include "batch.h"
 #include "stencil.cuh"

@@ -16,7 +16,6 @@
 // (x/y in shared memory, z in registers while marching through z, or all
 // planes of an output plane at once on levels that fit one wave of CTAs);
 // other 3D levels run as separable 1D passes.
-#include <mutex>
 #include <type_traits>
 
 #include "internal.h"
@@ -456,7 +455,8 @@ __global__ void __launch_bounds__(256, 4) dwt2d_synthesis_fast_kernel(const floa
 }
 
 // Resident CTAs of a 256-thread kernel with `smem` bytes of dynamic shared
-// memory on the current device (the attribute set once per kernel).
+// memory on the current device, whose limit for that kernel it raises (called
+// once per kernel and device).
 int resident_ctas(const void* fn, int smem) {
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
     cudaGetLastError();
@@ -482,9 +482,8 @@ int grid3d(long long work, int cap) {
 template <int L>
 cudaError_t launch_a2(cudaStream_t st, const float* in, int nx, int ny, float* A, float* H, float* V, float* D,
                       float wdet, const Filt& f) {
-  static std::once_flag once;
-  static int cap = 0;
-  std::call_once(once, [] { cap = resident_ctas((const void*)dwt2d_analysis_fast_kernel<L>, A2F<L>::SMEM); });
+  static PerDevice ctas;
+  const int cap = ctas.get(current_device(), [] { return resident_ctas((const void*)dwt2d_analysis_fast_kernel<L>, A2F<L>::SMEM); });
   if (cap <= 0) return cudaErrorInvalidConfiguration;
   const int tx = ((nx >> 1) + A2F<L>::OX - 1) / A2F<L>::OX, ty = ((ny >> 1) + A2F<L>::OY - 1) / A2F<L>::OY;
   const int ntiles = tx * ty;
@@ -495,9 +494,8 @@ cudaError_t launch_a2(cudaStream_t st, const float* in, int nx, int ny, float* A
 template <int L>
 cudaError_t launch_s2(cudaStream_t st, const float* A, const float* H, const float* V, const float* D, float wdet,
                       int nx, int ny, float* out, const Filt& f) {
-  static std::once_flag once;
-  static int cap = 0;
-  std::call_once(once, [] { cap = resident_ctas((const void*)dwt2d_synthesis_fast_kernel<L>, S2F<L>::SMEM); });
+  static PerDevice ctas;
+  const int cap = ctas.get(current_device(), [] { return resident_ctas((const void*)dwt2d_synthesis_fast_kernel<L>, S2F<L>::SMEM); });
   if (cap <= 0) return cudaErrorInvalidConfiguration;
   const int tx = ((nx >> 1) + S2F<L>::OX - 1) / S2F<L>::OX, ty = ((ny >> 1) + S2F<L>::OY - 1) / S2F<L>::OY;
   const int ntiles = tx * ty;
@@ -951,13 +949,11 @@ __global__ void __launch_bounds__(256, 2) dwt3d_synthesis_fast_kernel(const CBan
 template <int L>
 cudaError_t launch_a3(cudaStream_t st, const float* in, int nx, int ny, int nz, const Bands8& b, float wdet,
                       const Filt& f) {
-  static std::once_flag once;
-  static int cap = 0;
-  static int cap_pp = 0;
-  std::call_once(once, [] {
-    cap = resident_ctas((const void*)dwt3d_analysis_fast_kernel<L>, A3F<L>::SMEM);
-    cap_pp = resident_ctas((const void*)dwt3d_analysis_pp_kernel<L>, A3P<L>::SMEM);
-  });
+  static PerDevice ctas, ctas_pp;
+  const int dev = current_device();
+  const int cap = ctas.get(dev, [] { return resident_ctas((const void*)dwt3d_analysis_fast_kernel<L>, A3F<L>::SMEM); });
+  const int cap_pp =
+      ctas_pp.get(dev, [] { return resident_ctas((const void*)dwt3d_analysis_pp_kernel<L>, A3P<L>::SMEM); });
   if (cap <= 0) return cudaErrorInvalidConfiguration;
   const int cols_x = ((nx >> 1) + A3F<L>::OX - 1) / A3F<L>::OX;
   const int ncols = cols_x * (((ny >> 1) + A3F<L>::OY - 1) / A3F<L>::OY);
@@ -972,9 +968,8 @@ cudaError_t launch_a3(cudaStream_t st, const float* in, int nx, int ny, int nz, 
 template <int L>
 cudaError_t launch_s3(cudaStream_t st, const CBands8& b, float wdet, int nx, int ny, int nz, float* out,
                       const Filt& f) {
-  static std::once_flag once;
-  static int cap = 0;
-  std::call_once(once, [] { cap = resident_ctas((const void*)dwt3d_synthesis_fast_kernel<L>, 0); });
+  static PerDevice ctas;
+  const int cap = ctas.get(current_device(), [] { return resident_ctas((const void*)dwt3d_synthesis_fast_kernel<L>, 0); });
   if (cap <= 0) return cudaErrorInvalidConfiguration;
   const int cols_x = ((nx >> 1) + S3F<L>::OX - 1) / S3F<L>::OX;
   const int ncols = cols_x * (((ny >> 1) + S3F<L>::OY - 1) / S3F<L>::OY);

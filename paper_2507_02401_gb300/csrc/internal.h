@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "pat.h"
+#include "per_device.h"
 
 namespace pat {
 
@@ -36,6 +37,14 @@ pat_status cuda_fail(cudaError_t e, const char* what);
     pat_status _s = (expr);                 \
     if (_s != PAT_OK) return _s;            \
   } while (0)
+
+// The calling thread's device, or -1.
+inline int current_device() {
+  int dev = -1;
+  if (cudaGetDevice(&dev) == cudaSuccess) return dev;
+  cudaGetLastError();
+  return -1;
+}
 
 // ------------------------------------------------------- device structs
 // One sensor's bilinear sampling entry inside a persistent 2D tile.

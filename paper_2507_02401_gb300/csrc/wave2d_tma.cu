@@ -31,7 +31,6 @@
 // medium.
 #include <cudaTypedefs.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "internal.h"
@@ -374,24 +373,24 @@ cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CU
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// Persistent grid: as many CTAs as fit on the device, at most one per tile.
+// Persistent grid: as many CTAs as fit on the device, at most one per tile (0: the kernel does not run there).
 int tma2d_ctas(int nx, int ny, int R, int mode, int sp, bool full) {
-  static int cached[2][4][3][8] = {{{{0}}}};
-  int& c = cached[full][mode][sp][R];
-  if (!c) {
-    int dev = 0, sms = 148, per = 1;
+  static PerDevice resident[2][4][3][8];
+  const int fit = resident[full][mode][sp][R].get(current_device(), [&] {
+    int dev = 0, sms = 0, per = 0;
     const void* fn = kernel_for(R, mode, sp, full);
     const size_t smem = smem_for(R, mode);
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, THREADS, smem) != cudaSuccess || per < 1) {
+    if (!fn || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, THREADS, smem) != cudaSuccess) {
       cudaGetLastError();
-      per = 1;
+      return 0;
     }
-    c = per * sms;
-  }
+    return per * sms;
+  });
   const int ntiles = ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
-  return ntiles < c ? ntiles : c;
+  return ntiles < fit ? ntiles : fit;
 }
 
 long long tma2d_threads(int nx, int ny, int R, int mode, int sp, bool full) {
@@ -402,7 +401,8 @@ cudaError_t step2d_tma_launch(int R, int mode, int sp, bool full, const StepArgs
                               const CUtensorMap& lo, int* status, long long timeout_ns, cudaStream_t st) {
   const void* fn = kernel_for(R, mode, sp, full);
   if (!fn) return cudaErrorInvalidValue;
-  const int nctas = tma2d_ctas(a.nx, a.ny, R, mode, sp, full);  // sets the kernel's attributes once
+  const int nctas = tma2d_ctas(a.nx, a.ny, R, mode, sp, full);  // the first call sets the kernel's attributes
+  if (nctas <= 0) return cudaErrorInvalidConfiguration;
   CUtensorMap map = p, mapl = lo;
   StepArgs args = a;
   void* params[] = {&args, &map, &mapl, &status, &timeout_ns};

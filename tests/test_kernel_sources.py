@@ -2,6 +2,10 @@
 read, and when.  Each rule is checked on the text of the CUDA files."""
 import os
 import re
+import shutil
+import subprocess
+
+import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2507_02401_gb300", "csrc")
 
@@ -42,3 +46,55 @@ def test_programmatic_kernels_read_only_path_takes_plan_constants():
             seen += 1
             assert re.search(constants, m.group(1)), (name, m.group(0))
     assert seen >= 8
+
+
+def test_no_value_of_one_device_serves_another():
+    """Occupancies and kernel attributes belong to a device.  A function-local
+    static that is not constant holds the first caller's, for every device and
+    without synchronisation; PerDevice (csrc/per_device.h) keeps one per device.
+    (The tensor-map encoder, under a once_flag, is the driver's, not a device's.)"""
+    for name in sorted(os.listdir(CSRC)):
+        for m in re.finditer(r"^[ \t]+static\s+(?!const|inline)([^;({=]*)[;({=]", source(name), re.M):
+            encoder = name == "wave3d_tma.cu" and re.search(r"\b(fn|once)\s*$", m.group(1))
+            ok = m.group(1).startswith("PerDevice ") or encoder
+            assert ok, (name, m.group(0))
+
+
+PER_DEVICE_MAIN = r"""
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include "per_device.h"
+static pat::PerDevice kept;
+int main() {
+  std::atomic<int> calls{0};
+  auto value = [&](int d) { return kept.get(d, [&] { ++calls; return d == 5 ? 0 : 100 + d; }); };
+  std::vector<std::thread> t;
+  std::atomic<int> bad{0};
+  for (int i = 0; i < 8; ++i)
+    t.emplace_back([&, i] {
+      for (int k = 0; k < 2000; ++k) {
+        const int d = (k + i) % 5;
+        if (value(d) != 100 + d) ++bad;
+      }
+    });
+  for (auto& x : t) x.join();
+  if (calls > 8 * 5) ++bad;            // kept: at most once per thread and device
+  if (value(5) != 0 || value(5) != 0) ++bad;  // a failure is not kept
+  const int before = calls;
+  if (kept.get(5, [] { return 7; }) != 7 || value(5) != 7 || calls != before) ++bad;
+  if (kept.get(64, [] { return 3; }) != 3 || kept.get(-1, [] { return 4; }) != 4) ++bad;  // no entry: worked out anew
+  std::printf("%d\n", (int)bad);
+  return bad != 0;
+}
+"""
+
+
+def test_per_device_values(tmp_path):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no host compiler")
+    (tmp_path / "m.cpp").write_text(PER_DEVICE_MAIN)
+    exe = str(tmp_path / "m")
+    subprocess.run([cxx, "-std=c++17", "-O2", "-pthread", "-I", CSRC, str(tmp_path / "m.cpp"), "-o", exe], check=True)
+    subprocess.run([exe], check=True)
