@@ -26,7 +26,7 @@ def test_default_segment_is_kept_when_the_long_one_does_not_fit():
     allocates and frees nothing, so that it can be captured, and its bits are
     those of the first."""
     torch = need_gpu()
-    w = custom((1024, 1024), 258, 2, False, 16, seed=5)
+    w = custom((1024, 1024), 257, 2, False, 16, seed=5)
     plan, _, _ = make_pair(w)
     x = torch.as_tensor(w.x_true, dtype=torch.float32, device="cuda")
     r = torch.as_tensor(np.random.default_rng(5).standard_normal((w.ns, w.nt)), dtype=torch.float32, device="cuda")
