@@ -165,15 +165,14 @@ struct StepArgs {
 bool persist2d_supported(int R, bool varc);
 int persist2d_tile_x();
 int persist2d_tile_y();
-size_t persist2d_smem_bytes(int R, bool adj);
-size_t persist2d_xbuf_words(int R, bool adj, int ntiles, int nr = 1);  // 64-bit exchange words, nr fields
+size_t persist2d_xbuf_words(int R, int ntiles, int nr = 1);  // 64-bit exchange words, nr fields
 int persist2d_max_ctas(int R, bool adj, bool varc);  // co-resident CTA limit on this device
-cudaError_t persist2d_launch(int R, bool adj, bool varc, const Persist2DArgs& a, int nctas, cudaStream_t st);
+// layer: with the absorbing layer (a.sp_a, a.sp_b set)
+cudaError_t persist2d_launch(int R, bool adj, bool varc, bool layer, const Persist2DArgs& a, int nctas,
+                             cudaStream_t st);
 // Two right-hand sides per launch (no absorbing layer): a.in / a.out and a.in1 / a.out1.
 int persist2d_max_ctas2(int R, bool adj, bool varc);
 cudaError_t persist2d_launch2(int R, bool adj, bool varc, const Persist2DArgs& a, int nctas, cudaStream_t st);
-// the same with the absorbing layer (a.sp_a, a.sp_b set)
-cudaError_t persist2d_launch_layer(int R, bool adj, bool varc, const Persist2DArgs& a, int nctas, cudaStream_t st);
 // the kernel with 128 x 64 tiles (wave2d_persist_large.cu); its injection lists are split into the tile's frame of
 // persist2dl_edge() cells and its interior (two list bounds per tile)
 int persist2dl_tile_x();

@@ -60,10 +60,8 @@ static pat_status persist_launch(pat_plan* p, bool adj, const Persist2DArgs& a, 
   PAT_TRY_CUDA(cudaMemsetAsync(p->d_abort, 0, sizeof(int), st));
   if (p->persist_large)
     PAT_TRY_CUDA(persist2dl_launch(p->R, adj, p->varc, p->sponge_w > 0, a, p->ntiles, st));
-  else if (p->sponge_w > 0)
-    PAT_TRY_CUDA(persist2d_launch_layer(p->R, adj, p->varc, a, p->ntiles, st));
   else
-    PAT_TRY_CUDA(persist2d_launch(p->R, adj, p->varc, a, p->ntiles, st));
+    PAT_TRY_CUDA(persist2d_launch(p->R, adj, p->varc, p->sponge_w > 0, a, p->ntiles, st));
   return PAT_OK;
 }
 
@@ -872,7 +870,7 @@ static pat_status multi_setup(pat_plan* p, cudaStream_t st) {
   if (p->path == PAT_PATH_PERSISTENT && !p->persist_large && p->sponge_w == 0 &&
       persist2d_max_ctas2(p->R, false, p->varc) >= p->ntiles && persist2d_max_ctas2(p->R, true, p->varc) >= p->ntiles) {
     PAT_TRY(fl(&p->m2.part, (size_t)4 * p->nsplit * p->nt, "split sensor parts (second)"));
-    p->m2.xbuf_bytes = persist2d_xbuf_words(p->R, true, p->ntiles, 2) * 8;
+    p->m2.xbuf_bytes = persist2d_xbuf_words(p->R, p->ntiles, 2) * 8;
     PAT_TRY(plan_alloc(p, &p->m2.xbuf, p->m2.xbuf_bytes, "two-field exchange strips"));
     p->m2.two_field = true;
   }

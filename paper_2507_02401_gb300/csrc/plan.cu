@@ -256,7 +256,7 @@ static pat_status setup_persistent(pat_plan* p, cudaStream_t st) {
   PAT_TRY(upload(p, &p->d_tile_inj_ptr, inj_ptr, "tile injection offsets", st));
   PAT_TRY(upload(p, &p->d_tinj, inj, "tile injection cells", st));
   // tagged exchange words, invalidated (0xff bytes) before every launch
-  p->xbuf_bytes = (large ? persist2dl_xbuf_words(p->ntiles) : persist2d_xbuf_words(p->R, true, p->ntiles)) * 8;
+  p->xbuf_bytes = (large ? persist2dl_xbuf_words(p->ntiles) : persist2d_xbuf_words(p->R, p->ntiles)) * 8;
   PAT_TRY(plan_alloc(p, &p->d_xbuf, p->xbuf_bytes, "exchange strips"));
   if (const char* e = getenv("PAT_POLL_NS")) p->poll_ns = std::max(0, atoi(e));
   PAT_TRY(alloc_n(p, &p->d_abort, 1, "abort flag"));

@@ -46,6 +46,8 @@
 // global-timer limit and a shared abort flag; a CTA that gives up records
 // PAT_ERR_TIMEOUT, raises the abort flag and leaves the loop, so the launch
 // always ends.
+#include <algorithm>
+
 #include "internal.h"
 #include "persist2d.cuh"
 #include "stencil.cuh"
@@ -59,21 +61,31 @@ constexpr int TY = 32;
 constexpr int NTHREADS = (TX / 2) * (TY / 2);  // 512: each thread owns 2 rows x 2 columns
 constexpr int XOFF = 8;                         // left halo columns in shared memory (>= R, multiple of 4)
 constexpr int PITCH = TX + 16;                  // 8 halo columns each side
-constexpr int RCOUNT = 64;                      // threads serving one neighbour (warps 0 .. 7)
-constexpr int EDGE = 8;                         // frame depth (>= R, even)
-constexpr int NFRAME = (TX * 2 * EDGE + (TY - 2 * EDGE) * 2 * EDGE) / 4;  // 320: whole warps
-static_assert(EDGE >= kMaxR && NFRAME % 32 == 0 && NFRAME >= 4 * RCOUNT, "frame and interior are whole warps");
+
+// The tile's frame: the cells whose stencils reach beyond it.  Its threads, whole warps, wait for the halo.  EDGE is
+// even and at least R.
+template <int R, bool ADJ>
+struct Frame {
+  static constexpr int EDGE = 8;
+  static constexpr int RCOUNT = R == 1 ? 32 : 64;  // threads serving one neighbour (warps 0 .. 3 or 0 .. 7)
+  static constexpr int BLOCKS = (TX * 2 * EDGE + (TY - 2 * EDGE) * 2 * EDGE) / 4;  // 320 blocks of 2 x 2
+  static constexpr int N = (BLOCKS + 31) / 32 * 32;  // the last warp filled up with interior blocks
+  static_assert(EDGE >= R && EDGE % 2 == 0 && N >= 4 * RCOUNT && N < NTHREADS, "interior stencils need no halo");
+};
 
 // Thread of the frame that owns row pair rp, column pair cp (the inverse of cells_of).
+template <int R, bool ADJ>
 __device__ __forceinline__ int frame_thread(int rp, int cp) {
-  constexpr int E2 = EDGE / 2, MIDR = (TY - 2 * EDGE) / 2, MID = (TX - 2 * EDGE) / 2;
+  constexpr int EDGE = Frame<R, ADJ>::EDGE, E2 = EDGE / 2, MIDR = (TY - 2 * EDGE) / 2, MID = (TX - 2 * EDGE) / 2;
   if (rp < E2) return rp * (TX / 2) + cp;
   if (rp >= E2 + MIDR) return (rp - MIDR) * (TX / 2) + cp;
   return EDGE * TX / 2 + (rp - E2) * EDGE + (cp < E2 ? cp : cp - MID);
 }
 
 // First cell (row, column) of thread t: the frame's top and bottom rows, then its side columns, then the interior.
+template <int R, bool ADJ>
 __device__ __forceinline__ void cells_of(int t, int& row, int& col) {
+  constexpr int EDGE = Frame<R, ADJ>::EDGE;
   constexpr int BAND = EDGE * TX / 4;           // threads of the top (and of the bottom) rows
   constexpr int SIDE = EDGE;                    // column pairs of the two sides in one row pair
   constexpr int MID = (TX - 2 * EDGE) / 2;      // column pairs of the interior in one row pair
@@ -81,12 +93,12 @@ __device__ __forceinline__ void cells_of(int t, int& row, int& col) {
     const int rp = t / (TX / 2);
     row = 2 * (rp < EDGE / 2 ? rp : rp + (TY - 2 * EDGE) / 2);
     col = 2 * (t % (TX / 2));
-  } else if (t < NFRAME) {
+  } else if (t < Frame<R, ADJ>::BLOCKS) {
     const int u = t - 2 * BAND, cp = u % SIDE;
     row = EDGE + 2 * (u / SIDE);
     col = 2 * (cp < SIDE / 2 ? cp : cp + MID);
   } else {
-    const int u = t - NFRAME;
+    const int u = t - Frame<R, ADJ>::BLOCKS;
     row = EDGE + 2 * (u / MID);
     col = EDGE + 2 * (u % MID);
   }
@@ -102,7 +114,8 @@ struct Geo {
   // edges as strips of words, [top TX][bottom TX][left TY][right TY] (512^2 order 2: K 1.21 us per step with
   // strips, 1.23 with blocks; 64^2 0.81 and 0.89; 768 x 704, two CTAs per SM, 1.34 and 1.52).
   static constexpr int D = (R + 1) / 2;
-  static constexpr int SLOT = 4 * NFRAME;          // words per tile, slot and right-hand side
+  static constexpr int SLOT = R == 1 ? 2 * (TX + TY) : 4 * Frame<R, ADJ>::BLOCKS;  // words per tile, slot and right-hand side
+  static constexpr int RCOUNT = Frame<R, ADJ>::RCOUNT;
   static constexpr int PER = (D * TX / 2 + RCOUNT - 1) / RCOUNT;  // blocks a polling thread takes at most
   static_assert(D * TY / 2 <= RCOUNT * PER, "west and east blocks fit as well");
 };
@@ -176,7 +189,7 @@ __device__ __forceinline__ HaloDuty<Geo<R, ADJ>::PER> halo_duty(int region, int 
   HaloDuty<G::PER> h;
 #pragma unroll
   for (int j = 0; j < G::PER; ++j) {
-    const int i = rrank + j * RCOUNT;
+    const int i = rrank + j * G::RCOUNT;
     h.src[j] = h.dst[j] = h.rows[j] = 0;
     if (R == 1) {  // north and south: a pair of words per thread; west and east: one word
       if (i >= 32) continue;
@@ -191,14 +204,14 @@ __device__ __forceinline__ HaloDuty<Geo<R, ADJ>::PER> halo_duty(int region, int 
     if (region < 2) {  // north: the neighbour's last D row pairs; south: its first D
       if (i >= G::D * TX / 2) continue;
       const int b = i / (TX / 2), cp = i % (TX / 2);
-      h.src[j] = 4 * frame_thread(region == 0 ? TY / 2 - G::D + b : b, cp);
+      h.src[j] = 4 * frame_thread<R, ADJ>(region == 0 ? TY / 2 - G::D + b : b, cp);
       h.dst[j] = (region == 0 ? R - 2 * G::D + 2 * b : R + TY + 2 * b) * PITCH + XOFF + 2 * cp;
       // R is odd: the outermost block reaches one row beyond the halo
       h.rows[j] = region == 0 ? (b == 0 ? 2 : 3) : (b == G::D - 1 ? 1 : 3);
     } else {  // west: the neighbour's last D column pairs; east: its first D
       if (i >= G::D * TY / 2) continue;
       const int rp = i / G::D, g = i % G::D;
-      h.src[j] = 4 * frame_thread(rp, region == 2 ? TX / 2 - G::D + g : g);
+      h.src[j] = 4 * frame_thread<R, ADJ>(rp, region == 2 ? TX / 2 - G::D + g : g);
       h.dst[j] = (R + 2 * rp) * PITCH + (region == 2 ? XOFF - 2 * G::D : XOFF + TX) + 2 * g;
       h.rows[j] = 3;
     }
@@ -208,7 +221,7 @@ __device__ __forceinline__ HaloDuty<Geo<R, ADJ>::PER> halo_duty(int region, int 
 
 // Copy the halo of state `step` of NR fields from the neighbour's slots X[r]
 // into the shared buffers Sc[r] (second field at Sc[r] + SBUF).  Executed by
-// the RCOUNT threads of one region; returns false if the wait ran out.  Each
+// the threads of one region; returns false if the wait ran out.  Each
 // poll first issues the loads of every block still pending (all fields), then
 // checks their tags, so the L2 round trips of one poll overlap instead of
 // following one another.
@@ -295,10 +308,13 @@ __device__ __forceinline__ bool load_halo(float* const (&Sc)[NR], const u64* con
 // solves of one medium): every step exchanges both fields' strips in the same round trip and runs both
 // updates between the same barriers.  Inputs / outputs of field r are a.in / a.out (r = 0) and a.in1 /
 // a.out1 (r = 1); field r's exchange words follow field 0's in each slot.
-// (Order 2 leaves room for two CTAs per SM, so its grids may have twice as many tiles as there are SMs.)
-template <int R, bool ADJ, bool VARC, bool SP, int NR>
-__global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_persist_kernel(const Persist2DArgs a) {
+// CTAS: CTAs per SM to leave registers for.  Order 2 has a form for two (64 registers), for grids with more tiles
+// than SMs; with a layer it spills, so a grid whose tiles have an SM each takes the form for one (order 2 varying,
+// K* with a layer, us per step in 64 registers -> here: 64^2 1.90 -> 1.43, 512^2 1.88 -> 1.45).
+template <int R, bool ADJ, bool VARC, bool SP, int NR, int CTAS>
+__global__ void __launch_bounds__(NTHREADS, CTAS) wave2d_persist_kernel(const Persist2DArgs a) {
   using G = Geo<R, ADJ>;
+  constexpr int NFRAME = Frame<R, ADJ>::N;
   static_assert(NR == 1 || !SP, "several right-hand sides run without the absorbing layer");
   extern __shared__ float4 smem4[];
   float* S0 = reinterpret_cast<float*>(smem4);   // [slot][rhs][field] buffers
@@ -314,7 +330,7 @@ __global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_pe
   const int tiy = tile / a.tiles_x;
   const int gx0 = tix * TX, gy0 = tiy * TY;
   int c0, r0;
-  cells_of(t, r0, c0);
+  cells_of<R, ADJ>(t, r0, c0);
   const int nx = a.nx, ny = a.ny, nt = a.nt;
   u64* xbuf = reinterpret_cast<u64*>(a.xbuf);
   float2 w2[R + 1];  // stencil weights, packed
@@ -324,11 +340,11 @@ __global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_pe
   float* OUT[2] = {a.out, a.out1};
   float* PART[2] = {a.part, a.part1};
 
-  // halo duty of warps 0 .. 7: 0 = north, 1 = south, 2 = west, 3 = east neighbour
+  // halo duty of the first warps: 0 = north, 1 = south, 2 = west, 3 = east neighbour
   const int region = warp & 3;
   const int rrank = (warp >> 2) * 32 + lane;
   int nb = -1;
-  if (warp < 8) {
+  if (warp < 4 * G::RCOUNT / 32) {
     if (region == 0 && tiy > 0) nb = tile - a.tiles_x;
     if (region == 1 && tiy < a.tiles_y - 1) nb = tile + a.tiles_x;
     if (region == 2 && tix > 0) nb = tile - 1;
@@ -379,8 +395,9 @@ __global__ void __launch_bounds__(NTHREADS, R == 1 && NR == 1 ? 2 : 1) wave2d_pe
     store_state<R, ADJ>(Sbuf(0, r), Xown(0, r), P[r], Pl[r], r0, c0, 0u);
 
   // The interior's threads serve the tile's sensors.  Adjoint: S^T r_n, n = nt-1-k, of the injected cells into
-  // step k's accumulators (KEEP: the first cell of a thread, with its first sensor, stays in registers).
-  constexpr bool KEEP = R > 1;
+  // step k's accumulators (KEEP: the first cell of a thread, with its first sensor, stays in registers; the form for
+  // two CTAs per SM has none to spare, and kept in shared memory it takes 1.91 instead of 1.82 us at 640 x 512).
+  constexpr bool KEEP = CTAS == 1;
   const int ut = t - NFRAME;
   constexpr int NINNER = NTHREADS - NFRAME;
   int e0 = 0, e1 = 0, is0 = 0;
@@ -555,27 +572,28 @@ __global__ void split_combine_kernel(const float* __restrict__ part, const int* 
   y[(long long)split_sensor[q] * nt + t] = ((p[0] + p[nt]) + p[2 * nt]) + p[3 * nt];
 }
 
-template <int R, bool ADJ, bool VARC, bool SP, int NR = 1>
+template <int R, bool ADJ, bool VARC, bool SP, int NR, int CTAS = 1>
 void* kfn() {
-  return (void*)wave2d_persist_kernel<R, ADJ, VARC, SP, NR>;
+  return (void*)wave2d_persist_kernel<R, ADJ, VARC, SP, NR, CTAS>;
 }
 
-template <bool SP>
-void* pick_sp(int R, bool adj, bool varc) {
-#define PAT_P2D(RR)                                                               \
-  if (R == RR) {                                                                  \
-    if (adj) return varc ? kfn<RR, true, true, SP>() : kfn<RR, true, false, SP>(); \
-    return varc ? kfn<RR, false, true, SP>() : kfn<RR, false, false, SP>();       \
+template <int R, bool SP, int CTAS>
+void* pick_r(bool adj, bool varc) {
+  if (adj) return varc ? kfn<R, true, true, SP, 1, CTAS>() : kfn<R, true, false, SP, 1, CTAS>();
+  return varc ? kfn<R, false, true, SP, 1, CTAS>() : kfn<R, false, false, SP, 1, CTAS>();
+}
+
+// ctas: CTAs per SM wanted, 1 or (order 2) 2
+void* pick(int R, bool adj, bool varc, bool layer, int ctas) {
+  if (ctas == 2) return R == 1 ? (layer ? pick_r<1, true, 2>(adj, varc) : pick_r<1, false, 2>(adj, varc)) : nullptr;
+  switch (R) {
+    case 1: return layer ? pick_r<1, true, 1>(adj, varc) : pick_r<1, false, 1>(adj, varc);
+    case 3: return layer ? pick_r<3, true, 1>(adj, varc) : pick_r<3, false, 1>(adj, varc);
+    case 5: return layer ? pick_r<5, true, 1>(adj, varc) : pick_r<5, false, 1>(adj, varc);
+    case 7: return layer ? pick_r<7, true, 1>(adj, varc) : pick_r<7, false, 1>(adj, varc);
+    default: return nullptr;
   }
-  PAT_P2D(1)
-  PAT_P2D(3)
-  PAT_P2D(5)
-  PAT_P2D(7)
-#undef PAT_P2D
-  return nullptr;
 }
-
-void* pick(int R, bool adj, bool varc) { return pick_sp<false>(R, adj, varc); }
 
 // two right-hand sides, no absorbing layer
 void* pick2(int R, bool adj, bool varc) {
@@ -602,6 +620,19 @@ cudaError_t prepare(void* f, int R, bool adj, int nr = 1) {
   return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(R, adj, nr));
 }
 
+// CTAs of a kernel that the current device holds at once.
+int resident(void* f, int R, bool adj, int nr = 1) {
+  int dev = 0, sms = 0, per_sm = 0;
+  if (!f || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      prepare(f, R, adj, nr) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, NTHREADS, smem_bytes(R, adj, nr)) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return sms * per_sm;
+}
+
 }  // namespace
 
 cudaError_t persist2d_split_combine(const float* part, const int* split_sensor, int nsplit, int nt, float* y,
@@ -615,52 +646,31 @@ cudaError_t persist2d_split_combine(const float* part, const int* split_sensor, 
 bool persist2d_supported(int R, bool) { return R == 1 || R == 3 || R == 5 || R == 7; }
 int persist2d_tile_x() { return TX; }
 int persist2d_tile_y() { return TY; }
-size_t persist2d_smem_bytes(int R, bool adj) { return smem_bytes(R, adj); }
-size_t persist2d_xbuf_words(int, bool, int ntiles, int nr) { return (size_t)nr * ntiles * 2 * 4 * NFRAME; }
-
-int persist2d_max_ctas(int R, bool adj, bool varc) {
-  void* f = pick(R, adj, varc);
-  if (!f) return 0;
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (prepare(f, R, adj) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, NTHREADS, smem_bytes(R, adj)) != cudaSuccess)
-    return 0;
-  return sms * per_sm;
+size_t persist2d_xbuf_words(int R, int ntiles, int nr) {
+  const int slot = R == 1 ? Geo<1, true>::SLOT : Geo<3, true>::SLOT;  // 8-cell frames from R = 3 on
+  return (size_t)nr * ntiles * 2 * slot;
 }
 
-cudaError_t persist2d_launch_layer(int R, bool adj, bool varc, const Persist2DArgs& a, int nctas, cudaStream_t st) {
-  void* f = pick_sp<true>(R, adj, varc);
+int persist2d_max_ctas(int R, bool adj, bool varc) {
+  const int fit = resident(pick(R, adj, varc, false, 1), R, adj);
+  return R == 1 ? std::max(fit, resident(pick(R, adj, varc, false, 2), R, adj)) : fit;
+}
+
+cudaError_t persist2d_launch(int R, bool adj, bool varc, bool layer, const Persist2DArgs& a, int nctas,
+                             cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  void* f = pick(R, adj, varc, layer, nctas > sms ? 2 : 1);
   if (!f) return cudaErrorInvalidValue;
-  int per_sm = 0, dev = 0, sms = 0;  // the layer variant must fit as many CTAs as the plan's tiles
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return cudaErrorUnknown;
-  cudaError_t e = prepare(f, R, adj);
+  e = prepare(f, R, adj);
   if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, NTHREADS, smem_bytes(R, adj));
-  if (e != cudaSuccess) return e;
-  if (per_sm * sms < nctas) return cudaErrorCooperativeLaunchTooLarge;
   void* args[] = {(void*)&a};
   return cudaLaunchCooperativeKernel(f, dim3(nctas), dim3(NTHREADS), args, smem_bytes(R, adj), st);
 }
 
-int persist2d_max_ctas2(int R, bool adj, bool varc) {
-  void* f = pick2(R, adj, varc);
-  if (!f) return 0;
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (prepare(f, R, adj, 2) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, NTHREADS, smem_bytes(R, adj, 2)) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return sms * per_sm;
-}
+int persist2d_max_ctas2(int R, bool adj, bool varc) { return resident(pick2(R, adj, varc), R, adj, 2); }
 
 cudaError_t persist2d_launch2(int R, bool adj, bool varc, const Persist2DArgs& a, int nctas, cudaStream_t st) {
   void* f = pick2(R, adj, varc);
@@ -669,15 +679,6 @@ cudaError_t persist2d_launch2(int R, bool adj, bool varc, const Persist2DArgs& a
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&a};
   return cudaLaunchCooperativeKernel(f, dim3(nctas), dim3(NTHREADS), args, smem_bytes(R, adj, 2), st);
-}
-
-cudaError_t persist2d_launch(int R, bool adj, bool varc, const Persist2DArgs& a, int nctas, cudaStream_t st) {
-  void* f = pick(R, adj, varc);
-  if (!f) return cudaErrorInvalidValue;
-  cudaError_t e = prepare(f, R, adj);
-  if (e != cudaSuccess) return e;
-  void* args[] = {(void*)&a};
-  return cudaLaunchCooperativeKernel(f, dim3(nctas), dim3(NTHREADS), args, smem_bytes(R, adj), st);
 }
 
 }  // namespace pat
