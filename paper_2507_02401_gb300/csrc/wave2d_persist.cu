@@ -63,12 +63,14 @@ constexpr int XOFF = 8;                         // left halo columns in shared m
 constexpr int PITCH = TX + 16;                  // 8 halo columns each side
 
 // The tile's frame: the cells whose stencils reach beyond it.  Its threads, whole warps, wait for the halo.  EDGE is
-// even and at least R.
+// even and at least R.  Order 2 has the choice: K with 4 cells (six warps wait, ten work meanwhile: 512^2 1.08 us per
+// step, 1.26 with 8 cells, 1.25 with 2), K* with 8, its two stencils taking longer than the halo (640 x 512, two
+// CTAs on some SMs: 1.81 us, 1.92 with 4, 1.97 with 2).
 template <int R, bool ADJ>
 struct Frame {
-  static constexpr int EDGE = 8;
+  static constexpr int EDGE = R == 1 && !ADJ ? 4 : 8;
   static constexpr int RCOUNT = R == 1 ? 32 : 64;  // threads serving one neighbour (warps 0 .. 3 or 0 .. 7)
-  static constexpr int BLOCKS = (TX * 2 * EDGE + (TY - 2 * EDGE) * 2 * EDGE) / 4;  // 320 blocks of 2 x 2
+  static constexpr int BLOCKS = (TX * 2 * EDGE + (TY - 2 * EDGE) * 2 * EDGE) / 4;  // 176 or 320 blocks of 2 x 2
   static constexpr int N = (BLOCKS + 31) / 32 * 32;  // the last warp filled up with interior blocks
   static_assert(EDGE >= R && EDGE % 2 == 0 && N >= 4 * RCOUNT && N < NTHREADS, "interior stencils need no halo");
 };
