@@ -154,11 +154,13 @@ pat_status build_tables(pat_batch* b, int variant, cudaStream_t st) {
   PAT_TRY_CUDA(cudaMemcpyAsync(b->d_tiles, tiles.data(), sizeof(BTile) * tiles.size(), cudaMemcpyHostToDevice, st));
   PAT_TRY_CUDA(cudaMemcpyAsync(b->d_maps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice, st));
   PAT_TRY_CUDA(cudaStreamSynchronize(st));  // host vectors go out of scope
-  b->nctas = batch_max_ctas(b->R, variant, false);
-  b->nctas_adj = batch_max_ctas(b->R, variant, true);
-  if (b->nctas <= 0 || b->nctas_adj <= 0) {
-    set_error("batched step kernel does not fit on this device");
-    return PAT_ERR_CUDA;
+  for (int ra = 0; ra < 2; ++ra) {
+    b->nctas[ra] = batch_max_ctas(b->R, variant, false, ra != 0);
+    b->nctas_adj[ra] = batch_max_ctas(b->R, variant, true, ra != 0);
+    if (b->nctas[ra] <= 0 || b->nctas_adj[ra] <= 0) {
+      set_error("batched step kernel does not fit on this device");
+      return PAT_ERR_CUDA;
+    }
   }
   return PAT_OK;
 }
@@ -181,7 +183,7 @@ BatchStepArgs step_args(const pat_batch* b, int t, bool adjoint) {
 // Steps 0 .. T-1 of K or K*: one launch per step, or all of them in one
 // cooperative launch with a grid barrier between steps (b->runall).
 pat_status batch_steps(pat_batch* b, int T, bool adjoint, cudaStream_t st) {
-  const int nctas = adjoint ? b->nctas_adj : b->nctas;
+  const int nctas = (adjoint ? b->nctas_adj : b->nctas)[b->runall ? 1 : 0];
   if (b->runall) {
     if (T <= 0) return PAT_OK;
     PAT_TRY_CUDA(cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned), st));
@@ -189,7 +191,7 @@ pat_status batch_steps(pat_batch* b, int T, bool adjoint, cudaStream_t st) {
     a.t_end = T;
     a.active_dev = b->d_active;
     a.bar = b->d_bar;
-    PAT_TRY_CUDA(batch_run_launch(b->R, b->variant, a, nctas, st));
+    PAT_TRY_CUDA(batch_run_launch(b->R, b->variant, a, std::min(nctas, a.active), st));
     return PAT_OK;
   }
   for (int t = 0; t < T; ++t) PAT_TRY_CUDA(batch_step_launch(b->R, b->variant, step_args(b, t, adjoint), nctas, st));
@@ -460,7 +462,7 @@ pat_status pat_batch_info(pat_batch* b, int* tile_rows, int* ctas, long long* gr
     return PAT_ERR_INVALID;
   }
   if (tile_rows) *tile_rows = batch_tile_y(b->variant);
-  if (ctas) *ctas = b->nctas;
+  if (ctas) *ctas = b->nctas[b->runall ? 1 : 0];
   if (graph_nodes) *graph_nodes = (long long)b->graph_nodes;
   if (tune_ms) {
     tune_ms[0] = b->tune_ms[0];

@@ -62,7 +62,7 @@ bool batch_eligible(pat_plan* const* plans, int B);
 // batch_kernels.cu
 int batch_tile_y(int variant);  // tile height of a kernel variant (0: 64 rows, 1: 32 rows)
 size_t batch_smem(int R, int variant, bool adj);
-int batch_max_ctas(int R, int variant, bool adj);  // co-resident CTAs on this device
+int batch_max_ctas(int R, int variant, bool adj, bool runall);  // co-resident CTAs on this device
 cudaError_t batch_step_launch(int R, int variant, const BatchStepArgs& a, int nctas, cudaStream_t st);
 // All steps a.t .. a.t_end - 1 in one cooperative launch of nctas co-resident CTAs,
 // a bounded grid-wide barrier between steps (a.bar zeroed beforehand).
@@ -74,7 +74,7 @@ cudaError_t batch_encode(const float* base, int nx, int ny, int R, int variant, 
 struct pat_batch {
   std::vector<pat_plan*> plans;  // borrowed, in the caller's order
   std::vector<int> order;        // instance slots sorted by nt, longest first (slot -> caller index)
-  int B = 0, R = 1, variant = 0, nctas = 0, nctas_adj = 0, max_nt = 0, ntiles = 0;
+  int B = 0, R = 1, variant = 0, nctas[2] = {0, 0}, nctas_adj[2] = {0, 0}, max_nt = 0, ntiles = 0;
   std::vector<int> active;       // active[t]: tiles still running at global step t
   pat::BInst* d_inst = nullptr;
   pat::BTile* d_tiles = nullptr;

@@ -38,7 +38,11 @@ constexpr int TX = 64, XH = 8, BW = TX + 2 * XH;
 // Each thread owns 4 columns x 4 rows, as in the single-instance kernel: a 64-row tile is a CTA of 256
 // threads, a 32-row tile one of 128.  CTAs per SM to leave registers for with 32-row tiles: four, three in the
 // adjoint above order 4 (32 uneven instances, order 8, K us per step: 10.2 with four forward CTAs, 10.9 with three).
-constexpr int min_ctas(int R, int TY, bool adj) { return TY == 64 ? 1 : R > 3 && adj ? 3 : 4; }
+// One launch for all steps (RUNALL) also keeps its place in the tile table: at order 8 it gets a CTA less, or it
+// spills 200 bytes (16 instances of up to 512^2, K 190 steps: 2.01 -> 1.89 ms; lower orders lose by it).
+constexpr int min_ctas(int R, int TY, bool adj, bool runall) {
+  return TY == 64 ? 1 : (R > 3 && adj ? 3 : 4) - (runall && R == 7 ? 1 : 0);
+}
 constexpr int NP = 2, RUN = 4, TCOLS = TX / (2 * NP);
 
 template <int R, int TY, bool ADJ>
@@ -80,7 +84,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned round, int*
 }
 
 template <int R, int TY, bool ADJ, bool RUNALL>
-__global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS, min_ctas(R, TY, ADJ)) batch_step_kernel(const BatchStepArgs a) {
+__global__ void __launch_bounds__(GB<R, TY, ADJ>::THREADS, min_ctas(R, TY, ADJ, RUNALL)) batch_step_kernel(const BatchStepArgs a) {
   using G = GB<R, TY, ADJ>;
   constexpr int THREADS = G::THREADS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -322,27 +326,18 @@ size_t batch_smem(int R, int variant, bool adj) {
   return sizeof(float) * 2 * (adj ? 2 : 1) * (size_t)BW * (batch_tile_y(variant) + 2 * R) + 16;
 }
 
-int batch_max_ctas(int R, int variant, bool adj) {
-  // co-resident CTAs of the per-step and of the run-all kernel alike (the smaller of the two)
-  int best = -1;
-  for (int runall = 0; runall < 2; ++runall) {
-    const void* fn = kernel_for(R, variant, adj, runall != 0);
-    if (!fn) return 0;
-    const size_t smem = batch_smem(R, variant, adj);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    int dev = 0, sms = 0, per = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads_for(variant), smem) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    best = best < 0 ? per * sms : std::min(best, per * sms);
+int batch_max_ctas(int R, int variant, bool adj, bool runall) {
+  const void* fn = kernel_for(R, variant, adj, runall);
+  const size_t smem = batch_smem(R, variant, adj);
+  int dev = 0, sms = 0, per = 0;
+  if (!fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads_for(variant), smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
   }
-  return best;
+  return per * sms;
 }
 
 cudaError_t batch_step_launch(int R, int variant, const BatchStepArgs& a, int nctas, cudaStream_t st) {
