@@ -323,24 +323,6 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
   p->ns = ns;
   p->corners = 1 << p->dim;
 
-  // ---- step engines: TMA kernels when the driver provides the descriptor encoder.  Their rows start on
-  // 16-byte boundaries, so fields of other widths get padded rows (the pad columns are never read back: the
-  // descriptors end at nx).
-  const char* env2 = getenv("PAT_STEP2D");
-  const char* env3 = getenv("PAT_STEP3D");
-  const char* env = p->dim == 2 ? env2 : env3;
-  bool tma = tma_encoder() != nullptr && !(env && strcmp(env, "plain") == 0) &&
-             (p->dim == 2 ? tma2d_supported(p->R) : tma3d_supported(p->R));
-  p->pitch = p->n[0];
-  if (tma) {
-    p->pitch = (p->n[0] + 3) / 4 * 4;
-    if ((long long)p->pitch * p->n[1] * p->n[2] >= (1LL << 31)) {  // cell indices are int
-      tma = p->n[0] % 4 == 0;
-      p->pitch = p->n[0];
-    }
-  }
-  p->Np = (long long)p->pitch * p->n[1] * p->n[2];
-
   // ---- medium and CFL (c_max dt / h <= 1 / (sqrt(d) sum |c_k|))
   double cmax = 0.0, cmin = 0.0;
   bool constant = true;
@@ -383,6 +365,30 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
     p->kappa0 = (float)k0;
     p->kappa0_lo = (float)(k0 - (double)p->kappa0);
   }
+  // ---- step engines: TMA kernels when the driver provides the descriptor encoder.  Their rows start on
+  // 16-byte boundaries, so fields of other widths get padded rows (the pad columns are never read back: the
+  // descriptors end at nx).
+  // They keep the adjoint's state as Z = kappa Q and divide by kappa where Q itself is asked for (the absorbing layer's
+  // last step, the medium gradient, 3D with a varying medium), so kappa must be far from FP32's smallest numbers: Z's
+  // low part, ~2^-24 Z, has to hold its bits too.  Slower cells (under ~1e-9 of the fastest) keep the plain kernels,
+  // whose state is Q, wherever these served before: 3D varying media and rows of no multiple of 4 cells.
+  const bool z_safe = !p->varc || (cmin * dt / p->h) * (cmin * dt / p->h) >= 0x1p-60;
+  const bool rows4 = p->n[0] % 4 == 0;
+  const char* env2 = getenv("PAT_STEP2D");
+  const char* env3 = getenv("PAT_STEP3D");
+  const char* env = p->dim == 2 ? env2 : env3;
+  bool tma = tma_encoder() != nullptr && !(env && strcmp(env, "plain") == 0) &&
+             (p->dim == 2 ? tma2d_supported(p->R) : tma3d_supported(p->R)) && (z_safe || (p->dim == 2 && rows4));
+  p->pitch = p->n[0];
+  if (tma) {
+    p->pitch = (p->n[0] + 3) / 4 * 4;
+    if ((long long)p->pitch * p->n[1] * p->n[2] >= (1LL << 31)) {  // cell indices are int
+      tma = rows4;
+      p->pitch = p->n[0];
+    }
+  }
+  p->Np = (long long)p->pitch * p->n[1] * p->n[2];
+
   if (p->varc) {
     std::vector<float> kap(p->N), kap_lo(p->N);
     for (long long i = 0; i < p->N; ++i) {
@@ -504,7 +510,7 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
     p->persist_ok = tiles(persist2d_tile_x(), persist2d_tile_y()) <=
                     std::min(persist2d_max_ctas(p->R, false, p->varc), persist2d_max_ctas(p->R, true, p->varc));
     // grids with too many 64 x 32 tiles: 128 x 64 tiles, whose kernel reads kappa and the layer's factors in pairs
-    if (!p->persist_ok && p->pitch % 2 == 0) {
+    if (!p->persist_ok && p->pitch % 2 == 0 && (z_safe || rows4)) {
       const int cap = std::min(persist2dl_max_ctas(p->R, false, p->varc), persist2dl_max_ctas(p->R, true, p->varc));
       int TX, TY, dev = 0, sms = 0;
       tma2d_tile(&TX, &TY);
