@@ -64,6 +64,66 @@ static pat_status upload(pat_plan* p, T** ptr, const std::vector<T>& host, const
   return PAT_OK;
 }
 
+static size_t padded(size_t bytes) { return (std::max<size_t>(bytes, 1) + 255) / 256 * 256; }
+
+// Device arrays of one allocation: their sizes are collected first, those with contents in front, so that a plan's
+// many small lists and its workspace cost one cudaMalloc and one copy (a plan has some forty arrays; at 1024^2 order 8
+// creation took 0.77 ms with one of each per array and the
+// kernels' occupancies queried anew, 0.25 so).  Lives until the stream has been synchronised.
+class Arena {
+ public:
+  template <typename T>
+  void array(T** ptr, size_t count) {
+    add(reinterpret_cast<void**>(ptr), count * sizeof(T), false);
+  }
+  template <typename T>
+  void array(T** ptr, const std::vector<T>& host) {
+    fill(reinterpret_cast<void**>(ptr), host.data(), host.size() * sizeof(T));
+  }
+  template <typename T>
+  void zeros(T** ptr, size_t count) {
+    fill(reinterpret_cast<void**>(ptr), nullptr, count * sizeof(T));
+  }
+  pat_status commit(pat_plan* p, const char* what, cudaStream_t st) {
+    void* base;
+    PAT_TRY(plan_alloc(p, &base, image_.size() + rest_, what));
+    for (const Item& i : items_) *i.ptr = static_cast<char*>(base) + i.offset + (i.filled ? 0 : image_.size());
+    if (!image_.empty()) PAT_TRY_CUDA(cudaMemcpyAsync(base, image_.data(), image_.size(), cudaMemcpyHostToDevice, st));
+    return PAT_OK;
+  }
+
+ private:
+  struct Item {
+    void** ptr;
+    size_t offset;
+    bool filled;
+  };
+  void add(void** ptr, size_t bytes, bool filled) {
+    items_.push_back(Item{ptr, filled ? image_.size() : rest_, filled});
+    if (!filled) rest_ += padded(bytes);
+  }
+  void fill(void** ptr, const void* host, size_t bytes) {
+    add(ptr, bytes, true);
+    const size_t at = image_.size();
+    image_.resize(at + padded(bytes), 0);
+    if (host && bytes) std::memcpy(image_.data() + at, host, bytes);
+  }
+  std::vector<Item> items_;
+  std::vector<char> image_;
+  size_t rest_ = 0;
+};
+
+// Items 0 .. n-1 grouped by bin, in order within a bin: items[k] for k in [ptr[b], ptr[b + 1]).
+struct Groups {
+  std::vector<int> ptr, items;
+  Groups(int bins, const std::vector<int>& bin_of) : ptr((size_t)bins + 1, 0), items(bin_of.size()) {
+    for (int b : bin_of) ++ptr[(size_t)b + 1];
+    for (int b = 0; b < bins; ++b) ptr[(size_t)b + 1] += ptr[b];
+    std::vector<int> next(ptr.begin(), ptr.end() - 1);
+    for (size_t i = 0; i < bin_of.size(); ++i) items[next[bin_of[i]]++] = (int)i;
+  }
+};
+
 // ------------------------------------------------------ staggered weights
 // Staggered first-derivative weights of order 2M at half-integer offsets.
 static const double kStag[4][4] = {{1.0, 0, 0, 0},
@@ -176,7 +236,7 @@ static pat_status pitched(pat_plan* p, float* dense, float** out, const char* wh
 }
 
 // --------------------------------------------------- persistent 2D set-up
-static pat_status setup_persistent(pat_plan* p, cudaStream_t st) {
+static void setup_persistent(pat_plan* p, Arena& arena) {
   const bool large = p->persist_large;
   const int TX = large ? persist2dl_tile_x() : persist2d_tile_x(), TY = large ? persist2dl_tile_y() : persist2d_tile_y();
   p->tiles_x = (p->n[0] + TX - 1) / TX;
@@ -186,7 +246,8 @@ static pat_status setup_persistent(pat_plan* p, cudaStream_t st) {
 
   // sampling entries grouped by the tile holding each sensor's base cell; a
   // sensor whose 2x2 block crosses a tile corner is split into four parts
-  std::vector<std::vector<SampEntry>> per_tile(p->ntiles);
+  std::vector<SampEntry> entry;
+  std::vector<int> tile_of;
   std::vector<int> split_sensor;
   for (int s = 0; s < p->ns; ++s) {
     const int c0 = p->h_sens_cell[s * 4];
@@ -200,7 +261,8 @@ static pat_status setup_persistent(pat_plan* p, cudaStream_t st) {
       e.lx = (short)(bx % TX);
       e.ly = (short)(by % TY);
       for (int k = 0; k < 4; ++k) e.w[k] = p->h_sens_w[s * 4 + k];
-      per_tile[tile].push_back(e);
+      entry.push_back(e);
+      tile_of.push_back(tile);
       continue;
     }
     const int q = (int)split_sensor.size();
@@ -215,52 +277,42 @@ static pat_status setup_persistent(pat_plan* p, cudaStream_t st) {
       e.ly = (short)(cy % TY);
       e.w[0] = p->h_sens_w[s * 4 + k];
       e.w[1] = e.w[2] = e.w[3] = 0.f;
-      per_tile[(cy / TY) * p->tiles_x + cx / TX].push_back(e);
+      entry.push_back(e);
+      tile_of.push_back((cy / TY) * p->tiles_x + cx / TX);
     }
   }
   p->nsplit = (int)split_sensor.size();
-  PAT_TRY(upload(p, &p->d_split_sensor, split_sensor, "split sensors", st));
-  PAT_TRY(alloc_n(p, &p->d_part, (size_t)4 * p->nsplit * p->nt, "split sensor parts"));
-  std::vector<int> samp_ptr(p->ntiles + 1, 0);
+  const Groups by_tile(p->ntiles, tile_of);
   std::vector<SampEntry> samp;
-  for (int t = 0; t < p->ntiles; ++t) {
-    samp_ptr[t] = (int)samp.size();
-    samp.insert(samp.end(), per_tile[t].begin(), per_tile[t].end());
-  }
-  samp_ptr[p->ntiles] = (int)samp.size();
+  samp.reserve(entry.size());
+  for (int i : by_tile.items) samp.push_back(entry[i]);
 
   // injected cells grouped by tile (large tiles: frame, then interior)
   const int nlist = large ? 2 : 1, edge = persist2dl_edge();
-  std::vector<std::vector<InjCell>> inj_tile((size_t)nlist * p->ntiles);
+  std::vector<int> list_of(p->n_inj);
+  std::vector<InjCell> cell(p->n_inj), inj;
   for (int i = 0; i < p->n_inj; ++i) {
     const int c = p->h_inj_cell[i];
-    const int cx = c % nx, cy = c / nx;
-    const int tile = (cy / TY) * p->tiles_x + cx / TX;
-    InjCell ic;
-    ic.local = (cy % TY) * TX + (cx % TX);
-    ic.beg = p->h_inj_ptr[i];
-    ic.end = p->h_inj_ptr[i + 1];
-    const int lx = cx % TX, ly = cy % TY;
+    const int cx = c % nx, cy = c / nx, lx = cx % TX, ly = cy % TY;
     const bool inner = lx >= edge && lx < TX - edge && ly >= edge && ly < TY - edge;
-    inj_tile[(size_t)nlist * tile + (large && inner ? 1 : 0)].push_back(ic);
+    cell[i] = InjCell{ly * TX + lx, p->h_inj_ptr[i], p->h_inj_ptr[i + 1]};
+    list_of[i] = nlist * ((cy / TY) * p->tiles_x + cx / TX) + (large && inner ? 1 : 0);
   }
-  std::vector<int> inj_ptr(1, 0);
-  std::vector<InjCell> inj;
-  for (const auto& cells : inj_tile) {
-    inj.insert(inj.end(), cells.begin(), cells.end());
-    inj_ptr.push_back((int)inj.size());
-  }
+  const Groups by_list(nlist * p->ntiles, list_of);
+  inj.reserve(cell.size());
+  for (int i : by_list.items) inj.push_back(cell[i]);
 
-  PAT_TRY(upload(p, &p->d_tile_samp_ptr, samp_ptr, "tile sampling offsets", st));
-  PAT_TRY(upload(p, &p->d_samp, samp, "tile sampling entries", st));
-  PAT_TRY(upload(p, &p->d_tile_inj_ptr, inj_ptr, "tile injection offsets", st));
-  PAT_TRY(upload(p, &p->d_tinj, inj, "tile injection cells", st));
+  arena.array(&p->d_split_sensor, split_sensor);
+  arena.array(&p->d_part, (size_t)4 * p->nsplit * p->nt);
+  arena.array(&p->d_tile_samp_ptr, by_tile.ptr);
+  arena.array(&p->d_samp, samp);
+  arena.array(&p->d_tile_inj_ptr, by_list.ptr);
+  arena.array(&p->d_tinj, inj);
   // tagged exchange words, invalidated (0xff bytes) before every launch
   p->xbuf_bytes = (large ? persist2dl_xbuf_words(p->ntiles) : persist2d_xbuf_words(p->R, p->ntiles)) * 8;
-  PAT_TRY(plan_alloc(p, &p->d_xbuf, p->xbuf_bytes, "exchange strips"));
+  arena.array(reinterpret_cast<char**>(&p->d_xbuf), p->xbuf_bytes);
   if (const char* e = getenv("PAT_POLL_NS")) p->poll_ns = std::max(0, atoi(e));
-  PAT_TRY(alloc_n(p, &p->d_abort, 1, "abort flag"));
-  return PAT_OK;
+  arena.array(&p->d_abort, 1);
 }
 
 static pat_status create(const pat_grid* grid, const double* c, double c0, const double* sensors, int ns, double dt,
@@ -458,12 +510,13 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
     return v;
   };
   const std::vector<int> sens_cell = pitched_cells(p->h_sens_cell), inj_cell = pitched_cells(p->h_inj_cell);
-  PAT_TRY(upload(p, &p->d_sens_cell, sens_cell, "sensor cells", st));
-  PAT_TRY(upload(p, &p->d_sens_w, p->h_sens_w, "sensor weights", st));
-  PAT_TRY(upload(p, &p->d_inj_cell, inj_cell, "injection cells", st));
-  PAT_TRY(upload(p, &p->d_inj_ptr, p->h_inj_ptr, "injection offsets", st));
-  PAT_TRY(upload(p, &p->d_ent_sensor, ent_sensor, "injection sensors", st));
-  PAT_TRY(upload(p, &p->d_ent_w, ent_w, "injection weights", st));
+  Arena arena, lists;
+  arena.array(&p->d_sens_cell, sens_cell);
+  arena.array(&p->d_sens_w, p->h_sens_w);
+  arena.array(&p->d_inj_cell, inj_cell);
+  arena.array(&p->d_inj_ptr, p->h_inj_ptr);
+  arena.array(&p->d_ent_sensor, ent_sensor);
+  arena.array(&p->d_ent_w, ent_w);
 
   // ---- wavelet filters
   p->family = wav->family;
@@ -482,26 +535,20 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
 
   // ---- workspace
   const size_t N = (size_t)p->N;
-  for (int i = 0; i < (p->dim == 2 ? 6 : 3); ++i) PAT_TRY(alloc_n(p, &p->d_wv[i], (size_t)p->Np, "wave fields"));
-  PAT_TRY(alloc_n(p, &p->d_dwt_a, N >> p->dim, "dwt approximation"));
-  PAT_TRY(alloc_n(p, &p->d_dwt_b, N >> p->dim, "dwt approximation"));
+  for (int i = 0; i < (p->dim == 2 ? 6 : 3); ++i) arena.array(&p->d_wv[i], (size_t)p->Np);
+  arena.array(&p->d_dwt_a, N >> p->dim);
+  arena.array(&p->d_dwt_b, N >> p->dim);
   if (p->dim == 3) {
-    PAT_TRY(alloc_n(p, &p->d_dwt_t1, N, "dwt pass buffer"));
-    PAT_TRY(alloc_n(p, &p->d_dwt_t2, N, "dwt pass buffer"));
+    arena.array(&p->d_dwt_t1, N);
+    arena.array(&p->d_dwt_t2, N);
   }
-  PAT_TRY(alloc_n(p, &p->d_r, N, "cg r"));
-  PAT_TRY(alloc_n(p, &p->d_p, N, "cg p"));
-  PAT_TRY(alloc_n(p, &p->d_q, N, "cg q"));
-  PAT_TRY(alloc_n(p, &p->d_img, N, "image buffer"));
-  PAT_TRY(alloc_n(p, &p->d_u, N, "cg u"));
-  PAT_TRY(alloc_n(p, &p->d_ybuf, (size_t)ns * nt, "sensor data buffer"));
-  PAT_TRY(alloc_n(p, &p->d_sc, 1, "cg scalars"));
-  PAT_TRY(alloc_n(p, &p->d_partials, (size_t)cg_grid_blocks(), "cg partials"));
-  PAT_TRY(alloc_n(p, &p->d_counter, 1, "cg counter"));
-  PAT_TRY(alloc_n(p, &p->d_status, 1, "status"));
-  PAT_TRY_CUDA(cudaMemsetAsync(p->d_counter, 0, sizeof(unsigned), st));
-  PAT_TRY_CUDA(cudaMemsetAsync(p->d_status, 0, sizeof(int), st));
-  PAT_TRY_CUDA(cudaMemsetAsync(p->d_sc, 0, sizeof(CgScalars), st));
+  for (float** v : {&p->d_r, &p->d_p, &p->d_q, &p->d_img, &p->d_u}) arena.array(v, N);
+  arena.array(&p->d_ybuf, (size_t)ns * nt);
+  arena.zeros(&p->d_sc, 1);
+  arena.array(&p->d_partials, (size_t)cg_grid_blocks());
+  arena.zeros(&p->d_counter, 1);
+  arena.zeros(&p->d_status, 1);
+  PAT_TRY(arena.commit(p, "sensor lists and workspace", st));
 
   // ---- engine choice: the persistent kernel when all tiles can be co-resident
   p->persist_ok = false;
@@ -519,7 +566,7 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
       p->persist_ok = p->persist_large = tiles(persist2dl_tile_x(), persist2dl_tile_y()) <= cap &&
                                          tiles(TX, TY) > (long long)persist2dl_min_tiles(p->R, p->varc) * sms;
     }
-    if (p->persist_ok) PAT_TRY(setup_persistent(p, st));
+    if (p->persist_ok) setup_persistent(p, lists);
   }
   p->path = p->persist_ok ? PAT_PATH_PERSISTENT : PAT_PATH_STEP;
   const char* env_path = getenv("PAT_WAVE_PATH");
@@ -541,23 +588,20 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
     int TX, TY;
     tma2d_tile(&TX, &TY);
     const int tx = (nx + TX - 1) / TX, ty = (ny + TY - 1) / TY;
-    std::vector<std::vector<InjCell>> bins((size_t)(p->tma3d ? p->tma3d_split.nctas : tx * ty));
+    std::vector<int> bin(p->n_inj);
     for (int i = 0; i < p->n_inj; ++i) {
       const long long c = p->h_inj_cell[i];
       const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-      const int bin = p->tma3d ? tma3d_cta_of(nx, ny, nz, p->tma3d_split, x, y, z) : (y / TY) * tx + x / TX;
-      bins[bin].push_back(InjCell{inj_cell[i], p->h_inj_ptr[i], p->h_inj_ptr[i + 1]});
+      bin[i] = p->tma3d ? tma3d_cta_of(nx, ny, nz, p->tma3d_split, x, y, z) : (y / TY) * tx + x / TX;
     }
-    std::vector<int> ptr(1, 0);
+    const Groups by_bin(p->tma3d ? p->tma3d_split.nctas : tx * ty, bin);
     std::vector<InjCell> cells;
-    for (auto& b : bins) {
-      cells.insert(cells.end(), b.begin(), b.end());
-      ptr.push_back((int)cells.size());
-    }
-    PAT_TRY(upload(p, &p->d_tinj_step_ptr, ptr, "injection lists of the step kernels", st));
-    PAT_TRY(upload(p, &p->d_tinj_step, cells, "injection lists of the step kernels", st));
-    PAT_TRY_CUDA(cudaStreamSynchronize(st));  // the host vectors go out of scope
+    cells.reserve(bin.size());
+    for (int i : by_bin.items) cells.push_back(InjCell{inj_cell[i], p->h_inj_ptr[i], p->h_inj_ptr[i + 1]});
+    lists.array(&p->d_tinj_step_ptr, by_bin.ptr);
+    lists.array(&p->d_tinj_step, cells);
   }
+  PAT_TRY(lists.commit(p, "lists of the wave engines", st));
   PAT_TRY_CUDA(cudaStreamSynchronize(st));
   return PAT_OK;
 }

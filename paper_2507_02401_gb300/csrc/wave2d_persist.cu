@@ -654,8 +654,11 @@ size_t persist2d_xbuf_words(int R, int ntiles, int nr) {
 }
 
 int persist2d_max_ctas(int R, bool adj, bool varc) {
-  const int fit = resident(pick(R, adj, varc, false, 1), R, adj);
-  return R == 1 ? std::max(fit, resident(pick(R, adj, varc, false, 2), R, adj)) : fit;
+  static PerDevice kept[kMaxR + 1][2][2];
+  return kept[R][adj][varc].get(current_device(), [&] {
+    const int fit = resident(pick(R, adj, varc, false, 1), R, adj);
+    return R == 1 ? std::max(fit, resident(pick(R, adj, varc, false, 2), R, adj)) : fit;
+  });
 }
 
 cudaError_t persist2d_launch(int R, bool adj, bool varc, bool layer, const Persist2DArgs& a, int nctas,

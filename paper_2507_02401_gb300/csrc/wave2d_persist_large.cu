@@ -476,20 +476,24 @@ int persist2dl_edge() { return EDGE; }
 size_t persist2dl_xbuf_words(int ntiles) { return (size_t)ntiles * 2 * 2 * RUN * NFRAME; }
 
 int persist2dl_max_ctas(int R, bool adj, bool varc) {
-  int best = 0;
-  for (int layer = 0; layer < 2; ++layer) {
-    void* f = pick(R, adj, varc, layer);
-    int dev = 0, sms = 0, per_sm = 0;
-    if (!f || cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(R, adj, varc)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, NTHREADS, smem_bytes(R, adj, varc)) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
+  static PerDevice kept[kMaxR + 1][2][2];
+  return kept[R][adj][varc].get(current_device(), [&] {
+    int best = 0;
+    for (int layer = 0; layer < 2; ++layer) {
+      void* f = pick(R, adj, varc, layer);
+      int dev = 0, sms = 0, per_sm = 0;
+      const size_t smem = smem_bytes(R, adj, varc);
+      if (!f || cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+          cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, NTHREADS, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+      }
+      best = layer == 0 || sms * per_sm < best ? sms * per_sm : best;
     }
-    best = layer == 0 || sms * per_sm < best ? sms * per_sm : best;
-  }
-  return best;
+    return best;
+  });
 }
 
 // Where this kernel beats a launch per step, in 64 x 32 tiles per SM (the per-step kernel's time goes up with every

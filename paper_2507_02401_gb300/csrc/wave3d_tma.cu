@@ -348,26 +348,30 @@ int smem_for(int R) {
   return (int)(R == 1 ? G3<1>::SMEM : R == 3 ? G3<3>::SMEM : R == 5 ? G3<5>::SMEM : G3<7>::SMEM);
 }
 
-// Co-resident CTAs of the step kernel (with and without injection and ring) on the current device; sets the
-// kernels' shared-memory attribute.
+// Co-resident CTAs of the step kernel (with and without injection and ring) on the current device; the first call
+// sets the kernels' shared-memory attribute.
 int resident(int R, bool varc) {
-  int dev = 0, sms = 0, best = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  for (int v = 0; v < 4; ++v) {
-    const KernelFn fn = kernel_for(R, v & 1, v & 2, varc);
-    int per = 0;
-    if (!fn ||
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_for(R)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, THREADS, smem_for(R)) != cudaSuccess) {
+  static PerDevice kept[kMaxR + 1][2];
+  return kept[R][varc].get(current_device(), [&] {
+    int dev = 0, sms = 0, best = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
-    best = v == 0 || per < best ? per : best;
-  }
-  return sms * best;
+    for (int v = 0; v < 4; ++v) {
+      const KernelFn fn = kernel_for(R, v & 1, v & 2, varc);
+      int per = 0;
+      if (!fn ||
+          cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_for(R)) != cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, THREADS, smem_for(R)) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+      }
+      best = v == 0 || per < best ? per : best;
+    }
+    return sms * best;
+  });
 }
 
 }  // namespace
