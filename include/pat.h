@@ -315,13 +315,15 @@ pat_status pat_batch_launch(pat_batch* batch, int mode, int* runall, double* ms)
  *   g = sum_{n=1}^{nt-2} Q^{n+1} .* L P^n + 1/2 Q^1 .* L P^0.
  * The forward fields are needed in reverse order: the forward run keeps its
  * restart state every `segment` steps (0 = ceil(sqrt(nt)), in 2D as many more
- * as 1 GiB of segment memory holds where that is free) and each segment but the
- * last is recomputed when the adjoint reaches it.  Runs on the per-step engine.
+ * as 1 GiB of segment memory holds) and each segment but the last is recomputed
+ * when the adjoint reaches it.  Runs on the per-step engine.
  *   x  N floats;  r  ns*nt floats;  g  N floats (output).
  * Memory: (2 ceil((nt-1)/segment) + segment + 3) N floats + N doubles,
  * allocated by the first call and kept by the plan (PAT_ERR_OOM if absent).
- * The segment granted to the first call with 0 is the one of every later such
- * call: these allocate nothing and may be captured.
+ * The longer segments of calls with 0 take at most 4 GiB over all plans of a
+ * device and an eighth of what is free; a caller that wants the memory names
+ * `segment`.  The segment granted to the first call with 0 is the one of every
+ * later such call: these allocate nothing and may be captured.
  */
 pat_status pat_grad_kappa(pat_plan* plan, const float* x, const float* r, float* g, int segment, void* stream);
 

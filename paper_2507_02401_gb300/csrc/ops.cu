@@ -1,5 +1,6 @@
 // Operators and solver behind the C ABI: K, K*, E_s, E_s*, CG.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 
@@ -519,7 +520,32 @@ pat_status apply_Es(pat_plan* p, double s, const float* u, float* x, cudaStream_
 // keeps the restart state every C steps, the adjoint runs backwards and, for
 // each segment it reaches, the segment's fields are recomputed from its
 // checkpoint so that L P^n is available in reverse order.
-static void kg_free(pat_plan* p) {
+//
+// A default segment may be longer (see kappa_grad_device).  That is a loan: over all plans on a device at most
+// kLongTotal bytes, and never more than an eighth of what is free when it is taken, so that several plans, or a
+// program that fills the device, do not find their memory gone; given back when the plan goes or its buffers are
+// replaced.
+static constexpr long long kLongSegment = 1LL << 30, kLongTotal = 4LL << 30;
+static std::atomic<long long> g_long_lent[PerDevice::kDevices];
+
+static bool kg_borrow(pat_plan* p, long long bytes) {
+  const int dev = current_device();
+  size_t free_bytes = 0, total = 0;
+  if (dev < 0 || dev >= PerDevice::kDevices || cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (bytes > (long long)(free_bytes / 8)) return false;
+  if (g_long_lent[dev].fetch_add(bytes) + bytes > kLongTotal) {
+    g_long_lent[dev].fetch_sub(bytes);
+    return false;
+  }
+  p->kg_lent = bytes;
+  p->kg_lent_dev = dev;
+  return true;
+}
+
+void kg_free(pat_plan* p) {
   cudaFree(p->kg_ckpt);
   cudaFree(p->kg_seg);
   cudaFree(p->kg_work);
@@ -527,11 +553,11 @@ static void kg_free(pat_plan* p) {
   p->kg_ckpt = p->kg_seg = p->kg_work = nullptr;
   p->kg_acc = nullptr;
   p->kg_segment = 0;
+  if (p->kg_lent > 0) g_long_lent[p->kg_lent_dev].fetch_sub(p->kg_lent);
+  p->kg_lent = 0;
 }
 
 static pat_status kg_alloc(pat_plan* p, int C, int nseg) {
-  if (p->kg_segment == C) return PAT_OK;
-  kg_free(p);
   const size_t N = (size_t)p->Np;
   cudaError_t e = cudaMalloc(&p->kg_ckpt, sizeof(float) * N * 2 * nseg);
   if (e == cudaSuccess) e = cudaMalloc(&p->kg_seg, sizeof(float) * N * C);
@@ -645,19 +671,23 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
   } else if (by_default) {
     C = root;
     if (p->tma2d) {
-      C = (int)std::min<long long>(nt - 1, std::max<long long>(root, (1LL << 28) / N));
+      C = (int)std::min<long long>(nt - 1, std::max<long long>(root, kLongSegment / (long long)sizeof(float) / N));
       C = (nt - 2) / ((nt - 2) / C + 1) + 1;  // equal segments: the last, kept one is as long as the others
     }
   }
   if (C > nt - 1) C = nt - 1;
   auto segments = [&] { return (nt - 2) / C + 1; };  // of n = 0 .. nt-2
-  pat_status rc = kg_alloc(p, C, segments());
-  if (rc != PAT_OK && by_default && C > root) {
-    C = root;
-    rc = kg_alloc(p, C, segments());
+  if (p->kg_segment != C) {
+    kg_free(p);
+    if (by_default && C > root && !kg_borrow(p, (long long)sizeof(float) * N * C)) C = root;
+    pat_status rc = kg_alloc(p, C, segments());
+    if (rc != PAT_OK && by_default && C > root) {
+      C = root;
+      rc = kg_alloc(p, C, segments());
+    }
+    PAT_TRY(rc);
   }
-  if (rc == PAT_OK && by_default) p->kg_default = C;
-  PAT_TRY(rc);
+  if (by_default) p->kg_default = C;
   const bool two_d = p->dim == 2;
   float* W0 = p->kg_work;
   float* W1 = p->kg_work + N;

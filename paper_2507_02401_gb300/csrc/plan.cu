@@ -642,10 +642,7 @@ void pat_plan_destroy(pat_plan* plan) {
   for (int i = 0; i < 4; ++i)
     if (plan->d_stage[i]) cudaFree(plan->d_stage[i]);
   for (cudaEvent_t e : plan->prof_ev) cudaEventDestroy(e);
-  cudaFree(plan->kg_ckpt);
-  cudaFree(plan->kg_seg);
-  cudaFree(plan->kg_work);
-  cudaFree(plan->kg_acc);
+  kg_free(plan);
   delete plan;
 }
 

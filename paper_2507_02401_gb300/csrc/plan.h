@@ -114,6 +114,8 @@ struct pat_plan {
   // ---- medium-gradient workspace (allocated by the first pat_grad_kappa call)
   int kg_segment = 0;           // checkpoint interval the buffers were sized for
   int kg_default = 0;           // interval granted to the first call that named none (0: no such call yet)
+  long long kg_lent = 0;        // bytes of a long default segment (0: none), and the device they count on
+  int kg_lent_dev = 0;
   float* kg_ckpt = nullptr;     // per checkpoint: two fields (P and D, or P and P^{n-1})
   float* kg_seg = nullptr;      // one segment of recomputed fields
   float* kg_work = nullptr;     // forward-pass fields (3 x N)
@@ -138,6 +140,7 @@ pat_status apply_EsT(pat_plan* p, double s, const float* x, float* u, cudaStream
 pat_status solve_device(pat_plan* p, const float* y, double alpha, double s, int iters, const float* u0, float* u,
                         float* x, double* log, cudaStream_t st);
 pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float* g, int segment, cudaStream_t st);
+void kg_free(pat_plan* p);  // the medium gradient's buffers
 bool fourier_supported(int dim, int nx, int ny);
 pat_status fourier_setup(pat_plan* p, double length_cells, cudaStream_t st);
 pat_status fourier_apply(pat_plan* p, double s, const float* in, float* out, cudaStream_t st);

@@ -1,5 +1,5 @@
 """Memory of the medium gradient: what the first call was granted serves the
-later ones."""
+later ones, and the long default segments stay within their bounds."""
 import numpy as np
 import pytest
 
@@ -48,3 +48,50 @@ def test_default_segment_is_kept_when_the_long_one_does_not_fit():
     # room again: an explicit segment still replaces the buffers, and the default comes back
     assert torch.equal(plan.grad_kappa(x, r, segment=100), ref)
     assert torch.equal(plan.grad_kappa(x, r), ref)
+
+
+def gradient_bytes(torch, plan, x, r):
+    """Device memory that the plan's first default call takes for good."""
+    free = torch.cuda.mem_get_info()[0]
+    plan.grad_kappa(x, r)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return free - torch.cuda.mem_get_info()[0]
+
+
+def test_default_segments_of_many_plans_are_bounded():
+    """One plan takes 1 GiB for its long segment here; ten take 4 GiB between
+    them and sqrt(nt) segments beyond that (under 0.35 GB each), with the same
+    bits; what one gives back the next may take."""
+    torch = need_gpu()
+    w = custom((1024, 1024), 257, 2, False, 16, seed=5)
+    x = torch.as_tensor(w.x_true, dtype=torch.float32, device="cuda")
+    r = torch.as_tensor(np.random.default_rng(5).standard_normal((w.ns, w.nt)), dtype=torch.float32, device="cuda")
+    plans = [make_pair(w)[0] for _ in range(10)]
+    used = [gradient_bytes(torch, p, x, r) for p in plans]
+    assert used[0] > 1 << 30
+    assert sum(used) <= (4 << 30) + 10 * 350e6
+    assert torch.equal(plans[0].grad_kappa(x, r), plans[-1].grad_kappa(x, r))
+    for p in plans:
+        p.close()
+    again = make_pair(w)[0]
+    assert gradient_bytes(torch, again, x, r) > 1 << 30
+    again.grad_kappa(x, r, segment=16)  # gives its long segment back as well
+    rest = [make_pair(w)[0] for _ in range(3)]
+    assert all(gradient_bytes(torch, p, x, r) > 1 << 30 for p in rest)
+
+
+def test_default_segment_leaves_a_full_device_alone():
+    """With 4 GB free the default is sqrt(nt): an eighth of that is less than the long segment."""
+    torch = need_gpu()
+    w = custom((1024, 1024), 257, 2, False, 16, seed=5)
+    x = torch.as_tensor(w.x_true, dtype=torch.float32, device="cuda")
+    r = torch.as_tensor(np.random.default_rng(5).standard_normal((w.ns, w.nt)), dtype=torch.float32, device="cuda")
+    plan = make_pair(w)[0]
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (4 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        assert gradient_bytes(torch, plan, x, r) < 350e6
+    finally:
+        del fill
+        torch.cuda.empty_cache()
