@@ -1038,11 +1038,6 @@ __global__ void dwt1d_synthesis_kernel(const float* __restrict__ lo, const float
   }
 }
 
-__global__ void scale_copy_kernel(float* __restrict__ d, const float* __restrict__ s, long long n, float w) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    d[i] = w * s[i];
-}
-
 Filt make_filt(const float* h, const float* g, int L) {
   Filt f{};
   for (int j = 0; j < L; ++j) {
@@ -1142,12 +1137,6 @@ cudaError_t dwt3d_synthesis_level(const float* const bands[8], float wdet, int n
   if (L == 2) return launch_s3<2>(st, b, wdet, nx, ny, nz, out, f);
   if (L == 4) return launch_s3<4>(st, b, wdet, nx, ny, nz, out, f);
   return launch_s3<8>(st, b, wdet, nx, ny, nz, out, f);
-}
-
-cudaError_t scale_copy_launch(float* dst, const float* src, long long n, float w, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  scale_copy_kernel<<<grid1d(n), 256, 0, st>>>(dst, src, n, w);
-  return cudaGetLastError();
 }
 
 }  // namespace pat

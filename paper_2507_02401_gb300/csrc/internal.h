@@ -236,7 +236,6 @@ cudaError_t grad_finish_launch(float* g, const float* hi, const float* lo, const
 cudaError_t d2f_launch(float* out, const double* in, long long n, cudaStream_t st);
 cudaError_t dfill_launch(double* p, long long n, cudaStream_t st);
 cudaError_t fill_launch(float* p, long long n, float v, cudaStream_t st);
-cudaError_t copy_launch(float* dst, const float* src, long long n, cudaStream_t st);
 
 // dwt.cu
 cudaError_t dwt2d_analysis_level(const float* in, int nx, int ny, float* approx, float* bandH, float* bandV,
@@ -255,7 +254,6 @@ cudaError_t dwt3d_analysis_level(const float* in, int nx, int ny, int nz, float*
                                  const float* h, const float* g, int L, cudaStream_t st);
 cudaError_t dwt3d_synthesis_level(const float* const bands[8], float wdet, int nx, int ny, int nz, float* out,
                                   const float* h, const float* g, int L, cudaStream_t st);
-cudaError_t scale_copy_launch(float* dst, const float* src, long long n, float w, cudaStream_t st);
 
 // cg.cu
 struct CgScalars {

@@ -779,7 +779,7 @@ pat_status kappa_grad_device(pat_plan* p, const float* x, const float* r, float*
     const int n = m - 1;
     if (n / C != loaded) PAT_TRY(load_segment(n / C));
     PAT_TRY_CUDA(grad_acc_launch(p->R, p->kg_acc, Q, Qlo, seg(n - loaded * C), n == 0 ? 0.5f : 1.f, a, p->dim,
-                                 two_d ? p->tma2d : p->tma3d && p->varc, st));
+                                 !two_d && p->tma3d && p->varc, st));
     return PAT_OK;
   };
   PAT_TRY_CUDA(dfill_launch(p->kg_acc, p->N, st));

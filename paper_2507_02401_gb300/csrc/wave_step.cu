@@ -269,11 +269,6 @@ __global__ void fill_kernel(float* p, long long n, float v) {
     p[i] = v;
 }
 
-__global__ void copy_kernel(float* __restrict__ d, const float* __restrict__ s, long long n) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    d[i] = s[i];
-}
-
 __global__ void pitch_copy_kernel(float* __restrict__ d, int dpitch, const float* __restrict__ s, int spitch, int nx,
                                   long long rows) {
   const long long n = rows * nx;
@@ -359,12 +354,6 @@ cudaError_t fill_launch(float* p, long long n, float v, cudaStream_t st) {
 cudaError_t pitch_copy_launch(float* d, int dpitch, const float* s, int spitch, int nx, long long rows,
                               cudaStream_t st) {
   pitch_copy_kernel<<<grid_for(rows * nx), 256, 0, st>>>(d, dpitch, s, spitch, nx, rows);
-  return cudaGetLastError();
-}
-
-cudaError_t copy_launch(float* d, const float* s, long long n, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  copy_kernel<<<grid_for(n), 256, 0, st>>>(d, s, n);
   return cudaGetLastError();
 }
 
