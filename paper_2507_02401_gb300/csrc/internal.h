@@ -206,15 +206,18 @@ cudaError_t step3d_tma_launch(int R, const StepArgs& a, const CUtensorMap& cur, 
 
 // wave2d_tma.cu: 2D increment-form step with TMA tile pipelines
 bool tma2d_supported(int R);
-void tma2d_tile(int* tx, int* ty);  // tile extents in cells (tiles numbered row by row)
-// halo boxes (80 x (32+2R)) of an nx x ny float field of row pitch `pitch`
-cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CUtensorMap* halo);
+// Plain: 64 x 32 tiles.  Full: the same with the forward stencil in the difference form and the adjoint's G compensated
+// in a.dbuf_lo.  Tall: 64 x 64 tiles, forward only.
+enum class Form2d { Plain, Full, Tall };
+void tma2d_tile(int* tx, int* ty);  // tile extents in cells (tiles numbered row by row), Plain and Full
+bool tma2d_tall(int pitch, long long cells);  // whether a grid's plain forward steps take the tall form
+// halo boxes (80 x (32+2R), tall 80 x (64+2R)) of an nx x ny float field of row pitch `pitch`
+cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, bool tall, CUtensorMap* halo);
 // mode 0: forward, constant medium; 1: forward, varying medium; 2: adjoint (either medium); 3: adjoint with the
 // medium gradient's sum (sp 0);
-// sp 0: no absorbing layer, 1: layer with the forward update, 2: layer with the adjoint update;
-// full: forward stencil in the difference form, adjoint with G compensated in a.dbuf_lo
-long long tma2d_threads(int nx, int ny, int R, int mode, int sp, bool full);  // threads of one launch
-cudaError_t step2d_tma_launch(int R, int mode, int sp, bool full, const StepArgs& a, const CUtensorMap& p,
+// sp 0: no absorbing layer, 1: layer with the forward update, 2: layer with the adjoint update
+long long tma2d_threads(int nx, int ny, int R, int mode, int sp, Form2d form);  // threads of one launch
+cudaError_t step2d_tma_launch(int R, int mode, int sp, Form2d form, const StepArgs& a, const CUtensorMap& p,
                               const CUtensorMap& lo, int* status, long long timeout_ns, cudaStream_t st);
 
 // wave_step.cu

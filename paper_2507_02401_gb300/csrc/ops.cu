@@ -97,8 +97,11 @@ static const pat_plan::TmaDesc* tma_desc(pat_plan* p, const float* base) {
   pat_plan::TmaDesc d;
   d.base = base;
   const cudaError_t e = p->dim == 3 ? tma3d_encode(base, p->n[0], p->pitch, p->n[1], p->n[2], p->R, &d.halo, &d.own)
-                                     : tma2d_encode(base, p->n[0], p->pitch, p->n[1], p->R, &d.halo);
+                                     : tma2d_encode(base, p->n[0], p->pitch, p->n[1], p->R, false, &d.halo);
   if (e != cudaSuccess) return nullptr;
+  if (p->dim == 2 && p->tall &&
+      tma2d_encode(base, p->n[0], p->pitch, p->n[1], p->R, true, &d.own) != cudaSuccess)
+    return nullptr;
   if (p->tma_desc.size() >= 16) p->tma_desc.erase(p->tma_desc.begin());
   p->tma_desc.push_back(d);
   return &p->tma_desc.back();
@@ -131,16 +134,16 @@ static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t 
     // compensated (boxes of Z and Z_lo), the next step's injection added to G after each tile
     const int mode = adj ? (a.gsum_hi ? 3 : 2) : (p->varc ? 1 : 0);
     const int sp = p->sponge_w > 0 ? (adj ? 2 : 1) : 0;
-    // odd widths used to take the plain kernel, whose forward stencil is the difference form and whose adjoint
-    // carries G as a compensated pair: the kernel's full form keeps that accuracy
-    // (as did the medium gradient's L P, whose difference form comes with the full forward)
+    // rows of no multiple of 4 cells, and the medium gradient's L P, take the full form: the difference form of the
+    // forward stencil, G as a compensated pair in the adjoint
     const bool full = p->n[0] % 4 != 0 || (!adj && a.full);
-    const long long nthr = tma2d_threads(p->n[0], p->n[1], p->R, mode, sp, full);
+    const Form2d form = full ? Form2d::Full : !adj && p->tall ? Form2d::Tall : Form2d::Plain;
+    const long long nthr = tma2d_threads(p->n[0], p->n[1], p->R, mode, sp, form);
     if (y && a.ns > nthr) a.y = nullptr;
     // copies: a second lookup may move the cached descriptors
     const pat_plan::TmaDesc* dp = tma_desc(p, a.cur);
     if (!dp) return cudaErrorInvalidValue;
-    const CUtensorMap mcur = dp->halo;
+    const CUtensorMap mcur = form == Form2d::Tall ? dp->own : dp->halo;
     CUtensorMap mlo = mcur;
     if (adj) {
       const pat_plan::TmaDesc* dl = tma_desc(p, a.cur_lo);
@@ -153,7 +156,7 @@ static cudaError_t step_launch(pat_plan* p, bool adj, StepArgs& a, cudaStream_t 
     b.inj_tile = p->d_tinj_step;
     b.ent_sensor = p->d_ent_sensor;
     b.ent_w = p->d_ent_w;
-    e = step2d_tma_launch(p->R, mode, sp, full, b, mcur, mlo, p->d_status, p->timeout_ns, st);
+    e = step2d_tma_launch(p->R, mode, sp, form, b, mcur, mlo, p->d_status, p->timeout_ns, st);
   } else if (p->dim == 2) {
     const long long nthr = (long long)((p->n[0] + 63) / 64) * ((p->n[1] + 31) / 32) * 256;
     if (y && a.ns > nthr) a.y = nullptr;

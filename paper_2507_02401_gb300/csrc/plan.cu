@@ -575,7 +575,8 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
   p->tma2d = p->tma3d = false;
   if (tma && p->dim == 2) {
     CUtensorMap mh;
-    p->tma2d = tma2d_encode(p->d_wv[0], p->n[0], p->pitch, p->n[1], p->R, &mh) == cudaSuccess;
+    p->tma2d = tma2d_encode(p->d_wv[0], p->n[0], p->pitch, p->n[1], p->R, false, &mh) == cudaSuccess;
+    p->tall = p->tma2d && !p->varc && tma2d_tall(p->pitch, p->N);
   } else if (tma) {
     CUtensorMap mc, mp;
     if (tma3d_encode(p->d_wv[0], p->n[0], p->pitch, p->n[1], p->n[2], p->R, &mc, &mp) == cudaSuccess) {

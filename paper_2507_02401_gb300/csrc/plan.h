@@ -67,11 +67,12 @@ struct pat_plan {
   bool tma3d = false;  // 3D steps through the TMA plane-pipeline kernel
   pat::Tma3dSplit tma3d_split{0, 0};  // work split of a 3D TMA step launch
   bool tma2d = false;  // 2D steps through the TMA tile-pipeline kernel (where it applies)
-  int* d_tinj_step_ptr = nullptr;       // TMA step kernels: injection lists per tile (2D: 64 x 64 cells) or per
+  bool tall = false;   // its plain forward steps take 64 x 64 tiles
+  int* d_tinj_step_ptr = nullptr;       // TMA step kernels: injection lists per tile (2D: 64 x 32 cells) or per
   pat::InjCell* d_tinj_step = nullptr;  // CTA (3D: 64 x 16 columns x z range); .local = linear cell index
   struct TmaDesc {
     const float* base;
-    CUtensorMap halo, own;  // stencil-input boxes with halo; 3D: own-tile boxes
+    CUtensorMap halo, own;  // stencil-input boxes with halo; 3D: own-tile boxes, 2D: the tall tiles' boxes
   };
   std::vector<TmaDesc> tma_desc;  // descriptors by field address (small, most recent last)
 

@@ -49,20 +49,31 @@ namespace {
 //   4 columns x 8 rows, 64 x 64 tiles (2 to 3 CTAs)     40.0 / 93.1 | 6.8 / 16.6 | 5.8 / 9.5
 // The first needs the fewest shared-memory wavefronts per cell of those that leave 12 warps on an SM in the
 // adjoint, whose two stencils keep the FP32 and shared-memory pipes about half busy each.
-constexpr int TX = 64, TY = 32, NP = 2, TCOLS = TX / (2 * NP), RUN = 4;
-constexpr int THREADS = TCOLS * (TY / RUN);
+//
+// Forward steps of a constant medium, on rows of whole 128-byte lines and fields of 256 MiB or more, take tiles twice
+// as tall, a CTA of 256 threads each, two CTAs per SM: there DRAM is the bound, and it serves 64 rows of a tile better
+// than 32.  K us per step, tall | not: order 8 16384^2 653 | 786, 12000^2 350 | 386, 8192^2 159 | 161, 4096^2 41.8 |
+// 40.4; order 2 627 | 726, 339 | 378, 150 | 163, 37.2 | 35.1.  Rows that are no multiple of 128 bytes do not gain
+// (12000 x 12004 order 8 503 | 497), nor do varying media (12000^2 order 2 563 | 508) and the adjoint.
+constexpr int TX = 64, NP = 2, TCOLS = TX / (2 * NP), RUN = 4;
+__host__ __device__ constexpr int tile_y(bool tall) { return tall ? 64 : 32; }
+__host__ __device__ constexpr int threads_of(bool tall) { return TCOLS * (tile_y(tall) / RUN); }
 // CTAs per SM to leave registers for: a fourth pays up to order 4 (1024^2 order 4 K* 6.3 against 7.4 us), except
 // in the full form, which spills then (1000 x 875 order 4 K* 7.8 against 6.8 us)
-constexpr int min_ctas(int R, bool full, bool grad) { return grad ? 2 : R <= 3 && !full ? 4 : 3; }
+constexpr int min_ctas(int R, bool full, bool grad, bool tall) { return grad || tall ? 2 : R <= 3 && !full ? 4 : 3; }
 constexpr int XH = 8;            // box columns left of the tile (>= R, 16-byte aligned)
 constexpr int BW = TX + 2 * XH;  // box width, 80 floats
 
-template <int R, int NBOX = 1>
+template <int R, int NBOX = 1, bool TALL = false>
 struct G2 {
-  static constexpr int BH = TY + 2 * R;
+  static constexpr int BH = tile_y(TALL) + 2 * R;
   static constexpr int PBOX = BW * BH;       // floats (multiple of 32: 128-byte aligned)
   static constexpr int STAGE = NBOX * PBOX;  // the adjoint stages Z and Z_lo
-  static constexpr size_t SMEM = sizeof(float) * 2 * STAGE + 16;
+  static constexpr size_t USED = sizeof(float) * 2 * STAGE + 16;
+  // Tall tiles: two CTAs per SM and no room for a third, which the next step's grid, launched programmatically, would
+  // take on some SMs and leave others with one of its CTAs (order 2, whose registers leave that room: 12000^2 339 us
+  // per step so, 358 with it).
+  static constexpr size_t SMEM = TALL && R == 1 ? 100 * 1024 : USED;
 };
 
 // Sensor s = b + t * gridDim.x is sampled by thread t of CTA b (the sensors spread over every CTA).
@@ -86,12 +97,13 @@ __device__ __forceinline__ void fused_sample2(const StepArgs& a, long long bid, 
 // GRAD (adjoint): adds this step's term gcoef Z^m .* L P^{m-1} of the medium gradient to a compensated sum.
 // The sums are pairs of FP32 (TwoSum with the product's rounding error, ~2^-47): FP64 arithmetic runs at 2
 // operations per clock and SM here, and dividing by kappa once at the end replaces a division per step.
-template <int R, int MODE, int SP, bool FULL, bool GRAD = false>
-__global__ void __launch_bounds__(THREADS, min_ctas(R, FULL, GRAD)) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
+template <int R, int MODE, int SP, bool FULL, bool GRAD = false, bool TALL = false>
+__global__ void __launch_bounds__(threads_of(TALL), min_ctas(R, FULL, GRAD, TALL)) step2d_tma_kernel(const StepArgs a, const __grid_constant__ CUtensorMap mp,
                                                              const __grid_constant__ CUtensorMap ml, int* status,
                                                              long long timeout_ns) {
   constexpr bool VARC = MODE == 1, ADJ = MODE == 2;
-  using G = G2<R, ADJ ? 2 : 1>;
+  constexpr int TY = tile_y(TALL), THREADS = threads_of(TALL);
+  using G = G2<R, ADJ ? 2 : 1, TALL>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* stage0 = reinterpret_cast<float*>(smem_raw);
   uint64_t* bars = reinterpret_cast<uint64_t*>(stage0 + 2 * G::STAGE);
@@ -336,37 +348,58 @@ const void* kernel_r(int mode, int sp) {
   }
 }
 
-const void* kernel_for(int R, int mode, int sp, bool full) {
+template <int R>
+const void* kernel_tall(int mode, int sp) {  // forward, constant medium
+  if (mode != 0) return nullptr;
+  return sp == 0   ? reinterpret_cast<const void*>(&step2d_tma_kernel<R, 0, 0, false, false, true>)
+         : sp == 1 ? reinterpret_cast<const void*>(&step2d_tma_kernel<R, 0, 1, false, false, true>)
+                   : nullptr;
+}
+
+template <int R>
+const void* kernel_form(int mode, int sp, Form2d form) {
+  return form == Form2d::Tall ? kernel_tall<R>(mode, sp)
+         : form == Form2d::Full ? kernel_r<R, true>(mode, sp)
+                                : kernel_r<R, false>(mode, sp);
+}
+
+const void* kernel_for(int R, int mode, int sp, Form2d form) {
   switch (R) {
-    case 1: return full ? kernel_r<1, true>(mode, sp) : kernel_r<1, false>(mode, sp);
-    case 3: return full ? kernel_r<3, true>(mode, sp) : kernel_r<3, false>(mode, sp);
-    case 5: return full ? kernel_r<5, true>(mode, sp) : kernel_r<5, false>(mode, sp);
-    case 7: return full ? kernel_r<7, true>(mode, sp) : kernel_r<7, false>(mode, sp);
+    case 1: return kernel_form<1>(mode, sp, form);
+    case 3: return kernel_form<3>(mode, sp, form);
+    case 5: return kernel_form<5>(mode, sp, form);
+    case 7: return kernel_form<7>(mode, sp, form);
     default: return nullptr;
   }
 }
 
-size_t smem_for(int R, int mode) {
-  if (mode >= 2) return R == 1 ? G2<1, 2>::SMEM : R == 3 ? G2<3, 2>::SMEM : R == 5 ? G2<5, 2>::SMEM : G2<7, 2>::SMEM;
-  return R == 1 ? G2<1>::SMEM : R == 3 ? G2<3>::SMEM : R == 5 ? G2<5>::SMEM : G2<7>::SMEM;
+template <int R>
+size_t smem_r(int mode, Form2d form) {
+  return mode >= 2 ? G2<R, 2>::SMEM : form == Form2d::Tall ? G2<R, 1, true>::SMEM : G2<R>::SMEM;
+}
+
+size_t smem_for(int R, int mode, Form2d form) {
+  return R == 1 ? smem_r<1>(mode, form) : R == 3 ? smem_r<3>(mode, form) : R == 5 ? smem_r<5>(mode, form) : smem_r<7>(mode, form);
 }
 
 }  // namespace
 
 void tma2d_tile(int* tx, int* ty) {
   *tx = TX;
-  *ty = TY;
+  *ty = tile_y(false);
 }
+
+bool tma2d_tall(int pitch, long long cells) { return pitch % 32 == 0 && cells >= 1LL << 26; }
 
 bool tma2d_supported(int R) { return R == 1 || R == 3 || R == 5 || R == 7; }
 
-cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CUtensorMap* halo) {
+cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, bool tall, CUtensorMap* halo) {
   auto fn = tma_encoder();
   if (!fn) return cudaErrorNotSupported;
   const cuuint64_t dims[2] = {(cuuint64_t)nx, (cuuint64_t)ny};
   const cuuint64_t strides[1] = {(cuuint64_t)pitch * 4};
   const cuuint32_t estr[2] = {1, 1};
-  const cuuint32_t box_h[2] = {(cuuint32_t)BW, (cuuint32_t)(TY + 2 * R)};
+  const cuuint32_t box_h[2] = {(cuuint32_t)BW, (cuuint32_t)(tile_y(tall) + 2 * R)};
   const CUresult r = fn(halo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box_h, estr,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -374,42 +407,43 @@ cudaError_t tma2d_encode(const float* base, int nx, int pitch, int ny, int R, CU
 }
 
 // Persistent grid: as many CTAs as fit on the device, at most one per tile (0: the kernel does not run there).
-int tma2d_ctas(int nx, int ny, int R, int mode, int sp, bool full) {
-  static PerDevice resident[2][4][3][8];
-  const int fit = resident[full][mode][sp][R].get(current_device(), [&] {
+int tma2d_ctas(int nx, int ny, int R, int mode, int sp, Form2d form) {
+  static PerDevice resident[3][4][3][8];
+  const bool tall = form == Form2d::Tall;
+  const int fit = resident[(int)form][mode][sp][R].get(current_device(), [&] {
     int dev = 0, sms = 0, per = 0;
-    const void* fn = kernel_for(R, mode, sp, full);
-    const size_t smem = smem_for(R, mode);
+    const void* fn = kernel_for(R, mode, sp, form);
+    const size_t smem = smem_for(R, mode, form);
     if (!fn || cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, THREADS, smem) != cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads_of(tall), smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
     return per * sms;
   });
-  const int ntiles = ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
+  const int ntiles = ((nx + TX - 1) / TX) * ((ny + tile_y(tall) - 1) / tile_y(tall));
   return ntiles < fit ? ntiles : fit;
 }
 
-long long tma2d_threads(int nx, int ny, int R, int mode, int sp, bool full) {
-  return (long long)tma2d_ctas(nx, ny, R, mode, sp, full) * THREADS;
+long long tma2d_threads(int nx, int ny, int R, int mode, int sp, Form2d form) {
+  return (long long)tma2d_ctas(nx, ny, R, mode, sp, form) * threads_of(form == Form2d::Tall);
 }
 
-cudaError_t step2d_tma_launch(int R, int mode, int sp, bool full, const StepArgs& a, const CUtensorMap& p,
+cudaError_t step2d_tma_launch(int R, int mode, int sp, Form2d form, const StepArgs& a, const CUtensorMap& p,
                               const CUtensorMap& lo, int* status, long long timeout_ns, cudaStream_t st) {
-  const void* fn = kernel_for(R, mode, sp, full);
+  const void* fn = kernel_for(R, mode, sp, form);
   if (!fn) return cudaErrorInvalidValue;
-  const int nctas = tma2d_ctas(a.nx, a.ny, R, mode, sp, full);  // the first call sets the kernel's attributes
+  const int nctas = tma2d_ctas(a.nx, a.ny, R, mode, sp, form);  // the first call sets the kernel's attributes
   if (nctas <= 0) return cudaErrorInvalidConfiguration;
   CUtensorMap map = p, mapl = lo;
   StepArgs args = a;
   void* params[] = {&args, &map, &mapl, &status, &timeout_ns};
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(nctas);
-  cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = smem_for(R, mode);
+  cfg.blockDim = dim3(threads_of(form == Form2d::Tall));
+  cfg.dynamicSmemBytes = smem_for(R, mode, form);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];  // starts while the previous step drains (the kernel waits for it itself)
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
