@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(threads_of(TALL), min_ctas(R, FULL, GRAD, TALL
                                                              long long timeout_ns) {
   constexpr bool VARC = MODE == 1, ADJ = MODE == 2;
   constexpr int TY = tile_y(TALL), THREADS = threads_of(TALL);
+  constexpr bool ALL_K = VARC && R > 1 && !FULL;
   using G = G2<R, ADJ ? 2 : 1, TALL>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* stage0 = reinterpret_cast<float*>(smem_raw);
@@ -164,7 +165,9 @@ __global__ void __launch_bounds__(threads_of(TALL), min_ctas(R, FULL, GRAD, TALL
     const int gx0 = (tt % tiles_x) * TX, gy0 = (tt / tiles_x) * TY;
     const int gx = gx0 + c0;
     // own-cell fields straight into registers, in flight while the boxes land: D or G of every row; kappa
-    // and G_lo (fetch) two rows ahead of their use
+    // and G_lo (fetch) two rows ahead of their use, or, in the forward of a varying medium from order 4 on, kappa of
+    // every row as well (K us per step, all rows | two ahead: 12000^2 order 8 524 | 556, order 6 with a layer 540 |
+    // 609, 4096^2 order 8 57 | 62; order 2 530 | 494)
     Cells<NP> d2[RUN], kh2[RUN], kl2[RUN], gl2[RUN], lp2[RUN], sh2[RUN], sl2[RUN];
     // (the adjoint's final step takes kappa inside the layer; a partial tile has cells beyond the field, so every
     // access to a field by cell is under a test like fetch's)
@@ -192,7 +195,7 @@ __global__ void __launch_bounds__(threads_of(TALL), min_ctas(R, FULL, GRAD, TALL
       if (load_d && gy < ny && gx < nx) d2[rr].stream(a.dbuf + (long long)gy * pitch + gx);
     }
 #pragma unroll
-    for (int rr = 0; rr < 2; ++rr) fetch(rr);
+    for (int rr = 0; rr < (ALL_K ? RUN : 2); ++rr) fetch(rr);
     const bool good = mbar_wait(&bars[s], (k >> 1) & 1, timeout_ns);
     if (__syncthreads_or(!good)) {
       if (t == 0) atomicCAS(status, (int)PAT_OK, (int)PAT_ERR_TIMEOUT);
@@ -223,7 +226,7 @@ __global__ void __launch_bounds__(threads_of(TALL), min_ctas(R, FULL, GRAD, TALL
         const int gy = gy0 + r0 + rr;
         const long long gi = (long long)gy * pitch + gx;
         const bool in = gy < ny && gx < nx;
-        if (rr + 2 < RUN) fetch(rr + 2);
+        if (!ALL_K && rr + 2 < RUN) fetch(rr + 2);
         Cells<NP> sa2, sb2, zl2;
         sa2.fill(1.f);
         sb2.fill(1.f);
