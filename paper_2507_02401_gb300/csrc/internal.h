@@ -107,7 +107,7 @@ struct Persist2DArgs {
 //      (adjoint: L(kappa cur)).
 //   2D adjoint carries compensation terms in cur_lo/next_lo (and dbuf_lo): the TMA kernel keeps
 //      the state Z = kappa Q with its low part in cur_lo/next_lo (G plain, or with G_lo in dbuf_lo on
-//      grids of odd width); the plain kernel keeps Q with Q_lo there and G_lo in dbuf_lo, feeding the
+//      rows of no multiple of 4 cells); the plain kernel keeps Q with Q_lo there and G_lo in dbuf_lo, feeding the
 //      stencil kappa*Q as a hi + lo pair.
 //   3D adjoint of a varying medium on the TMA kernel: the state is Z = kappa Q (plain),
 //      Z^n = 2 Z^{n+1} - Z^{n+2} + kappa (L Z^{n+1} + S^T r_n); the final step divides by kappa.
@@ -121,7 +121,7 @@ struct StepArgs {
   const float* cur;    // P^n (forward) or Q^{n+1} (adjoint)
   const float* cur_lo;  // 2D adjoint: compensation of Q^{n+1} (Z^{n+1} on the TMA kernel)
   float* next_lo;       // 2D adjoint: compensation of Q^n (Z^n on the TMA kernel)
-  float* dbuf_lo;       // 2D adjoint, plain kernel: compensation of G
+  float* dbuf_lo;       // 2D adjoint, plain kernel and the TMA kernel's full form: compensation of G
   const float* prev;   // 3D: P^{n-1} or Q^{n+2}   (nullptr = 0)
   float* dbuf;         // 2D: increment D (forward) / G (adjoint), updated in place
   int d_zero;          // 2D: treat the incoming increment as 0
@@ -137,9 +137,6 @@ struct StepArgs {
   const float* sens_w;
   int corners;
   float* y;
-  // Adjoint injection S^T r_{inj_t} after the step (inj_r nullptr = none): 2D into dbuf (for the step that
-  // follows), 3D into next; fused in the TMA kernels through per-tile / per-CTA lists (inj_tile_ptr /
-  // inj_tile), a separate launch otherwise.
   // 2D absorbing layer (nullptr = none): per-cell factors a, b of the damped update and the layer
   // width in cells (tiles farther than that from every face skip the factors)
   const float* sp_a;
@@ -152,6 +149,9 @@ struct StepArgs {
   float gcoef;
   float* gsum_hi;
   float* gsum_lo;
+  // Adjoint injection S^T r_{inj_t} after the step (inj_r nullptr = none): 2D into dbuf (for the step that
+  // follows), 3D into next; fused in the TMA kernels through per-tile / per-CTA lists (inj_tile_ptr /
+  // inj_tile), a separate launch otherwise.
   const float* inj_r;
   int inj_t;
   const int* inj_tile_ptr;

@@ -284,8 +284,8 @@ static pat_status wave_adjoint_impl(pat_plan* p, const float* y, float* x, cudaS
   a.y = nullptr;
   if (p->dim == 2) {
     // increment form with compensation: G = wv[2] (+ wv[5]); Q^m in wv[(nt-m) % 2]
-    // (+ wv[3 + (nt-m) % 2]) with Q^nt = 0.  The TMA kernel keeps Z = kappa Q there (and G_lo on odd widths
-    // only); the plain kernel Q itself.
+    // (+ wv[3 + (nt-m) % 2]) with Q^nt = 0.  The TMA kernel keeps Z = kappa Q there (and G_lo only on rows of
+    // no multiple of 4 cells); the plain kernel Q itself.
     float* G = p->d_wv[2];
     auto Qbuf = [&](int m) { return p->d_wv[(nt - m) % 2]; };
     auto Qlo = [&](int m) { return p->d_wv[3 + (nt - m) % 2]; };

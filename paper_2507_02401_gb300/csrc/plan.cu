@@ -67,9 +67,8 @@ static pat_status upload(pat_plan* p, T** ptr, const std::vector<T>& host, const
 static size_t padded(size_t bytes) { return (std::max<size_t>(bytes, 1) + 255) / 256 * 256; }
 
 // Device arrays of one allocation: their sizes are collected first, those with contents in front, so that a plan's
-// many small lists and its workspace cost one cudaMalloc and one copy (a plan has some forty arrays; at 1024^2 order 8
-// creation took 0.77 ms with one of each per array and the
-// kernels' occupancies queried anew, 0.25 so).  Lives until the stream has been synchronised.
+// many small lists and its workspace cost one cudaMalloc and one copy (a plan has some forty arrays; 1024^2 order 8:
+// 0.77 ms with one of each per array and the kernels' occupancies queried anew, 0.25 so).  Lives until the stream has been synchronised.
 class Arena {
  public:
   template <typename T>

@@ -22,27 +22,28 @@
 //   G^n = G^{n+1} + S^T r_n + L Z^{n+1},  Z^n = Z^{n+1} + kappa G^n,
 // with Z kept as a compensated pair Z + Z_lo (TwoSum) that is exchanged and
 // fed to the stencil as two FP32 fields (Z through the difference form, whose
-// rounding is relative to the differences, Z_lo through the cheap form); G is
+// rounding is relative to the differences, Z_lo through the pair form); G is
 // plain.
 //
 // GB300 mapping.  The grid is cut into 64 x 32 tiles, one CTA per tile, all
 // co-resident (cooperative launch).  Each of 512 threads keeps its 2 x 2 cells'
 // state in registers for the whole loop; the CTA keeps the current field plus
 // an R-deep halo in shared memory (double buffered).  Ten warps own the tile's
-// 8-cell frame, six its 48 x 16 interior, whose stencils (R <= 7) need no halo:
-// while the frame's warps wait for the neighbours' strips the interior is
-// computed, and while they compute the frame the interior's warps sample the
-// sensors.  (One step of 256 threads with 2 x 4 cells each, all of them behind
-// the halo: 2.69 us (K) and 3.22 us (K*) at 512^2, order 8, of which 1.3 and
-// 1.6 us are left with the 3-point stencil of order 2; now 1.75 and 2.44 us.)  After each step the
-// threads that own boundary cells write their blocks straight to an
-// L2-resident exchange buffer (relaxed GPU-scope stores; 93.4 against 92.3
-// reconstruction iterations/s at 512^2 when they were staged in shared memory
-// and handed to the TMA engine), every value packed with the step it belongs
-// to into one 64-bit word; an aligned
-// 64-bit access is single-copy atomic, so a neighbour that reads a word with
-// the expected tag has the right value: no flags, no fences, one L2 round
-// trip per exchange and one CTA barrier per step.  Every wait is bounded by a
+// 8-cell frame, six its 48 x 16 interior, whose stencils (R <= 7) need no halo
+// (K of order 2: six warps a 4-cell frame, ten the rest): while the frame's
+// warps wait for the neighbours' strips the interior is computed, and while
+// they compute the frame the interior's warps sample the sensors.  (One step of
+// 256 threads with 2 x 4 cells each, all of them behind the halo: 2.69 us (K)
+// and 3.22 us (K*) at 512^2, order 8, of which 1.3 and 1.6 us are left with the
+// 3-point stencil of order 2; now 1.75 and 2.44 us.)  After each step the
+// threads that own boundary cells write their blocks straight to an L2-resident
+// exchange buffer (relaxed GPU-scope stores; 93.4 against 92.3 reconstruction
+// iterations/s at 512^2 when they were staged in shared memory and handed to
+// the TMA engine), every value packed with the step it belongs to into one
+// 64-bit word; an aligned 64-bit access is single-copy atomic, so a neighbour
+// that reads a word with the expected tag has the right value: no flags, no
+// fences, one L2 round
+// trip per exchange and two CTA barriers per step.  Every wait is bounded by a
 // global-timer limit and a shared abort flag; a CTA that gives up records
 // PAT_ERR_TIMEOUT, raises the abort flag and leaves the loop, so the launch
 // always ends.
@@ -113,8 +114,8 @@ struct Geo {
   static constexpr int SBUF = ROWS * PITCH;        // one shared-memory field buffer
   // exchange: every frame thread within R cells of the edge (D = (R + 1) / 2 block rows or columns) publishes
   // its 2 x 2 block as four consecutive words.  R = 1, where half of such a block is not needed: the tile's four
-  // edges as strips of words, [top TX][bottom TX][left TY][right TY] (512^2 order 2: K 1.21 us per step with
-  // strips, 1.23 with blocks; 64^2 0.81 and 0.89; 768 x 704, two CTAs per SM, 1.34 and 1.52).
+  // edges as strips of words, [top TX][bottom TX][left TY][right TY] (with an 8-cell frame, order 2 K us per step:
+  // 512^2 1.21 with strips, 1.23 with blocks; 64^2 0.81 and 0.89; 768 x 704, two CTAs per SM, 1.34 and 1.52).
   static constexpr int D = (R + 1) / 2;
   static constexpr int SLOT = R == 1 ? 2 * (TX + TY) : 4 * Frame<R, ADJ>::BLOCKS;  // words per tile, slot and right-hand side
   static constexpr int RCOUNT = Frame<R, ADJ>::RCOUNT;

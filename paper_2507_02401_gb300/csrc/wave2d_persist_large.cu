@@ -16,7 +16,7 @@
 // compute the frame while the others serve the sensors.  P, Z and Z_lo are read
 // from shared memory (two slots of the whole tile); D or G stays in registers.
 // The adjoint keeps G as a compensated pair as well, as the per-step engine
-// does on grids of odd width; the sensor injections S^T r are added to its low
+// does on rows of no multiple of 4 cells; the sensor injections S^T r are added to its low
 // part G_lo, which sits in shared memory and joins the next increment anyway:
 // to the frame's cells before the mid-step barrier (the frame reads them after
 // it), to the interior's after it.

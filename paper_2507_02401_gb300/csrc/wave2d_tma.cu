@@ -17,14 +17,15 @@
 // 7e-7 with the compensated Z.  Each step also adds S^T r_{m-1}, the sensor
 // injection of the step after it, to the G it has just stored (lists per tile).
 //
-// Persistent CTAs walk 64 x 32 tiles; one thread issues the TMA load of the
-// next tile's boxes (80 x (32+2R) floats, halo included, zero outside the
-// grid: P for the forward, Z and Z_lo for the adjoint) into the second of two
+// Persistent CTAs walk 64 x 32 tiles (64 x 64 in the forward on very large
+// fields, see below); one thread issues the TMA load of the next tile's boxes
+// (80 x (32+2R) floats, halo included, zero outside the grid: P for the forward, Z and Z_lo for the adjoint) into the second of two
 // shared-memory stages while the CTA computes the current one.  Each thread
 // owns 4 columns x 4 consecutive rows: y neighbours come from a sliding
 // register window of 2R+1 rows, x neighbours from the shared-memory row; its
 // own D / G cells are loaded straight into registers before the wait for the
-// boxes, kappa and G_lo two rows ahead of their use.
+// boxes, as is kappa in the forward from order 4 on; kappa otherwise and G_lo
+// two rows ahead of their use.
 // Compulsory DRAM traffic per point-update: forward P and D read, P^{n+1} and
 // D^{n+1} written (16 B), plus kappa hi/lo (8 B) for a varying medium;
 // adjoint Z, Z_lo, G read and written (24 B), plus kappa (4 B) for a varying
@@ -92,7 +93,7 @@ __device__ __forceinline__ void fused_sample2(const StepArgs& a, long long bid, 
 //   forward  D' = a D + b inc (first step: D' = (a-1) P + b inc),  P' = P + D'
 //   adjoint  G' = G + inc,  Q' = a Q + b G', i.e. Z' = a Z + b kappa G'  (final step: x = G' + ((a-1)/b) Q)
 // Tiles that do not reach the layer use a = b = 1 without loading the factors.
-// FULL (grids of odd width): the forward's stencil takes the difference form and the adjoint keeps G as a
+// FULL (rows of no multiple of 4 cells): the forward's stencil takes the difference form and the adjoint keeps G as a
 // compensated pair too (G_lo in dbuf_lo), with the rounding of kappa G carried into Z_lo.
 // GRAD (adjoint): adds this step's term gcoef Z^m .* L P^{m-1} of the medium gradient to a compensated sum.
 // The sums are pairs of FP32 (TwoSum with the product's rounding error, ~2^-47): FP64 arithmetic runs at 2

@@ -418,9 +418,9 @@ cudaError_t tma3d_encode(const float* base, int nx, int pitch, int ny, int nz, i
 // columns (fewer than a quarter of the co-resident CTAs; 64 at 256^3): as many z ranges as keep every
 // CTA in one wave (9 at 256^3: 576 CTAs of 28-29 planes), so no second wave leaves SMs idle at the end
 // of a step.  Many columns (256 at 512^3): ranges of at least 16 planes, doubled while the grid keeps
-// >= 6 CTAs per SM.  Measured at 256^3: 41.0 / 40.0 us per K / K* step against 41.4 / 44.1 us with
-// 16-plane ranges in 1024 CTAs (and 43.1 / 42.3 us with equal z-fastest shares of the (column, plane)
-// work, whose concurrent CTAs no longer share x/y halos through L2).
+// >= 6 CTAs per SM.  Measured at 256^3, order 4: 33.6 / 36.7 us per K / K* step against 38.0 / 40.3 us with
+// 16-plane ranges in 1024 CTAs.  (Equal z-fastest shares of the (column, plane) work lost on an earlier form
+// of the kernel: CTAs that run together no longer share x/y halos through L2.)
 Tma3dSplit tma3d_split(int R, bool varc, int nx, int ny, int nz) {
   const int cap = resident(R, varc);
   if (cap <= 0) return Tma3dSplit{0, 0, false};
@@ -437,8 +437,8 @@ Tma3dSplit tma3d_split(int R, bool varc, int nx, int ny, int nz) {
   }
   if (chunks > nz) chunks = nz;
   // the register-ring march saves the queue's register moves where issue is the bound (one-wave grids:
-  // 38.7 / 40.3 us against 39.4 / 41.2 per K / K* step at 256^3), but its larger body costs where DRAM is
-  // (many columns: 274.5 / 278.7 us against 264.8 / 268.9 at 512^3)
+  // 33.6 / 36.7 us against 36.6 / 39.0 per K / K* step at 256^3), but its larger body costs where DRAM is
+  // (many columns: 275.1 / 281.6 us against 261.5 / 270.8 at 512^3)
   return Tma3dSplit{(int)(cols * chunks), chunks, cols * 4 < cap && R <= 3};
 }
 
