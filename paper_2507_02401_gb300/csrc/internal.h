@@ -166,7 +166,7 @@ bool persist2d_supported(int R, bool varc);
 int persist2d_tile_x();
 int persist2d_tile_y();
 size_t persist2d_xbuf_words(int R, int ntiles, int nr = 1);  // 64-bit exchange words, nr fields
-int persist2d_max_ctas(int R, bool adj, bool varc);  // co-resident CTA limit on this device
+bool persist2d_fits(int R, bool varc, long long tiles);  // whether so many tiles are co-resident on this device, K and K*
 // layer: with the absorbing layer (a.sp_a, a.sp_b set)
 cudaError_t persist2d_launch(int R, bool adj, bool varc, bool layer, const Persist2DArgs& a, int nctas,
                              cudaStream_t st);
@@ -179,7 +179,7 @@ int persist2dl_tile_x();
 int persist2dl_tile_y();
 int persist2dl_edge();
 size_t persist2dl_xbuf_words(int ntiles);
-int persist2dl_max_ctas(int R, bool adj, bool varc);  // with and without the layer; 0: no such kernel
+int persist2dl_max_ctas(int R, bool adj, bool varc);  // 0: no such kernel
 int persist2dl_min_tiles(int R, bool varc);  // worth it above this many 64 x 32 tiles per SM
 cudaError_t persist2dl_launch(int R, bool adj, bool varc, bool layer, const Persist2DArgs& a, int nctas,
                               cudaStream_t st);

@@ -553,17 +553,17 @@ static pat_status create(const pat_grid* grid, const double* c, double c0, const
   p->persist_ok = false;
   if (p->dim == 2 && persist2d_supported(p->R, p->varc)) {
     auto tiles = [&](int TX, int TY) { return (long long)((p->n[0] + TX - 1) / TX) * ((p->n[1] + TY - 1) / TY); };
-    p->persist_ok = tiles(persist2d_tile_x(), persist2d_tile_y()) <=
-                    std::min(persist2d_max_ctas(p->R, false, p->varc), persist2d_max_ctas(p->R, true, p->varc));
+    p->persist_ok = persist2d_fits(p->R, p->varc, tiles(persist2d_tile_x(), persist2d_tile_y()));
     // grids with too many 64 x 32 tiles: 128 x 64 tiles, whose kernel reads kappa and the layer's factors in pairs
     if (!p->persist_ok && p->pitch % 2 == 0 && (z_safe || rows4)) {
-      const int cap = std::min(persist2dl_max_ctas(p->R, false, p->varc), persist2dl_max_ctas(p->R, true, p->varc));
       int TX, TY, dev = 0, sms = 0;
       tma2d_tile(&TX, &TY);
       PAT_TRY_CUDA(cudaGetDevice(&dev));
       PAT_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-      p->persist_ok = p->persist_large = tiles(persist2dl_tile_x(), persist2dl_tile_y()) <= cap &&
-                                         tiles(TX, TY) > (long long)persist2dl_min_tiles(p->R, p->varc) * sms;
+      const long long n = tiles(persist2dl_tile_x(), persist2dl_tile_y());
+      p->persist_ok = p->persist_large =
+          n <= sms && tiles(TX, TY) > (long long)persist2dl_min_tiles(p->R, p->varc) * sms &&
+          n <= persist2dl_max_ctas(p->R, false, p->varc) && n <= persist2dl_max_ctas(p->R, true, p->varc);
     }
     if (p->persist_ok) setup_persistent(p, lists);
   }

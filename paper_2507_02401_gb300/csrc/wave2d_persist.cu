@@ -654,12 +654,25 @@ size_t persist2d_xbuf_words(int R, int ntiles, int nr) {
   return (size_t)nr * ntiles * 2 * slot;
 }
 
-int persist2d_max_ctas(int R, bool adj, bool varc) {
+static int max_ctas(int R, bool adj, bool varc) {
   static PerDevice kept[kMaxR + 1][2][2];
   return kept[R][adj][varc].get(current_device(), [&] {
     const int fit = resident(pick(R, adj, varc, false, 1), R, adj);
     return R == 1 ? std::max(fit, resident(pick(R, adj, varc, false, 2), R, adj)) : fit;
   });
+}
+
+bool persist2d_fits(int R, bool varc, long long tiles) {
+  int dev = 0, sms = 0, smem = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  // more tiles than shared memory has room for need no question to the kernels (which loads them)
+  if (tiles > (long long)sms * (smem / (int)smem_bytes(R, true))) return false;
+  return tiles <= std::min(max_ctas(R, false, varc), max_ctas(R, true, varc));
 }
 
 cudaError_t persist2d_launch(int R, bool adj, bool varc, bool layer, const Persist2DArgs& a, int nctas,

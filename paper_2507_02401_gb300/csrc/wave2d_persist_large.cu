@@ -475,24 +475,22 @@ int persist2dl_tile_y() { return TY; }
 int persist2dl_edge() { return EDGE; }
 size_t persist2dl_xbuf_words(int ntiles) { return (size_t)ntiles * 2 * 2 * RUN * NFRAME; }
 
+// One per SM: the launch bounds give every variant, with the layer or without, the registers for that, and the layer
+// needs no shared memory, so one variant is asked (asking loads a kernel, 0.3 to 0.5 ms the first time).
 int persist2dl_max_ctas(int R, bool adj, bool varc) {
   static PerDevice kept[kMaxR + 1][2][2];
   return kept[R][adj][varc].get(current_device(), [&] {
-    int best = 0;
-    for (int layer = 0; layer < 2; ++layer) {
-      void* f = pick(R, adj, varc, layer);
-      int dev = 0, sms = 0, per_sm = 0;
-      const size_t smem = smem_bytes(R, adj, varc);
-      if (!f || cudaGetDevice(&dev) != cudaSuccess ||
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-          cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, NTHREADS, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-      }
-      best = layer == 0 || sms * per_sm < best ? sms * per_sm : best;
+    void* f = pick(R, adj, varc, false);
+    int dev = 0, sms = 0, per_sm = 0;
+    const size_t smem = smem_bytes(R, adj, varc);
+    if (!f || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, NTHREADS, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
     }
-    return best;
+    return per_sm > 0 ? sms : 0;
   });
 }
 
